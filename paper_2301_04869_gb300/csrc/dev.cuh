@@ -35,9 +35,11 @@ struct DevSym {
   const int4 *fs4, *bs4, *fr4, *br4;  // packed single-RHS sweeps (symbolic.cpp)
   const int *gu_ptr, *gu_col, *gu_src, *gut_ptr, *gut_col, *gut_src;
   const int *kx_ptr, *kx_col, *kx_src, *ku_ptr, *ku_col, *ku_src;
+  // the same product lists as {column, slot} pairs (zp_col/zp_slot,
+  // zp_tcol/zp_tslot, br_col/br_uslot) and {column, K entry} (kx_col/kx_src)
+  const int2 *zp2, *zpt2, *br2, *kx2;
   int zp_npan;  // forward schedules per 32-column panel of Z (symbolic.cpp)
-  const int *zp_lev_off, *zp_lev_ptr, *zp_rows, *zp_eptr, *zp_col, *zp_slot, *zp_zptr, *zp_zrows, *zp_tptr, *zp_tcol,
-      *zp_tslot;
+  const int *zp_lev_off, *zp_lev_ptr, *zp_rows, *zp_eptr, *zp_zptr, *zp_zrows, *zp_tptr;
   const double *xl, *xu, *ul, *uu, *sl, *su, *c2, *c1;
   const double *pd, *qd;  // [N][n]
   // line status per (line, scenario), lon[l * N + sc] in {0, 1}, or null

@@ -144,9 +144,15 @@ ipm_status upload_symbolic(ipm_ctx *c, const HostNet &net, const double *pd, con
   TRY(upload(c, &d.gut_ptr, S.gut_ptr)); TRY(upload(c, &d.gut_col, S.gut_col)); TRY(upload(c, &d.gut_src, S.gut_src));
   d.zp_npan = S.zp_npan;
   TRY(upload(c, &d.zp_lev_off, S.zp_lev_off)); TRY(upload(c, &d.zp_lev_ptr, S.zp_lev_ptr));
-  TRY(upload(c, &d.zp_rows, S.zp_rows)); TRY(upload(c, &d.zp_eptr, S.zp_eptr)); TRY(upload(c, &d.zp_col, S.zp_col));
-  TRY(upload(c, &d.zp_slot, S.zp_slot)); TRY(upload(c, &d.zp_zptr, S.zp_zptr)); TRY(upload(c, &d.zp_zrows, S.zp_zrows));
-  TRY(upload(c, &d.zp_tptr, S.zp_tptr)); TRY(upload(c, &d.zp_tcol, S.zp_tcol)); TRY(upload(c, &d.zp_tslot, S.zp_tslot));
+  TRY(upload(c, &d.zp_rows, S.zp_rows)); TRY(upload(c, &d.zp_eptr, S.zp_eptr)); TRY(upload(c, &d.zp_zptr, S.zp_zptr));
+  TRY(upload(c, &d.zp_zrows, S.zp_zrows)); TRY(upload(c, &d.zp_tptr, S.zp_tptr));
+  auto pairs = [c](const int2 **dst, const std::vector<int> &a, const std::vector<int> &b) {
+    std::vector<int2> v(a.size());
+    for (size_t i = 0; i < v.size(); ++i) v[i] = make_int2(a[i], b[i]);
+    return upload(c, dst, v);
+  };
+  TRY(pairs(&d.zp2, S.zp_col, S.zp_slot)); TRY(pairs(&d.zpt2, S.zp_tcol, S.zp_tslot));
+  TRY(pairs(&d.br2, S.br_col, S.br_uslot)); TRY(pairs(&d.kx2, S.kx_col, S.kx_src));
   TRY(upload(c, &d.kx_ptr, S.kx_ptr)); TRY(upload(c, &d.kx_col, S.kx_col)); TRY(upload(c, &d.kx_src, S.kx_src));
   TRY(upload(c, &d.ku_ptr, S.ku_ptr)); TRY(upload(c, &d.ku_col, S.ku_col)); TRY(upload(c, &d.ku_src, S.ku_src));
   TRY(upload(c, &d.xl, S.xl)); TRY(upload(c, &d.xu, S.xu)); TRY(upload(c, &d.ul, S.ul)); TRY(upload(c, &d.uu, S.uu));
@@ -274,6 +280,9 @@ ipm_status alloc_work(ipm_ctx *c) {
         return fail(c, IPM_ERR_CUDA, "tensor maps of the tensor-core block solve");
       c->tcs_on = true;
     }
+    c->rf.nk = (int)S.kx_col.size();
+    TRY(dalloc(c, &c->rf.LUf, N * round_lu_len(c->ds))); TRY(dalloc(c, &c->rf.rdf, N * nx));
+    TRY(dalloc(c, &c->rf.Kf, N * c->rf.nk));
     TRY(dalloc(c, &c->pcg_b, nu)); TRY(dalloc(c, &c->pcg_r, nu)); TRY(dalloc(c, &c->pcg_z, nu));
     TRY(dalloc(c, &c->pcg_p, nu)); TRY(dalloc(c, &c->pcg_Ap, nu));
   }
@@ -295,6 +304,12 @@ ipm_status alloc_work(ipm_ctx *c) {
     set_groups(c, 4 * G0);
     c->max_groups = c->ngroups;
     set_groups(c, G0);
+  }
+  {
+    // the multi-RHS solve's panels in flight; a mixed context also runs the FP64 solve (fallback iterations)
+    unsigned char *zw = nullptr;
+    TRY(dalloc(c, &zw, zsolve_work_bytes(c->ds, sizeof(double))));
+    c->zwork = zw;
   }
   c->zs_threads = (c->opt.solve_threads == 128 || c->opt.solve_threads == 256) ? c->opt.solve_threads : 256;
   TRY(dalloc(c, &c->tiles, tl.size()));
@@ -612,8 +627,8 @@ ipm_status autotune(ipm_ctx *c, cudaStream_t st) {
   double best = 1e300;
   int best_thr = 256;
   for (int thr : {128, 256}) {
-    const double ms = fp64 ? time_ms([&] { launch_zsolve64(S, D.LU, D.rd, D.J, D.K, c->Z, c->Y, c->Yu, st, thr); }, st)
-                           : time_ms([&] { launch_zsolve32(S, D.LU, D.rd, D.J, D.K, c->Z32, c->Y32, c->Yu, st, thr, tcs_of(c), D.flags); }, st);
+    const double ms = fp64 ? time_ms([&] { launch_zsolve64(S, D.LU, D.rd, D.J, D.K, (double *)c->zwork, c->Z, c->Y, c->Yu, st, thr); }, st)
+                           : time_ms([&] { launch_zsolve32(S, D.LU, D.rd, D.J, D.K, c->rf, (float *)c->zwork, c->Z32, c->Y32, c->Yu, st, thr, tcs_of(c), D.flags); }, st);
     c->tune_ms[thr == 128 ? 0 : 1] = ms;
     if (ms < best) best = ms, best_thr = thr;
   }
@@ -621,9 +636,9 @@ ipm_status autotune(ipm_ctx *c, cudaStream_t st) {
   // the solve outputs are identical for every thread count; rerun the winner
   // so that the mixed planes are split from them below
   if (fp64) {
-    launch_zsolve64(S, D.LU, D.rd, D.J, D.K, c->Z, c->Y, c->Yu, st, best_thr);
+    launch_zsolve64(S, D.LU, D.rd, D.J, D.K, (double *)c->zwork, c->Z, c->Y, c->Yu, st, best_thr);
   } else {
-    launch_zsolve32(S, D.LU, D.rd, D.J, D.K, c->Z32, c->Y32, c->Yu, st, best_thr, tcs_of(c), D.flags);
+    launch_zsolve32(S, D.LU, D.rd, D.J, D.K, c->rf, (float *)c->zwork, c->Z32, c->Y32, c->Yu, st, best_thr, tcs_of(c), D.flags);
     launch_split_t((long long)S.N * S.nx, S.nu, c->planZY.kpad, c->Z32, c->zpl, st);
     launch_split_t((long long)S.N * S.nx, S.nu, c->planZY.kpad, c->Y32, c->ypl, st);
   }
@@ -776,9 +791,9 @@ ipm_status do_condense(ipm_ctx *c, cudaStream_t st) {
     if (fp64 && c->emu)
       cudaMemsetAsync(c->emu_rs, 0, 2 * (size_t)S.N * S.nx * sizeof(int), st);  // row exponent maxima
     if (fp64)
-      launch_zsolve64(S, D.LU, D.rd, D.J, D.K, c->Z, c->Y, c->Yu, st, c->zs_threads, D.g, c->bpos,
+      launch_zsolve64(S, D.LU, D.rd, D.J, D.K, (double *)c->zwork, c->Z, c->Y, c->Yu, st, c->zs_threads, D.g, c->bpos,
                       c->emu ? c->emu_rs : nullptr);
-    else launch_zsolve32(S, D.LU, D.rd, D.J, D.K, c->Z32, c->Y32, c->Yu, st, c->zs_threads, tcs_of(c), D.flags);
+    else launch_zsolve32(S, D.LU, D.rd, D.J, D.K, c->rf, (float *)c->zwork, c->Z32, c->Y32, c->Yu, st, c->zs_threads, tcs_of(c), D.flags);
     ph_end(c, PH_ZSOLVE, st);
     if (fp64) {
       // the reduced right-hand side needs Z and b only: on the side stream,

@@ -46,8 +46,10 @@ void launch_lu_factor(const DevSym &S, int nL, const double *J, double *LU, doub
 // g, b (optional, [N][n_x]): also b = G_x^{-1} g in position order (g in
 // state order), in an extra right-hand-side lane, when zsolve64_folds_b
 void launch_zsolve64(const DevSym &S, const double *LU, const double *rd, const double *J, const double *K,
-                     double *Z, double *Y, double *Yu, cudaStream_t st, int threads = 256,
+                     double *work, double *Z, double *Y, double *Yu, cudaStream_t st, int threads = 256,
                      const double *g = nullptr, double *b = nullptr, int *ezy = nullptr);
+// bytes of the multi-RHS solves' work buffer (elem: 8 FP64, 4 FP32)
+size_t zsolve_work_bytes(const DevSym &S, size_t elem);
 bool zsolve64_folds_b(const DevSym &S);
 // kernels_big.cu: the large trailing block (S.big) in global memory
 void launch_big_lu_dense(const DevSym &S, double *LU, double *rd, const double *amax, int *flags, cudaStream_t st,
@@ -60,8 +62,16 @@ struct TcsPlan;
 // tcs: the tensor-core variant of the block updates (mixed path), or null
 void launch_big_trsm32(const DevSym &S, const double *LU, const double *rd, float *Z, cudaStream_t st,
                        const TcsPlan *tcs = nullptr, int *flags = nullptr);
+// FP32 copies the mixed path's solve reads, filled by launch_zsolve32: the
+// factor values ([N][round_lu_len]), the reciprocal pivots ([N][n_x]) and K in
+// the order of the row lists of K_x ([N][nk])
+struct RoundedFactors {
+  float *LUf = nullptr, *rdf = nullptr, *Kf = nullptr;
+  int nk = 0;
+};
+__host__ __device__ inline int round_lu_len(const DevSym &S) { return S.big ? S.dense_base : S.nnzLU; }
 void launch_zsolve32(const DevSym &S, const double *LU, const double *rd, const double *J, const double *K,
-                     float *Z, float *Y, double *Yu, cudaStream_t st, int threads = 256,
+                     const RoundedFactors &f, float *work, float *Z, float *Y, double *Yu, cudaStream_t st, int threads = 256,
                      const TcsPlan *tcs = nullptr, int *flags = nullptr);
 void launch_solve1(const DevSym &S, const double *LU, const double *rd, double *v, int trans,
                    cudaStream_t st);

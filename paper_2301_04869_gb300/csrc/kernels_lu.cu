@@ -269,245 +269,416 @@ __global__ void k_lu_factor(DevSym S, int nL, const double *__restrict__ J, doub
   for (int e = tid; e < ns * ns; e += bd) A[ts[(k0 + e / ns) * nd + k0 + e % ns]] = T[e];
 }
 
-// Multi-RHS reduction solve for one scenario and one panel of 32 RHS columns
-// (lane = column): Z = -U^{-1} L^{-1} (P G_u) (rows in LU position order),
-// then Y = K_x [Z; I] and Y_u = K_u [Z; I].  The sparse rows follow the level
-// schedule (one warp per row); the dense trailing block [t0, nx) is solved
-// column by column by the whole CTA, in shared memory when it fits
-// (tail_smem), else in place in Z.  T is the storage/arithmetic type of Z, Y
-// (double on the FP64 path, float on the mixed path); Y_u accumulates in FP64.
+// C consecutive elements in one 16-byte (or 8-byte) access
+template <typename T, int C>
+struct alignas(sizeof(T) * C) Pack {
+  T v[C];
+};
+
+// One scheduled row: its place, its products [f0, f0 + len).
+struct RowDesc {
+  int row, f0, len;
+};
+
+// Walks the rows of levels [0, nlev) (rows lev(l) .. lev(l + 1) of a
+// schedule; a CTA barrier after every level), W lanes to a row and C columns
+// of the right-hand sides to a lane: acc = init(row), then the row's
+// products in their order, acc -= (or +=) value * operand(place), then
+// finish(row, acc).  The lanes of a row fetch the places and values of W
+// products side by side (each once per row instead of once per lane) and
+// hand them round by shuffles; U products' operands are in flight.
+// meta(f, place, slot), value(slot); operand(place, mine) may clear mine
+// (no product for this lane, whatever the value).  Called by all threads.
+// Fetching the next chunk's places and values ahead of this one's operands
+// was measured too: its registers cost more warps than it hid latency
+// (3.58 -> 4.20 ms FP64, 1.27 -> 1.85 ms FP32 at 1,000 buses x 64).
+template <typename T, int W, int C, int U, bool SUB, class Lev, class Desc, class Meta, class Value, class Operand,
+          class Init, class Finish>
+__device__ __forceinline__ void sweep_rows(int nlev, Lev lev, Desc desc, Meta meta, Value value, Operand operand,
+                                           Init init, Finish finish) {
+  constexpr int R = 32 / W;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, cl = lane % W;
+  for (int l = 0; l < nlev; ++l) {
+    const int e1 = lev(l + 1);
+    for (int eb = lev(l) + warp * R; eb < e1; eb += (blockDim.x >> 5) * R) {
+      const int e = eb + lane / W;
+      RowDesc d = {-1, 0, 0};
+      if (e < e1) d = desc(e);
+      const int mlen = W == 32 ? d.len : (int)__reduce_max_sync(0xffffffffu, (unsigned)d.len);
+      Pack<T, C> acc = {};
+      if (d.row >= 0) acc = init(d.row);
+      for (int base = 0; base < mlen; base += W) {
+        int at = 0, slot;
+        T val = 0;
+        if (base + cl < d.len) {
+          meta(d.f0 + base + cl, at, slot);
+          val = value(slot);
+        }
+        const int n = min(W, mlen - base);
+        for (int j = 0; j < n; j += U) {
+          T v[U];
+          Pack<T, C> z[U];
+#pragma unroll
+          for (int k = 0; k < U; ++k) {
+            const int p = __shfl_sync(0xffffffffu, at, j + k, W);
+            v[k] = __shfl_sync(0xffffffffu, val, j + k, W);
+            z[k] = Pack<T, C>{};
+            bool mine = base + j + k < d.len;
+            if (mine) z[k] = operand(p, mine);
+            if (!mine) v[k] = 0;
+          }
+#pragma unroll
+          for (int k = 0; k < U; ++k)
+#pragma unroll
+            for (int q = 0; q < C; ++q) acc.v[q] = SUB ? acc.v[q] - v[k] * z[k].v[q] : acc.v[q] + v[k] * z[k].v[q];
+        }
+      }
+      if (d.row >= 0) finish(d.row, acc);
+    }
+    __syncthreads();
+  }
+}
+
+// Multi-RHS reduction solve for one scenario and one panel of PW = W C RHS
+// columns: Z = -U^{-1} L^{-1} (P G_u) (rows in LU position order), then
+// Y = K_x [Z; I] and Y_u = K_u [Z; I].  The sparse rows follow the level
+// schedule (W lanes per row, C columns per lane); the dense trailing block
+// [t0, nx) is solved by the whole CTA in shared memory.  T is the
+// storage/arithmetic type of Z, Y (double on the FP64 path, float on the
+// mixed path); Y_u accumulates in FP64.  A, r (factor values, reciprocal
+// pivots) and, on the mixed path, Kp (K in the order of the product lists)
+// are of type T: GB300 converts between FP64 and FP32 at the rate of its
+// FP64 units (a warp-wide conversion every ~19 cycles per SM), so a
+// conversion per product and lane made the FP32 solve as slow as the FP64
+// one; the mixed path converts each value once (k_round_factors, k_round_k).
+//
+// The panel is worked on in Zp, a contiguous buffer of the CTA's own
+// ([nx][PW], lane cl's C columns side by side: element cl C + q of a row is
+// column c0 + q W + cl), and written to Z as Y is formed: an operand is one
+// 16-byte load per lane at a shifted index, and a warp works on 32 / W rows
+// at once.  Bound by the FP64 units (75 % of their cycles) on the FP64 path
+// and by the latency of the operand loads on the mixed one.  Measured (the
+// whole solve, against a warp per row of 32 columns with one column and
+// every product's column, slot and value loaded by every lane): 1,000 buses
+// x 64 4.03 -> 3.63 ms FP64 and 3.08 -> 1.26 ms FP32, 433 buses x 19 685 ->
+// 413 us FP64, 10,000 buses x 32 67.3 -> 43.3 ms FP32 (17 ms of it the dense
+// block's own kernels).  CTAs of 512 or 1,024 threads for the large networks
+// were slower (50 and 60 ms), as were W x C = 16 x 2 (47 ms) and 32 x 1 (62).
+//
 // phase (large trailing block, S.big): 1 = the forward sparse rows and the
 // trailing rows' right-hand sides only (left in Z for the batched block
-// solves), 2 = the backward sparse rows and the products only; 0 = all.
-template <typename T>
-__device__ void zsolve_body(const DevSym &S, const double *__restrict__ LU, const double *__restrict__ rd,
-                            const double *__restrict__ J, const double *__restrict__ K, T *Z, T *Y, double *Yu,
-                            bool tail_smem, T *sh, const double *__restrict__ gvec, T *bvec, int *ezy,
-                            int phase = 0) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5, bd = blockDim.x;
+// solves), 2 = the rest, the trailing rows taken from Z (the forward sparse
+// rows, a few percent of the products, are formed again); 0 = all.
+template <typename T, int W, int C>
+__device__ void zsolve_panel(const DevSym &S, int sc, int panel, const T *__restrict__ A, const T *__restrict__ r,
+                             const double *__restrict__ J, const double *__restrict__ K, const T *__restrict__ Kp,
+                             T *__restrict__ Zp, T *Zs, T *Ys, double *Yus, T *sh, const double *__restrict__ gvec,
+                             T *bs, int *ezy, int phase) {
+  using P = Pack<T, C>;
+  constexpr int R = 32 / W, PW = W * C, U = 4;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  const int cl = lane % W, grp = warp * R + lane / W, ngrp = nw * R;
   const int nu = S.nu, nx = S.nx, N = S.N;
-  // the CTA after the panels of Z (when bvec is given) solves b alone
-  const bool bpanel = bvec != nullptr && (int)blockIdx.x == (nu + 31) / 32;
-  const int sc = blockIdx.y, c0 = blockIdx.x * 32, c = bpanel ? nu + lane : c0 + lane;
+  const int c0 = panel * PW, c = c0 + cl;  // the lane's columns c, c + W, ...
   const int t0 = S.t0, nd = S.nd;
-  const bool valid = c < nu;
-  const int cc = valid ? c : nu - 1;
-  const double *A = LU + (size_t)sc * S.nnzLU;
-  const double *r = rd + (size_t)sc * nx;
-  T *Zs = Z + (size_t)sc * nx * nu;
-  T *Ys = Y + (size_t)sc * nx * nu;
-  double *Yus = Yu + (size_t)sc * nu * nu;
-  // Optional extra column n_u (when bvec is given): b = G_x^{-1} g of the
-  // reduced right-hand side, solved by lane 0 of an extra CTA per scenario
-  // (its forward sweep is dense, unlike those of the columns of G_u, so it
-  // gets a CTA of its own instead of slowing one panel of Z), stored in
-  // bvec [N][n_x] (position order).  zb/zst read a lane's own column, zw
-  // writes it.
-  const bool xb = bpanel && lane == 0;
-  T *bs = bvec ? bvec + (size_t)sc * nx : nullptr;
-  const T *zb = xb ? bs : Zs + cc;
-  T *zw = xb ? bs : Zs + c;
-  const size_t zst = xb ? 1 : (size_t)nu;
-  const bool wr = valid || xb;
-  // forward, sparse rows: this panel's schedule (rows its columns of G_u
-  // reach, products against such rows only); the other rows are zero
-  const int pan = blockIdx.x;
-  if (phase != 2) {
-  for (int e = S.zp_zptr[pan] + warp; e < S.zp_zptr[pan + 1]; e += nw)
-    if (wr) zw[(size_t)S.zp_zrows[e] * zst] = (T)0;
-  for (int l = S.zp_lev_off[pan]; l < S.zp_lev_off[pan + 1]; ++l) {
-    for (int e = S.zp_lev_ptr[l] + warp; e < S.zp_lev_ptr[l + 1]; e += nw) {
-      const int row = S.zp_rows[e];
-      T acc = 0;
-      if (xb) acc = (T)gvec[(size_t)sc * nx + S.iperm[row]];
-      else
-        for (int g = S.gu_ptr[row]; g < S.gu_ptr[row + 1]; ++g)
-          if (S.gu_col[g] == cc) {
-            const int src = S.gu_src[g];
-            acc -= src >= 0 ? (T)J[(size_t)src * N + sc] : (T)-1.0;
-          }
-      for (int f = S.zp_eptr[e]; f < S.zp_eptr[e + 1]; ++f)
-        acc -= (T)A[S.zp_slot[f]] * zb[(size_t)S.zp_col[f] * zst];
-      if (wr) zw[(size_t)row * zst] = acc;
+  // Optional extra column n_u (bs given): b = G_x^{-1} g of the reduced
+  // right-hand side, in the first free place of the last panel (there is
+  // one: n_u = 2 n_g - 1 is odd).  Its forward sweep is dense, so that panel
+  // takes the schedule of all rows (+11 % of one panel's products at 1,000
+  // buses, against +85 % for a panel of its own).
+  const auto zrow = [&](int row) { return reinterpret_cast<P *>(Zp + (size_t)row * PW) + cl; };
+  const auto zread = [&](int row, bool &) { return *zrow(row); };
+  const auto lu_meta = [](const int2 *pr) {
+    return [pr](int f, int &col, int &slot) {
+      const int2 p = pr[f];
+      col = p.x;
+      slot = p.y;
+    };
+  };
+  const auto lu_value = [&](int slot) { return A[slot]; };
+  // right-hand side of a row: -G_u (or g, for b)
+  const auto rhs_of = [&](int row) {
+    P acc = {};
+    for (int g = S.gu_ptr[row]; g < S.gu_ptr[row + 1]; ++g) {
+      const int d = S.gu_col[g] - c;
+      if (d >= 0 && d < PW && d % W == 0) {
+        const int src = S.gu_src[g];
+        const T v = src >= 0 ? (T)J[(size_t)src * N + sc] : (T)-1.0;
+#pragma unroll
+        for (int q = 0; q < C; ++q)
+          if (d == q * W) acc.v[q] -= v;
+      }
+    }
+    if (bs)
+#pragma unroll
+      for (int q = 0; q < C; ++q)
+        if (c + q * W == nu) acc.v[q] = (T)gvec[(size_t)sc * nx + S.iperm[row]];
+    return acc;
+  };
+  // forward, sparse rows: the schedule of the 32-column panel that holds
+  // this one (rows its columns of G_u reach, products against such rows
+  // only; the other rows are zero), or of all rows beside b
+  const int pan = bs != nullptr && c0 + PW > nu ? S.zp_npan - 1 : c0 / 32;
+  for (int e = S.zp_zptr[pan] + grp; e < S.zp_zptr[pan + 1]; e += ngrp) *zrow(S.zp_zrows[e]) = P{};
+  {
+    const int *lp = S.zp_lev_ptr + S.zp_lev_off[pan];
+    sweep_rows<T, W, C, U, true>(
+        S.zp_lev_off[pan + 1] - S.zp_lev_off[pan], [&](int l) { return lp[l]; },
+        [&](int e) { return RowDesc{S.zp_rows[e], S.zp_eptr[e], S.zp_eptr[e + 1] - S.zp_eptr[e]}; },
+        lu_meta(S.zp2), lu_value, zread, rhs_of, [&](int row, const P &acc) { *zrow(row) = acc; });
+  }
+  if (phase == 2) {  // the solved trailing rows
+    for (int i = grp; i < nd; i += ngrp) {
+      P z = {};
+#pragma unroll
+      for (int q = 0; q < C; ++q)
+        if (c + q * W < nu) z.v[q] = Zs[(size_t)(unsigned)(t0 + i) * (unsigned)nu + c + q * W];
+      *zrow(t0 + i) = z;
     }
     __syncthreads();
-  }
-  if (nd > 0) {
+  } else {
     // trailing block: right-hand side and the sparse part of each row
-    for (int i = warp; i < nd; i += nw) {
-      const int row = t0 + i;
-      T acc = 0;
-      if (xb) acc = (T)gvec[(size_t)sc * nx + S.iperm[row]];
-      else
-        for (int g = S.gu_ptr[row]; g < S.gu_ptr[row + 1]; ++g)
-          if (S.gu_col[g] == cc) {
-            const int src = S.gu_src[g];
-            acc -= src >= 0 ? (T)J[(size_t)src * N + sc] : (T)-1.0;
+    P *shp = reinterpret_cast<P *>(sh) + cl;  // row i at shp[i * W]
+    const int *tp = S.zp_tptr + pan * nd;
+    sweep_rows<T, W, C, U, true>(
+        1, [&](int l) { return l * nd; }, [&](int i) { return RowDesc{i, tp[i], tp[i + 1] - tp[i]}; },
+        lu_meta(S.zpt2), lu_value, zread, [&](int i) { return rhs_of(t0 + i); },
+        [&](int i, const P &acc) {
+          if (phase == 0) {
+            shp[i * W] = acc;
+          } else {
+#pragma unroll
+            for (int q = 0; q < C; ++q)
+              if (c + q * W < nu) Zs[(size_t)(unsigned)(t0 + i) * (unsigned)nu + c + q * W] = acc.v[q];
           }
-      for (int f = S.zp_tptr[pan * nd + i]; f < S.zp_tptr[pan * nd + i + 1]; ++f)
-        acc -= (T)A[S.zp_tslot[f]] * zb[(size_t)S.zp_tcol[f] * zst];
-      if (tail_smem) sh[i * 32 + lane] = acc;
-      else if (valid) Zs[(size_t)row * nu + c] = acc;
-    }
-    __syncthreads();
+        });
     if (phase == 1) return;  // the block is solved by the batched kernels
-    const int *ts = S.tail_slot;
-    if (tail_smem) {
-      // Blocked by 32 in shared memory: one warp solves each 32 x 32
-      // diagonal block (lane = RHS column), then every warp applies the
-      // block's columns to the remaining rows (warp = row, lane = column).
-      // Column c of the block is contiguous in LU storage: (a, c) sits at
-      // tail_slot[c] + a (read straight from the LU values, the same address
-      // for all lanes).  Backward values are scaled as they are found.
-      for (int kb = 0; kb < nd; kb += 32) {
-        const int w = min(32, nd - kb);
-        if (warp == 0) {
-          for (int jj = 0; jj < w; ++jj) {
-            const T xj = sh[(kb + jj) * 32 + lane];
-            const double *col = A + ts[kb + jj] + kb;  // L(kb + i2, kb + jj) = col[i2]
-            for (int i2 = jj + 1; i2 < w; ++i2) sh[(kb + i2) * 32 + lane] -= (T)col[i2] * xj;
-          }
-        }
-        __syncthreads();
-        for (int i = kb + w + warp; i < nd; i += nw) {
-          T acc = sh[i * 32 + lane];
-          for (int j = 0; j < w; ++j) acc -= (T)A[ts[kb + j] + i] * sh[(kb + j) * 32 + lane];
-          sh[i * 32 + lane] = acc;
-        }
-        __syncthreads();
+    // Blocked by 32 in shared memory: one warp solves each diagonal block (R
+    // rows at a time), then every warp applies the block's columns to the
+    // remaining rows.  The block is column-major with leading dimension nd
+    // in LU storage (the same address for all lanes of a row).  Backward
+    // values are scaled as they are found.
+    const T *D = A + S.dense_base;
+    const auto sub = [&](int i, const P &x, T a) {
+      P y = shp[i * W];
+#pragma unroll
+      for (int q = 0; q < C; ++q) y.v[q] -= a * x.v[q];
+      shp[i * W] = y;
+    };
+    const auto apply = [&](int i, int kb, int w) {
+      P acc = shp[i * W];
+      const T *di = D + (size_t)kb * nd + i;
+#pragma unroll 4
+      for (int j = 0; j < w; ++j) {
+        const T a = di[(size_t)j * nd];
+        const P x = shp[(kb + j) * W];
+#pragma unroll
+        for (int q = 0; q < C; ++q) acc.v[q] -= a * x.v[q];
       }
-      for (int kb = ((nd - 1) / 32) * 32; kb >= 0; kb -= 32) {
-        const int w = min(32, nd - kb);
-        if (warp == 0) {
-          for (int jj = w - 1; jj >= 0; --jj) {
-            const T xj = sh[(kb + jj) * 32 + lane] * (T)r[t0 + kb + jj];
-            sh[(kb + jj) * 32 + lane] = xj;
-            const double *col = A + ts[kb + jj] + kb;  // U(kb + i2, kb + jj) = col[i2]
-            for (int i2 = 0; i2 < jj; ++i2) sh[(kb + i2) * 32 + lane] -= (T)col[i2] * xj;
-          }
-        }
-        __syncthreads();
-        for (int i = warp; i < kb; i += nw) {
-          T acc = sh[i * 32 + lane];
-          for (int j = 0; j < w; ++j) acc -= (T)A[ts[kb + j] + i] * sh[(kb + j) * 32 + lane];
-          sh[i * 32 + lane] = acc;
-        }
-        __syncthreads();
-      }
-      for (int e = tid; e < nd * 32; e += bd) {
-        const int i = e >> 5, q = e & 31;
-        if (bpanel) {
-          if (q == 0) bs[t0 + i] = sh[i * 32];
-        } else if (c0 + q < nu) {
-          Zs[(size_t)(t0 + i) * nu + c0 + q] = sh[i * 32 + q];
+      shp[i * W] = acc;
+    };
+    for (int kb = 0; kb < nd; kb += 32) {
+      const int w = min(32, nd - kb);
+      if (warp == 0) {
+        for (int jj = 0; jj < w; ++jj) {
+          const P xj = shp[(kb + jj) * W];
+          const T *col = D + (size_t)(kb + jj) * nd + kb;  // L(kb + i2, kb + jj) = col[i2]
+          for (int i2 = jj + 1 + lane / W; i2 < w; i2 += R) sub(kb + i2, xj, col[i2]);
+          __syncwarp();
         }
       }
       __syncthreads();
-    } else {
-      // in place in Z (trailing block too large for shared memory):
-      // forward, dense unit-lower part, column by column
-      for (int k = 0; k < nd - 1; ++k) {
-        const int m = (nd - k - 1) * 32;
-        for (int e = tid; e < m; e += bd) {
-          const int i = k + 1 + (e >> 5), q = e & 31;
-          const T l = (T)A[ts[i * nd + k]];
-          if (c0 + q < nu) Zs[(size_t)(t0 + i) * nu + c0 + q] -= l * Zs[(size_t)(t0 + k) * nu + c0 + q];
-        }
-        __syncthreads();
-      }
-      // backward, dense upper part (unscaled accumulators; x_k = acc_k / u_kk)
-      for (int k = nd - 1; k > 0; --k) {
-        const T rk = (T)r[t0 + k];
-        const int m = k * 32;
-        for (int e = tid; e < m; e += bd) {
-          const int i = e >> 5, q = e & 31;
-          const T u = (T)A[ts[i * nd + k]];
-          if (c0 + q < nu) Zs[(size_t)(t0 + i) * nu + c0 + q] -= u * (Zs[(size_t)(t0 + k) * nu + c0 + q] * rk);
-        }
-        __syncthreads();
-      }
-      for (int e = tid; e < nd * 32; e += bd) {
-        const int i = e >> 5, q = e & 31;
-        if (c0 + q < nu) {
-          T *dst = &Zs[(size_t)(t0 + i) * nu + c0 + q];
-          *dst = *dst * (T)r[t0 + i];
+      for (int i = kb + w + grp; i < nd; i += ngrp) apply(i, kb, w);
+      __syncthreads();
+    }
+    for (int kb = ((nd - 1) / 32) * 32; kb >= 0 && nd > 0; kb -= 32) {
+      const int w = min(32, nd - kb);
+      if (warp == 0) {
+        for (int jj = w - 1; jj >= 0; --jj) {
+          P xj = shp[(kb + jj) * W];
+          const T rk = r[t0 + kb + jj];
+#pragma unroll
+          for (int q = 0; q < C; ++q) xj.v[q] *= rk;
+          __syncwarp();
+          if (lane < W) shp[(kb + jj) * W] = xj;
+          const T *col = D + (size_t)(kb + jj) * nd + kb;  // U(kb + i2, kb + jj) = col[i2]
+          for (int i2 = lane / W; i2 < jj; i2 += R) sub(kb + i2, xj, col[i2]);
+          __syncwarp();
         }
       }
       __syncthreads();
+      for (int i = grp; i < kb; i += ngrp) apply(i, kb, w);
+      __syncthreads();
     }
-  }
-  }  // phase != 2
-  if (phase == 1) return;
-  // backward, sparse rows
-  for (int l = 0; l < S.nlev_bs; ++l) {
-    for (int e = S.bs_lev_ptr[l] + warp; e < S.bs_lev_ptr[l + 1]; e += nw) {
-      const int row = S.bs_rows[e];
-      T acc = zb[(size_t)row * zst];
-      for (int f = S.br_ptr[row]; f < S.br_ptr[row + 1]; ++f)
-        acc -= (T)A[S.br_uslot[f]] * zb[(size_t)S.br_col[f] * zst];
-      if (wr) zw[(size_t)row * zst] = acc * (T)r[row];
-    }
+    for (int i = grp; i < nd; i += ngrp) *zrow(t0 + i) = shp[i * W];
     __syncthreads();
   }
-  if (bpanel) return;  // b needs no product with K
-  for (int row = warp; row < nx; row += nw) {
-    T acc = 0;
-    for (int e = S.kx_ptr[row]; e < S.kx_ptr[row + 1]; ++e) {
-      const int col = S.kx_col[e];
-      const T v = (T)K[(size_t)S.kx_src[e] * N + sc];
-      if (col < nx) acc += v * Zs[(size_t)col * nu + cc];
-      else if (col - nx == cc) acc += v;
+  // backward, sparse rows
+  sweep_rows<T, W, C, U, true>(
+      S.nlev_bs, [&](int l) { return S.bs_lev_ptr[l]; },
+      [&](int e) {
+        const int4 q = S.bs4[e];
+        return RowDesc{q.x, q.y, q.z - q.y};
+      },
+      lu_meta(S.br2), lu_value, zread, [&](int row) { return *zrow(row); },
+      [&](int row, P acc) {
+        const T rr = r[row];
+#pragma unroll
+        for (int q = 0; q < C; ++q) acc.v[q] *= rr;
+        *zrow(row) = acc;
+      });
+  if (bs)
+#pragma unroll
+    for (int q = 0; q < C; ++q)
+      if (c + q * W == nu)
+        for (int row = grp; row < nx; row += ngrp) bs[row] = Zp[(size_t)row * PW + cl * C + q];
+  // an operand of K's products: a row of Z, or of I (places from nx on: no
+  // product in the other columns, whatever the entry)
+  const auto zi_read = [&](int p, bool &mine) {
+    if (p < nx) return *zrow(p);
+    P z = {};
+    mine = false;
+#pragma unroll
+    for (int q = 0; q < C; ++q) {
+      z.v[q] = (T)(p - nx == c + q * W);
+      mine |= p - nx == c + q * W;
     }
-    if (valid) Ys[(size_t)row * nu + c] = acc;
-    if (ezy) {
-      // largest biased exponents of the row of Z and of Y (the row balancing
-      // of the emulated contraction), over the panels by atomic maximum;
-      // ezy[k] for Z and ezy[N nx + k] for Y, k = sc nx + row
-      unsigned ez = 0, ey = 0;
-      if (valid) {
-        ez = (unsigned)(((unsigned long long)__double_as_longlong((double)Zs[(size_t)row * nu + c]) >> 52) & 0x7FF);
-        ey = (unsigned)(((unsigned long long)__double_as_longlong((double)acc) >> 52) & 0x7FF);
-      }
-      ez = __reduce_max_sync(0xffffffffu, ez);
-      ey = __reduce_max_sync(0xffffffffu, ey);
-      if (lane == 0) {
-        const size_t k = (size_t)sc * nx + row;
-        if (ez) atomicMax(&ezy[k], (int)ez);
-        if (ey) atomicMax(&ezy[(size_t)N * nx + k], (int)ey);
-      }
-    }
-  }
-  for (int j = warp; j < nu; j += nw) {
-    double acc = 0.0;
-    for (int e = S.ku_ptr[j]; e < S.ku_ptr[j + 1]; ++e) {
-      const int col = S.ku_col[e];
-      const double v = K[(size_t)S.ku_src[e] * N + sc];
-      if (col < nx) acc += v * (double)Zs[(size_t)col * nu + cc];
-      else if (col - nx == cc) acc += v;
-    }
-    if (valid) Yus[(size_t)j * nu + c] = acc;
-  }
+    return z;
+  };
+  const T *Ks = Kp ? Kp + (size_t)sc * S.kx_ptr[nx] : nullptr;
+  sweep_rows<T, W, C, U, false>(
+      1, [&](int l) { return l * nx; },
+      [&](int row) { return RowDesc{row, S.kx_ptr[row], S.kx_ptr[row + 1] - S.kx_ptr[row]}; },
+      [&](int f, int &col, int &slot) {
+        if (Ks) {
+          col = S.kx_col[f];
+          slot = f;
+        } else {
+          const int2 p = S.kx2[f];
+          col = p.x;
+          slot = p.y;
+        }
+      },
+      [&](int slot) { return Ks ? Ks[slot] : (T)K[(size_t)slot * N + sc]; }, zi_read, [](int) { return P{}; },
+      [&](int row, const P &acc) {
+        const P own = *zrow(row);
+        const size_t at = (size_t)(unsigned)row * (unsigned)nu + c;
+        // largest biased exponents of the row of Z and of Y (the row balancing
+        // of the emulated contraction), over the panels by atomic maximum;
+        // ezy[k] for Z and ezy[N nx + k] for Y, k = sc nx + row
+        const auto expo = [](T v) {
+          return (unsigned)(((unsigned long long)__double_as_longlong((double)v) >> 52) & 0x7FF);
+        };
+        unsigned ez = 0, ey = 0;
+#pragma unroll
+        for (int q = 0; q < C; ++q)
+          if (c + q * W < nu) {
+            Zs[at + q * W] = own.v[q];
+            Ys[at + q * W] = acc.v[q];
+            if (ezy) {
+              ez = max(ez, expo(own.v[q]));
+              ey = max(ey, expo(acc.v[q]));
+            }
+          }
+        if (ezy) {
+          const unsigned lanes = W == 32 ? 0xffffffffu : ((1u << W) - 1) << (lane - cl);
+          ez = __reduce_max_sync(lanes, ez);
+          ey = __reduce_max_sync(lanes, ey);
+          if (cl == 0) {
+            const size_t k = (size_t)sc * nx + row;
+            if (ez) atomicMax(&ezy[k], (int)ez);
+            if (ey) atomicMax(&ezy[(size_t)N * nx + k], (int)ey);
+          }
+        }
+      });
+  sweep_rows<double, W, C, U, false>(
+      1, [&](int l) { return l * nu; },
+      [&](int j) { return RowDesc{j, S.ku_ptr[j], S.ku_ptr[j + 1] - S.ku_ptr[j]}; },
+      [&](int f, int &col, int &slot) {
+        col = S.ku_col[f];
+        slot = S.ku_src[f];
+      },
+      [&](int slot) { return K[(size_t)slot * N + sc]; },
+      [&](int p, bool &mine) {
+        const P z = zi_read(p, mine);
+        Pack<double, C> d;
+#pragma unroll
+        for (int q = 0; q < C; ++q) d.v[q] = (double)z.v[q];
+        return d;
+      },
+      [](int) { return Pack<double, C>{}; },
+      [&](int j, const Pack<double, C> &acc) {
+#pragma unroll
+        for (int q = 0; q < C; ++q)
+          if (c + q * W < nu) Yus[(size_t)j * nu + c + q * W] = acc.v[q];
+      });
 }
 
-// 5 CTAs per SM (shared memory and registers sized for it): the 640 CTAs of
-// 64 scenarios x 10 panels then run in one wave on 152 SMs instead of 1.05
-__global__ void __launch_bounds__(256, 5) k_zsolve64(DevSym S, const double *__restrict__ LU,
+// A CTA works through (scenario, panel) items blockIdx.x, blockIdx.x +
+// gridDim.x, ... (the panels of a scenario side by side: they read the same
+// factors), each in its own slice of the work buffer.  5 CTAs of 256 threads
+// per SM (shared memory and registers sized for it).
+template <int W, int C>
+__global__ void __launch_bounds__(256, 5) k_zsolve64(DevSym S, int npan, const double *__restrict__ LU,
                                                   const double *__restrict__ rd,
                                                   const double *__restrict__ J,
-                                                  const double *__restrict__ K, double *Z, double *Y,
-                                                  double *Yu, int tail_smem, const double *__restrict__ gvec,
+                                                  const double *__restrict__ K, double *work, double *Z, double *Y,
+                                                  double *Yu, const double *__restrict__ gvec,
                                                   double *bvec, int *ezy, int phase) {
-  extern __shared__ double shd[];
-  zsolve_body<double>(S, LU, rd, J, K, Z, Y, Yu, tail_smem != 0, shd, gvec, bvec, ezy, phase);
+  extern __shared__ __align__(16) unsigned char smz[];
+  const size_t E = (size_t)S.nx * S.nu;
+  for (int it = blockIdx.x; it < npan * S.N; it += gridDim.x) {
+    const int sc = it / npan;
+    zsolve_panel<double, W, C>(S, sc, it - sc * npan, LU + (size_t)sc * S.nnzLU, rd + (size_t)sc * S.nx, J, K, nullptr,
+                               work + (size_t)blockIdx.x * S.nx * (W * C), Z + sc * E, Y + sc * E,
+                               Yu + (size_t)sc * S.nu * S.nu, reinterpret_cast<double *>(smz), gvec,
+                               bvec ? bvec + (size_t)sc * S.nx : nullptr, ezy, phase);
+    __syncthreads();
+  }
 }
 
-__global__ void __launch_bounds__(256, 5) k_zsolve32(DevSym S, const double *__restrict__ LU,
-                                                  const double *__restrict__ rd,
+template <int W, int C>
+__global__ void __launch_bounds__(256, 5) k_zsolve32(DevSym S, int npan, const float *__restrict__ LUf,
+                                                  const float *__restrict__ rdf, const float *__restrict__ Kf,
                                                   const double *__restrict__ J,
-                                                  const double *__restrict__ K, float *Z, float *Y,
-                                                  double *Yu, int tail_smem, int phase) {
-  extern __shared__ float shf[];
-  zsolve_body<float>(S, LU, rd, J, K, Z, Y, Yu, tail_smem != 0, shf, nullptr, (float *)nullptr, nullptr, phase);
+                                                  const double *__restrict__ K, float *work, float *Z, float *Y,
+                                                  double *Yu, int phase) {
+  extern __shared__ __align__(16) unsigned char smz[];
+  const size_t E = (size_t)S.nx * S.nu;
+  for (int it = blockIdx.x; it < npan * S.N; it += gridDim.x) {
+    const int sc = it / npan;
+    zsolve_panel<float, W, C>(S, sc, it - sc * npan, LUf + (size_t)sc * round_lu_len(S), rdf + (size_t)sc * S.nx, J, K,
+                              Kf, work + (size_t)blockIdx.x * S.nx * (W * C), Z + sc * E, Y + sc * E,
+                              Yu + (size_t)sc * S.nu * S.nu, reinterpret_cast<float *>(smz), nullptr,
+                              (float *)nullptr, nullptr, phase);
+    __syncthreads();
+  }
+}
+
+// FP32 copies of the factor values the mixed path's solve reads (the whole
+// LU, or its sparse part when the trailing block has kernels of its own) and
+// of the reciprocal pivots: one conversion per value (12 B each).
+__global__ void k_round_factors(DevSym S, const double *__restrict__ LU, const double *__restrict__ rd, float *LUf,
+                                float *rdf) {
+  const int sc = blockIdx.y, n = round_lu_len(S), p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p < n) LUf[(size_t)sc * n + p] = (float)LU[(size_t)sc * S.nnzLU + p];
+  else if (p - n < S.nx) rdf[(size_t)sc * S.nx + p - n] = (float)rd[(size_t)sc * S.nx + p - n];
+}
+
+// FP32 copy of K in the order of the row lists of K_x, scenario-major (K
+// itself is scenario-fastest): 32 x 32 tiles through shared memory.
+__global__ void __launch_bounds__(256) k_round_k(DevSym S, int nk, const double *__restrict__ K, float *Kf) {
+  __shared__ float tile[32][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, e0 = blockIdx.x * 32, s0 = blockIdx.y * 32;
+  for (int q = w; q < 32; q += 8) {
+    const int e = e0 + q, sc = s0 + lane;
+    if (e < nk && sc < S.N) tile[q][lane] = (float)K[(size_t)S.kx2[e].y * S.N + sc];
+  }
+  __syncthreads();
+  for (int q = w; q < 32; q += 8) {
+    const int e = e0 + lane, sc = s0 + q;
+    if (e < nk && sc < S.N) Kf[(size_t)sc * nk + e] = tile[lane][q];
+  }
 }
 
 // In-place solve of G_x v = b (trans = 0) or G_x^T v = b (trans = 1) for every
@@ -872,46 +1043,108 @@ void launch_lu_factor(const DevSym &S, int nL, const double *J, double *LU, doub
   (void)cap;
   k_lu_factor<<<S.N, 512, smem, st>>>(S, nL, J, LU, rd, flags, 1e-14, ns); ipm_count_launch();
 }
-static int zsolve_smem_ok(const DevSym &S, size_t elem) {
-  return (S.nd > 0 && (size_t)S.nd * 32 * elem <= 100 * 1024) ? 1 : 0;
+// b rides along unless the trailing block has kernels of its own
+bool zsolve64_folds_b(const DevSym &S) { return !S.big; }
+
+// CTAs of a multi-RHS solve that are on the GPU at once
+constexpr int ZS_CTAS = 5 * 152;
+
+// Columns per panel: 32, or 16 or 8 to spread a small problem over more SMs
+// and to level the last wave of a larger one.  Every SM works through
+// ceil(panels / 152) panels of w columns, so the width with the least
+// w ceil(panels / 152) is taken, the wider at a tie within an eighth (its
+// fetches serve more columns).
+static int zsolve_width(const DevSym &S, int ncol) {
+  if (S.big) return 32;
+  int best = 32;
+  long long cost = 0;
+  for (int w : {32, 16, 8}) {
+    const long long items = (long long)((ncol + w - 1) / w) * S.N, c = w * ((items + 151) / 152);
+    if (w == 32 || 8 * c < 7 * cost) best = w, cost = c;
+  }
+  return best;
 }
-bool zsolve64_folds_b(const DevSym &S) { return !S.big && (S.nd == 0 || zsolve_smem_ok(S, sizeof(double))); }
+// 128 threads when more panels share an SM than five CTAs of 256 can hold
+static int zsolve_cta(long long items, int w, int threads) { return w < 32 && items > ZS_CTAS ? 128 : threads; }
+static int zsolve_grid(long long items, int threads) {
+  return (int)(items < ZS_CTAS * (256 / threads) ? items : ZS_CTAS * (256 / threads));
+}
+
+size_t zsolve_work_bytes(const DevSym &S, size_t elem) {
+  size_t most = 0;
+  for (int threads : {128, 256})
+    for (int w : {8, 16, 32})
+      for (int extra : {0, 1}) {
+        const long long items = (long long)((S.nu + extra + w - 1) / w) * S.N;
+        const size_t b = (size_t)zsolve_grid(items, zsolve_cta(items, w, threads)) * S.nx * w * elem;
+        if (w == zsolve_width(S, S.nu + extra) && b > most) most = b;
+      }
+  return most;
+}
+
+template <int W, int C>
+static void zsolve64_launch(const DevSym &S, const double *LU, const double *rd, const double *J, const double *K,
+                            double *work, double *Z, double *Y, double *Yu, cudaStream_t st, int threads,
+                            const double *g, double *b, int *ezy, int phase) {
+  // dynamic plus static shared memory may pass the 48 KB default
+  static const bool cap = raise_smem_cap(k_zsolve64<W, C>);
+  (void)cap;
+  const int npan = (S.nu + (b ? 1 : 0) + W * C - 1) / (W * C);
+  const size_t bytes = phase == 0 ? (size_t)S.nd * W * C * sizeof(double) : 0;
+  threads = zsolve_cta((long long)npan * S.N, W * C, threads);
+  k_zsolve64<W, C><<<zsolve_grid((long long)npan * S.N, threads), threads, bytes, st>>>(
+      S, npan, LU, rd, J, K, work, Z, Y, Yu, g, b, ezy, phase);
+  ipm_count_launch();
+}
 
 void launch_zsolve64(const DevSym &S, const double *LU, const double *rd, const double *J,
-                     const double *K, double *Z, double *Y, double *Yu, cudaStream_t st, int threads,
+                     const double *K, double *work, double *Z, double *Y, double *Yu, cudaStream_t st, int threads,
                      const double *g, double *b, int *ezy) {
-  const int sm = zsolve_smem_ok(S, sizeof(double));
-  if (!zsolve64_folds_b(S)) b = nullptr;
-  dim3 grid((S.nu + 31) / 32 + (b ? 1 : 0), S.N);
-  const size_t bytes = sm ? (size_t)S.nd * 32 * sizeof(double) : 0;
-  // dynamic plus static shared memory may pass the 48 KB default
-  static const bool cap = raise_smem_cap(k_zsolve64);
-  (void)cap;
   if (S.big) {
-    // forward sparse rows and the block's right-hand sides, the block by the
-    // batched triangular solves, then the backward sparse rows and products
-    k_zsolve64<<<grid, threads, 0, st>>>(S, LU, rd, J, K, Z, Y, Yu, 0, g, b, ezy, 1); ipm_count_launch();
+    // the block's right-hand sides, the block by the batched triangular
+    // solves, then the sparse rows and products
+    zsolve64_launch<16, 2>(S, LU, rd, J, K, work, Z, Y, Yu, st, threads, nullptr, nullptr, ezy, 1);
     launch_big_trsm64(S, LU, rd, Z, st);
-    k_zsolve64<<<grid, threads, 0, st>>>(S, LU, rd, J, K, Z, Y, Yu, 0, g, b, ezy, 2); ipm_count_launch();
+    zsolve64_launch<16, 2>(S, LU, rd, J, K, work, Z, Y, Yu, st, threads, nullptr, nullptr, ezy, 2);
     return;
   }
-  k_zsolve64<<<grid, threads, bytes, st>>>(S, LU, rd, J, K, Z, Y, Yu, sm, g, b, ezy, 0); ipm_count_launch();
+  switch (zsolve_width(S, S.nu + (b ? 1 : 0))) {
+    case 8: zsolve64_launch<4, 2>(S, LU, rd, J, K, work, Z, Y, Yu, st, threads, g, b, ezy, 0); break;
+    case 16: zsolve64_launch<8, 2>(S, LU, rd, J, K, work, Z, Y, Yu, st, threads, g, b, ezy, 0); break;
+    default: zsolve64_launch<16, 2>(S, LU, rd, J, K, work, Z, Y, Yu, st, threads, g, b, ezy, 0);
+  }
 }
-void launch_zsolve32(const DevSym &S, const double *LU, const double *rd, const double *J,
-                     const double *K, float *Z, float *Y, double *Yu, cudaStream_t st, int threads,
-                     const TcsPlan *tcs, int *flags) {
-  dim3 grid((S.nu + 31) / 32, S.N);
-  const int sm = zsolve_smem_ok(S, sizeof(float));
-  const size_t bytes = sm ? (size_t)S.nd * 32 * sizeof(float) : 0;
-  static const bool cap = raise_smem_cap(k_zsolve32);
+
+template <int W, int C>
+static void zsolve32_launch(const DevSym &S, const RoundedFactors &f, const double *J, const double *K, float *work,
+                            float *Z, float *Y, double *Yu, cudaStream_t st, int threads, int phase) {
+  static const bool cap = raise_smem_cap(k_zsolve32<W, C>);
   (void)cap;
+  const int npan = (S.nu + W * C - 1) / (W * C);
+  const size_t bytes = phase == 0 ? (size_t)S.nd * W * C * sizeof(float) : 0;
+  threads = zsolve_cta((long long)npan * S.N, W * C, threads);
+  k_zsolve32<W, C><<<zsolve_grid((long long)npan * S.N, threads), threads, bytes, st>>>(
+      S, npan, f.LUf, f.rdf, f.Kf, J, K, work, Z, Y, Yu, phase);
+  ipm_count_launch();
+}
+
+void launch_zsolve32(const DevSym &S, const double *LU, const double *rd, const double *J,
+                     const double *K, const RoundedFactors &f, float *work, float *Z, float *Y, double *Yu,
+                     cudaStream_t st, int threads, const TcsPlan *tcs, int *flags) {
+  k_round_factors<<<dim3((round_lu_len(S) + S.nx + 255) / 256, S.N), 256, 0, st>>>(S, LU, rd, f.LUf, f.rdf);
+  ipm_count_launch();
+  k_round_k<<<dim3((f.nk + 31) / 32, (S.N + 31) / 32), 256, 0, st>>>(S, f.nk, K, f.Kf); ipm_count_launch();
   if (S.big) {
-    k_zsolve32<<<grid, threads, 0, st>>>(S, LU, rd, J, K, Z, Y, Yu, 0, 1); ipm_count_launch();
+    zsolve32_launch<8, 4>(S, f, J, K, work, Z, Y, Yu, st, threads, 1);
     launch_big_trsm32(S, LU, rd, Z, st, tcs, flags);
-    k_zsolve32<<<grid, threads, 0, st>>>(S, LU, rd, J, K, Z, Y, Yu, 0, 2); ipm_count_launch();
+    zsolve32_launch<8, 4>(S, f, J, K, work, Z, Y, Yu, st, threads, 2);
     return;
   }
-  k_zsolve32<<<grid, threads, bytes, st>>>(S, LU, rd, J, K, Z, Y, Yu, sm, 0); ipm_count_launch();
+  switch (zsolve_width(S, S.nu)) {
+    case 8: zsolve32_launch<4, 2>(S, f, J, K, work, Z, Y, Yu, st, threads, 0); break;
+    case 16: zsolve32_launch<8, 2>(S, f, J, K, work, Z, Y, Yu, st, threads, 0); break;
+    default: zsolve32_launch<8, 4>(S, f, J, K, work, Z, Y, Yu, st, threads, 0);
+  }
 }
 void launch_solve1(const DevSym &S, const double *LU, const double *rd, double *v, int trans,
                    cudaStream_t st) {
