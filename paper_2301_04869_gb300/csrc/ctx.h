@@ -32,7 +32,7 @@ struct ipm_ctx {
   int *tile_of = nullptr;
   int ntiles = 0, nt1 = 0, ngroups = 0;
   long long kchunk = 0;
-  double *Khat = nullptr, *M = nullptr, *F = nullptr, *diag1 = nullptr, *rhs_u = nullptr;
+  double *Khat = nullptr, *M = nullptr, *F = nullptr, *Finv = nullptr, *diag1 = nullptr, *rhs_u = nullptr;
   double *rhs_corr = nullptr, *cpos = nullptr;  // d(rhs_u)/d(delta); scratch [N][max(nx,nu)]
   double *gLu = nullptr, *HTt_u = nullptr;
   double *pg_curv = nullptr, *pmax_d = nullptr;

@@ -9,6 +9,8 @@
 constexpr int LU_LISTS = 1024;  // lists of trailing-block products of the LU factorization
 #endif
 
+constexpr int SWP = 4;  // products per lane of a single-vector sweep unit
+
 struct DevSym {
   int n, L, ng, N, nx, nu, m, nnzA, nnzKB, nnzLU, nlev, nlev_b, nlev_f, t0, nd, nlev_fs, nlev_bs;
   int nflow;  // line-flow rows of h (2 L with ratings, else 0)
@@ -31,8 +33,15 @@ struct DevSym {
   const int *tw_len, *tw_l, *tw_u, *tw_e;  // trailing-block products per LU thread
   const int *fw_lev_ptr, *fw_rows, *fr_ptr, *fr_col, *fr_lslot, *fr_uslot;
   const int *bw_lev_ptr, *bw_rows, *br_ptr, *br_col, *br_uslot, *br_lslot;
-  const int *fs_lev_ptr, *fs_rows, *bs_lev_ptr, *bs_rows;
-  const int4 *fs4, *bs4, *fr4, *br4;  // packed single-RHS sweeps (symbolic.cpp)
+  const int *bs_lev_ptr;
+  const int4 *bs4;  // backward sparse rows {row, first product, end, 0}
+  // units of the single-vector sweeps (symbolic.cpp) and the inverses of the
+  // trailing block's diagonal blocks they use (kernels_solve1.cu)
+  const int2 *sw_item, *sw_extra;
+  const int *sw_row, *swf_lev, *swb_lev;
+  int swf_n, swb_n;
+  size_t sw_items;  // items of one direction (the transposed ones follow)
+  double *dinv;
   const int *gu_ptr, *gu_col, *gu_src, *gut_ptr, *gut_col, *gut_src;
   const int *kx_ptr, *kx_col, *kx_src, *ku_ptr, *ku_col, *ku_src;
   // the same product lists as {column, slot} pairs (zp_col/zp_slot,

@@ -121,15 +121,18 @@ ipm_status upload_symbolic(ipm_ctx *c, const HostNet &net, const double *pd, con
   TRY(upload(c, &d.perm, S.perm)); TRY(upload(c, &d.iperm, S.iperm));
   TRY(upload(c, &d.lu_diag, S.lu_diag)); TRY(upload(c, &d.lu_init, S.lu_init));
   TRY(upload(c, &d.tail_slot, S.tail_slot));
-  TRY(upload(c, &d.fs_lev_ptr, S.fs_lev_ptr)); TRY(upload(c, &d.fs_rows, S.fs_rows));
   {
     const int *q = nullptr;
-    TRY(upload(c, &q, S.fs4)); d.fs4 = reinterpret_cast<const int4 *>(q);
     TRY(upload(c, &q, S.bs4)); d.bs4 = reinterpret_cast<const int4 *>(q);
-    TRY(upload(c, &q, S.fr4)); d.fr4 = reinterpret_cast<const int4 *>(q);
-    TRY(upload(c, &q, S.br4)); d.br4 = reinterpret_cast<const int4 *>(q);
+    TRY(upload(c, &q, S.sw_item)); d.sw_item = reinterpret_cast<const int2 *>(q);
+    TRY(upload(c, &q, S.sw_extra)); d.sw_extra = reinterpret_cast<const int2 *>(q);
   }
-  TRY(upload(c, &d.bs_lev_ptr, S.bs_lev_ptr)); TRY(upload(c, &d.bs_rows, S.bs_rows));
+  d.sw_items = S.sw_item.size() / 4;
+  TRY(upload(c, &d.sw_row, S.sw_row)); TRY(upload(c, &d.swf_lev, S.swf_lev)); TRY(upload(c, &d.swb_lev, S.swb_lev));
+  d.swf_n = (int)S.swf_lev.size() - 1;
+  d.swb_n = (int)S.swb_lev.size() - 1;
+  TRY(dalloc(c, &d.dinv, diag_inverse_doubles(d)));
+  TRY(upload(c, &d.bs_lev_ptr, S.bs_lev_ptr));
   TRY(upload(c, &d.f_lev_ptr, S.f_lev_ptr)); TRY(upload(c, &d.f_piv_ptr, S.f_piv_ptr)); TRY(upload(c, &d.f_piv, S.f_piv));
   TRY(upload(c, &d.f_tgt, S.f_tgt)); TRY(upload(c, &d.f_op_ptr, S.f_op_ptr)); TRY(upload(c, &d.f_op_l, S.f_op_l));
   TRY(upload(c, &d.f_op_u, S.f_op_u)); TRY(upload(c, &d.f_op_k, S.f_op_k));
@@ -318,6 +321,7 @@ ipm_status alloc_work(ipm_ctx *c) {
   CK(cudaMemcpy(c->tile_of, tof.data(), tof.size() * sizeof(int), cudaMemcpyHostToDevice));
   TRY(dalloc(c, &c->partial, (long long)c->max_groups * c->ntiles * 4096));
   TRY(dalloc(c, &c->Khat, nu * nu)); TRY(dalloc(c, &c->M, nu * nu)); TRY(dalloc(c, &c->F, nu * nu));
+  TRY(dalloc(c, &c->Finv, chol_inverse_doubles((int)nu)));
   TRY(dalloc(c, &c->diag1, nu)); TRY(dalloc(c, &c->rhs_u, nu));
   TRY(dalloc(c, &c->rhs_corr, nu)); TRY(dalloc(c, &c->cpos, N * std::max(nx, nu)));
   TRY(dalloc(c, &c->gLu, nu)); TRY(dalloc(c, &c->HTt_u, nu));
@@ -536,7 +540,7 @@ ipm_status run_part(ipm_ctx *c, cudaGraphExec_t &gx, long long &gn, Fn fn, cudaS
 void launch_adjoint_reduce(ipm_ctx *c, cudaStream_t st) {
   const DevSym &S = c->ds;
   launch_transpose_rows(S.N, S.nx, S.nu, c->Y, c->Wadj, st);
-  launch_solve1_batched(S, c->dw.LU, c->dw.rd, c->Wadj, 1, S.nu, 128, st);
+  launch_solve1_batched(S, c->dw.LU, c->dw.rd, c->Wadj, 1, S.nu, st);
   launch_adjoint_assemble(S, c->dw.J, c->Yu, c->Wadj, c->diag1, c->Khat, st);
 }
 
@@ -930,6 +934,7 @@ ipm_status do_factor(ipm_ctx *c, double delta, int *is_pd, cudaStream_t st, doub
   launch_shift(S.nu, c->Khat, c->M, delta, tau, c->F, st);
   CK(cudaMemsetAsync(c->dw.flags + FLAG_NOT_PD, 0, sizeof(int), st));
   launch_cholesky(S.nu, c->F, c->dw.flags, st);
+  launch_chol_inverse(S.nu, c->F, c->Finv, st);
   ph_end(c, PH_CHOL, st);
   CK(cudaGetLastError());
   TRY(read_flags(c, st));
@@ -967,11 +972,11 @@ ipm_status pcg_reduced(ipm_ctx *c, double delta, cudaStream_t st) {
   double *x = c->pu, *b = c->pcg_b, *r = c->pcg_r, *z = c->pcg_z, *p = c->pcg_p, *Ap = c->pcg_Ap;
   c->neg_curv = false;
   CK(cudaMemcpyAsync(b, x, nu * sizeof(double), cudaMemcpyDeviceToDevice, st));
-  launch_chol_solve(nu, c->F, x, st);
+  launch_chol_solve(nu, c->F, c->Finv, x, st);
   TRY(reduced_apply(c, x, Ap, delta, st));
   launch_lincomb(nu, r, 1.0, b, -1.0, Ap, 0.0, nullptr, st);
   CK(cudaMemcpyAsync(z, r, nu * sizeof(double), cudaMemcpyDeviceToDevice, st));
-  launch_chol_solve(nu, c->F, z, st);
+  launch_chol_solve(nu, c->F, c->Finv, z, st);
   CK(cudaMemcpyAsync(p, z, nu * sizeof(double), cudaMemcpyDeviceToDevice, st));
   launch_dot2(nu, r, z, b, b, c->red_out, st);
   TRY(read_red(c, 2, st));
@@ -995,7 +1000,7 @@ ipm_status pcg_reduced(ipm_ctx *c, double delta, cudaStream_t st) {
     launch_lincomb(nu, x, 1.0, x, alpha, p, 0.0, nullptr, st);
     launch_lincomb(nu, r, 1.0, r, -alpha, Ap, 0.0, nullptr, st);
     CK(cudaMemcpyAsync(z, r, nu * sizeof(double), cudaMemcpyDeviceToDevice, st));
-    launch_chol_solve(nu, c->F, z, st);
+    launch_chol_solve(nu, c->F, c->Finv, z, st);
     launch_dot2(nu, r, z, r, r, c->red_out, st);
     TRY(read_red(c, 2, st));
     const double rz_new = c->h_red[0];
@@ -1072,7 +1077,7 @@ ipm_status refine_aug(ipm_ctx *c, double delta, cudaStream_t st) {
       solve1(c, c->apos2, 1, st);
       launch_rhs_reduced(S, D.J, D.K, c->arh2, c->apos2, c->bpos2, c->dpu, st);
     }
-    launch_chol_solve(S.nu, c->F, c->dpu, st);
+    launch_chol_solve(S.nu, c->F, c->Finv, c->dpu, st);
     // Prop. 2.3: dp_x = -G_x^{-1}(r3' + G_u dp_u), dp_y = -G_x^{-T}(rhat1_x + (K_xx + delta) dp_x + K_xu dp_u)
     if (zfp64) {
       CK(cudaMemcpyAsync(c->vpos2, c->bpos2, NX * sizeof(double), cudaMemcpyDeviceToDevice, st));
@@ -1122,7 +1127,7 @@ ipm_status do_solve(ipm_ctx *c, cudaStream_t st, bool defer_py = false) {
   ph_begin(c, PH_RECOVER, st);
   launch_lincomb(S.nu, c->pu, 1.0, c->rhs_u, delta, delta != 0.0 ? c->rhs_corr : nullptr, 0.0, nullptr, st);
   if (!c->mixed || c->exact_iter) {
-    launch_chol_solve(S.nu, c->F, c->pu, st);
+    launch_chol_solve(S.nu, c->F, c->Finv, c->pu, st);
     // p_x = -G_x^{-1} (r3 + G_u p_u) = Z p_u - b
     CK(cudaMemcpyAsync(c->vpos, c->bpos, NX * sizeof(double), cudaMemcpyDeviceToDevice, st));
     launch_z_apply(S, c->Z, c->pu, -1.0, c->vpos, st);
@@ -1131,7 +1136,7 @@ ipm_status do_solve(ipm_ctx *c, cudaStream_t st, bool defer_py = false) {
       TRY(pcg_reduced(c, delta, st));
     } else {
       // the mixed-precision factor alone; refinement on eq. (6) follows
-      launch_chol_solve(S.nu, c->F, c->pu, st);
+      launch_chol_solve(S.nu, c->F, c->Finv, c->pu, st);
       c->refine_iters = 0;
       c->refine_res = 0.0;
       c->neg_curv = false;

@@ -74,10 +74,18 @@ struct Sym {
   long long n_tail_ops = 0;
   std::vector<int> fw_lev_ptr, fw_rows, fr_ptr, fr_col, fr_lslot, fr_uslot;
   std::vector<int> bw_lev_ptr, bw_rows, br_ptr, br_col, br_uslot, br_lslot;
-  // packed single-RHS sweeps (4 ints each): per scheduled row {row, first, end, 0}
-  // (fs4: forward sparse rows, bs4: backward), per product {col, slot, transposed slot, 0}
-  // (fr4 over fr_*, br4 over br_*)
-  std::vector<int> fs4, bs4, fr4, br4;
+  // backward sparse rows by level, 4 ints each: {row, first product, end, 0}
+  std::vector<int> bs4;
+  // The single-vector sweeps in units of one warp and four products per lane:
+  // product h of lane l of unit u is the pair {column, slot} at
+  // sw_item[2 ((4 u + h) 32 + l)], slot -1 for none; the same with the
+  // transposed slots follows (second half).  sw_row[32 u + l]: the lane's row
+  // and, from bit 26, the unit's code, -1 for no row; a row takes
+  // 2^(code & 7) neighbouring lanes.  Rows of more than 128 products (code &
+  // 8) go on in the units sw_extra[2 u] = {first, count}.  Units of level l:
+  // swf_lev[l] .. swf_lev[l + 1] (forward: the sparse levels, then one more
+  // for the sparse part of the trailing rows), swb_lev for the backward rows.
+  std::vector<int> sw_item, sw_row, sw_extra, swf_lev, swb_lev;
   // sparse operators by position (x rows) or u rows
   std::vector<int> gu_ptr, gu_col, gu_src;
   std::vector<int> gut_ptr, gut_col, gut_src;

@@ -55,9 +55,6 @@ bool zsolve64_folds_b(const DevSym &S);
 void launch_big_lu_dense(const DevSym &S, double *LU, double *rd, const double *amax, int *flags, cudaStream_t st,
                          const EmuLuPlan *emu_lu = nullptr);
 void launch_big_trsm64(const DevSym &S, const double *LU, const double *rd, double *Z, cudaStream_t st);
-// one vector per scenario (v: [N][n_x], positions) through the block: forward
-// then backward, with G_x (trans 0) or G_x^T (trans 1)
-void launch_big_trsv(const DevSym &S, const double *LU, const double *rd, double *v, int trans, cudaStream_t st);
 struct TcsPlan;
 // tcs: the tensor-core variant of the block updates (mixed path), or null
 void launch_big_trsm32(const DevSym &S, const double *LU, const double *rd, float *Z, cudaStream_t st,
@@ -73,12 +70,16 @@ __host__ __device__ inline int round_lu_len(const DevSym &S) { return S.big ? S.
 void launch_zsolve32(const DevSym &S, const double *LU, const double *rd, const double *J, const double *K,
                      const RoundedFactors &f, float *work, float *Z, float *Y, double *Yu, cudaStream_t st, int threads = 256,
                      const TcsPlan *tcs = nullptr, int *flags = nullptr);
+// kernels_solve1.cu: inverses of the trailing block's diagonal blocks (into
+// S.dinv, after every factorization), and solves of one vector per scenario
+// (v: [N][n_x], position order) with G_x (trans 0) or G_x^T (trans 1)
+size_t diag_inverse_doubles(const DevSym &S);
+void launch_diag_inverse(const DevSym &S, const double *LU, const double *rd, cudaStream_t st);
 void launch_solve1(const DevSym &S, const double *LU, const double *rd, double *v, int trans,
                    cudaStream_t st);
-// vps vectors per scenario: v [N * vps][n_x] (position order), one CTA of
-// `threads` (a multiple of 32) per vector
+// vps vectors per scenario: v [N * vps][n_x] (position order), one CTA per vector
 void launch_solve1_batched(const DevSym &S, const double *LU, const double *rd, double *v, int trans, int vps,
-                           int threads, cudaStream_t st);
+                           cudaStream_t st);
 // kernels_adjoint.cu: the paper's local reduction by adjoint solves
 // (K_hat V = L_u - G_u^T G_x^{-T} L_x, §3.2) on all n_u unit vectors at once
 void launch_transpose_rows(int N, int nx, int nu, const double *Y, double *W, cudaStream_t st);
@@ -104,7 +105,11 @@ void launch_shift(int nu, const double *Khat, const double *M, double delta, dou
                   cudaStream_t st);
 void launch_maxdiag(int n, const double *A, double *out, cudaStream_t st);
 void launch_cholesky(int n, double *A, int *flags, cudaStream_t st);
-void launch_chol_solve(int n, const double *L, double *b, cudaStream_t st);
+// inverses of the factor's diagonal blocks (after a successful
+// factorization), which the solves use
+size_t chol_inverse_doubles(int n);
+void launch_chol_inverse(int n, const double *L, double *inv, cudaStream_t st);
+void launch_chol_solve(int n, const double *L, const double *inv, double *b, cudaStream_t st);
 
 // kernels_step.cu
 void launch_errors(const DevSym &S, DevWork &D, const double *gLu, double *partial, double *out,

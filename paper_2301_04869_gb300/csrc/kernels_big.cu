@@ -352,161 +352,6 @@ void btrsm_tc(const DevSym &S, const double *LU, const double *rd, float *Z, con
   }
 }
 
-// ---- one vector per scenario through the block ------------------------------
-//
-// T(i, k) is the entry of the triangular factor a sweep applies: forward
-// (lower) T = L, or U^T with trans; backward (upper) T = U, or L^T with
-// trans.  In the column-major block T(i, k) = LU[k nd + i] without trans and
-// LU[i nd + k] with it; the sweeps that apply U or U^T multiply by the
-// reciprocal pivots.  Blocked by VB rows: a launch per block applies the
-// block's solved values to every later row, 64 rows per CTA over (chunk,
-// scenario), so the factor streams through many SMs at once; the CTA holding
-// the next block's rows then solves that diagonal block (a warp, in shared
-// memory).
-constexpr int VB = 64;
-
-template <bool TRANS>
-__device__ __forceinline__ double tval(const double *A, int nd, int i, int k) {
-  return TRANS ? A[(size_t)i * nd + k] : A[(size_t)k * nd + i];
-}
-
-// the diagonal block [b0, b1) (at most VB rows) in place on xs (indexed from
-// b0); called by the whole CTA
-template <bool TRANS, bool UPPER>
-__device__ void trsv_diag(const double *A, const double *r, int nd, int b0, int b1, double *xs,
-                          double (*Dg)[VB + 1]) {
-  const int tid = threadIdx.x, w = b1 - b0;
-  for (int e = tid; e < w * w; e += blockDim.x) {
-    const int i = e % w, k = e / w;
-    Dg[i][k] = tval<TRANS>(A, nd, b0 + i, b0 + k);
-  }
-  __syncthreads();
-  if (tid < 32) {
-    const int lane = tid;
-    constexpr bool scale = TRANS != UPPER;  // U^T going down or U coming up
-    double y0 = lane < w ? xs[lane] : 0.0, y1 = lane + 32 < w ? xs[lane + 32] : 0.0;
-    for (int s = 0; s < w; ++s) {
-      const int k = UPPER ? w - 1 - s : s;
-      double own = k < 32 ? y0 : y1;
-      if (scale) own *= r[b0 + k];
-      const double xk = __shfl_sync(0xffffffffu, own, k & 31);
-      if ((k & 31) == lane) {
-        if (k < 32) y0 = xk;
-        else y1 = xk;
-      }
-      if (UPPER) {
-        if (lane < k) y0 = fma(-Dg[lane][k], xk, y0);
-        if (lane + 32 < k) y1 = fma(-Dg[lane + 32][k], xk, y1);
-      } else {
-        if (lane > k && lane < w) y0 = fma(-Dg[lane][k], xk, y0);
-        if (lane + 32 > k && lane + 32 < w) y1 = fma(-Dg[lane + 32][k], xk, y1);
-      }
-    }
-    if (lane < w) xs[lane] = y0;
-    if (lane + 32 < w) xs[lane + 32] = y1;
-  }
-  __syncthreads();
-}
-
-// the first diagonal block of a sweep (lower: [0, VB), upper: the last one)
-template <bool TRANS, bool UPPER>
-__global__ void __launch_bounds__(256) k_trsv_first(int nd, int nx, int t0, long long nnzlu, int dense_base,
-                                                    const double *__restrict__ LU, const double *__restrict__ rd,
-                                                    double *v) {
-  __shared__ double xs[VB];
-  __shared__ double Dg[VB][VB + 1];
-  const int sc = blockIdx.x, tid = threadIdx.x;
-  const double *A = LU + (size_t)sc * nnzlu + dense_base;
-  const double *r = rd + (size_t)sc * nx + t0;
-  double *x = v + (size_t)sc * nx + t0;
-  const int b0 = UPPER ? ((nd - 1) / VB) * VB : 0, b1 = UPPER ? nd : min(nd, VB);
-  if (tid < b1 - b0) xs[tid] = x[b0 + tid];
-  __syncthreads();
-  trsv_diag<TRANS, UPPER>(A, r, nd, b0, b1, xs, Dg);
-  if (tid < b1 - b0) x[b0 + tid] = xs[tid];
-}
-
-// rows of chunk blockIdx.x minus T(rows, [kb, ke)) x([kb, ke)); chunk 0 is
-// the next diagonal block (lower: [ke, ke + VB), upper: [kb - VB, kb)),
-// solved after its update.  Grid (chunks, N), 256 threads.
-template <bool TRANS, bool UPPER>
-__global__ void __launch_bounds__(256) k_trsv_step(int nd, int nx, int t0, long long nnzlu, int dense_base,
-                                                   const double *__restrict__ LU, const double *__restrict__ rd,
-                                                   double *v, int kb, int ke) {
-  __shared__ double xk[VB];
-  __shared__ double part[4][VB];
-  __shared__ double xs[VB];
-  __shared__ double Dg[VB][VB + 1];
-  const int sc = blockIdx.y, tid = threadIdx.x, c = blockIdx.x;
-  const double *A = LU + (size_t)sc * nnzlu + dense_base;
-  const double *r = rd + (size_t)sc * nx + t0;
-  double *x = v + (size_t)sc * nx + t0;
-  int c0, c1;
-  if (UPPER) {
-    c1 = kb - VB * c;
-    c0 = c1 - VB > 0 ? c1 - VB : 0;
-  } else {
-    c0 = ke + VB * c;
-    c1 = c0 + VB < nd ? c0 + VB : nd;
-  }
-  const int w = ke - kb, h = c1 - c0;
-  if (tid < VB) xk[tid] = tid < w ? x[kb + tid] : 0.0;
-  __syncthreads();
-  if (!TRANS) {
-    // T(i, k) = LU[k nd + i]: a thread per (row, 16 columns), loads along the rows
-    const int rr = tid & (VB - 1), g = tid >> 6;
-    double s = 0.0;
-    if (rr < h)
-      for (int j = 16 * g; j < 16 * g + 16 && j < w; ++j) s = fma(A[(size_t)(kb + j) * nd + c0 + rr], xk[j], s);
-    part[g][rr] = s;
-  } else {
-    // T(i, k) = LU[i nd + k]: a warp per (row group, 32 columns), lanes along the columns
-    const int wp = tid >> 5, lane = tid & 31, rg = wp >> 1, hf = wp & 1, j = 32 * hf + lane;
-    const double xj = xk[j];
-    for (int m = 0; m < VB / 4; ++m) {
-      const int rr = rg + 4 * m;
-      double p = (rr < h && j < w) ? A[(size_t)(c0 + rr) * nd + kb + j] * xj : 0.0;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
-      if (lane == 0) part[hf][rr] = p;
-    }
-    if (tid < VB) part[2][tid] = part[3][tid] = 0.0;
-  }
-  __syncthreads();
-  if (tid < h) {
-    const double nv = x[c0 + tid] - ((part[0][tid] + part[1][tid]) + (part[2][tid] + part[3][tid]));
-    xs[tid] = nv;
-    if (c != 0) x[c0 + tid] = nv;
-  }
-  __syncthreads();
-  if (c == 0) {
-    trsv_diag<TRANS, UPPER>(A, r, nd, c0, c1, xs, Dg);
-    if (tid < h) x[c0 + tid] = xs[tid];
-  }
-}
-
-template <bool TRANS>
-void trsv_sweeps(const DevSym &S, const double *LU, const double *rd, double *v, cudaStream_t st) {
-  const int nd = S.nd;
-  k_trsv_first<TRANS, false><<<S.N, 256, 0, st>>>(nd, S.nx, S.t0, S.nnzLU, S.dense_base, LU, rd, v);
-  ipm_count_launch();
-  for (int kb = 0; kb + VB < nd; kb += VB) {
-    const int ke = kb + VB;
-    k_trsv_step<TRANS, false><<<dim3((nd - ke + VB - 1) / VB, S.N), 256, 0, st>>>(nd, S.nx, S.t0, S.nnzLU,
-                                                                                 S.dense_base, LU, rd, v, kb, ke);
-    ipm_count_launch();
-  }
-  const int lb = ((nd - 1) / VB) * VB;
-  k_trsv_first<TRANS, true><<<S.N, 256, 0, st>>>(nd, S.nx, S.t0, S.nnzLU, S.dense_base, LU, rd, v);
-  ipm_count_launch();
-  for (int kb = lb; kb > 0; kb -= VB) {
-    const int ke = kb + VB < nd ? kb + VB : nd;
-    k_trsv_step<TRANS, true><<<dim3(kb / VB, S.N), 256, 0, st>>>(nd, S.nx, S.t0, S.nnzLU, S.dense_base, LU, rd, v,
-                                                                kb, ke);
-    ipm_count_launch();
-  }
-}
-
 }  // namespace
 
 void launch_big_lu_dense(const DevSym &S, double *LU, double *rd, const double *amax, int *flags, cudaStream_t st,
@@ -546,9 +391,4 @@ void launch_big_trsm32(const DevSym &S, const double *LU, const double *rd, floa
     return;
   }
   btrsm<float>(S, LU, rd, Z, st);
-}
-
-void launch_big_trsv(const DevSym &S, const double *LU, const double *rd, double *v, int trans, cudaStream_t st) {
-  if (trans) trsv_sweeps<true>(S, LU, rd, v, st);
-  else trsv_sweeps<false>(S, LU, rd, v, st);
 }

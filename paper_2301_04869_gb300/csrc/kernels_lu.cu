@@ -1,6 +1,6 @@
 // K3-K5: batched static-pivot sparse LU of G_x (one pattern for all
-// scenarios), the multi-RHS reduction solves Z = -G_x^{-1} G_u fused with the
-// products Y = K [Z; I], and single-vector solves with G_x and G_x^T.
+// scenarios) and the multi-RHS reduction solves Z = -G_x^{-1} G_u fused with
+// the products Y = K [Z; I].
 //
 // Paper: §3.2 "Assembling the sparse matrices" (batched LU sharing one
 // pattern, G_x^{-1} b = Q U^{-1} L^{-1} P b) and "Local reduction" (steps
@@ -681,209 +681,6 @@ __global__ void __launch_bounds__(256) k_round_k(DevSym S, int nk, const double 
   }
 }
 
-// In-place solve of G_x v = b (trans = 0) or G_x^T v = b (trans = 1) for every
-// scenario; v is [N][nx] in LU position order.  One CTA per scenario: sparse
-// rows by levels (one warp per row, lanes over the row's entries), the dense
-// trailing block column by column in shared memory.
-// Sum over a group of GS consecutive lanes (GS a power of two <= 32).
-template <int GS>
-__device__ __forceinline__ double group_sum(double p) {
-#pragma unroll
-  for (int o = GS / 2; o > 0; o >>= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
-  return p;
-}
-
-// One level of sparse rows, GS lanes per row: x[row] = (x[row] - sum_f
-// A[slot_f] x[col_f]) * (scale ? r[row] : 1) over the row's products.  A
-// scheduled row is one 16-byte record {row, first, end} and a product one
-// {col, slot, transposed slot}, so each row costs three dependent loads
-// (record, product, value).  Rows of a level are independent; the loop
-// bounds are uniform over the CTA (shuffles).
-template <int GS>
-__device__ __forceinline__ void solve_level(const int4 *__restrict__ rows, int e0, int e1,
-                                            const int4 *__restrict__ prod, bool trans_slot,
-                                            const double *__restrict__ A, const double *__restrict__ r, bool scale,
-                                            double *x) {
-  const int grp = threadIdx.x / GS, sub = threadIdx.x % GS, ngrp = blockDim.x / GS;
-  for (int eb = e0; eb < e1; eb += ngrp) {
-    const int e = eb + grp;
-    double part = 0.0;
-    int row = -1;
-    if (e < e1) {
-      const int4 R = rows[e];
-      row = R.x;
-      for (int f = R.y + sub; f < R.z; f += GS) {
-        const int4 P = prod[f];
-        part = fma(A[trans_slot ? P.z : P.y], x[P.x], part);
-      }
-    }
-    part = group_sum<GS>(part);
-    if (sub == 0 && row >= 0) x[row] = scale ? (x[row] - part) * r[row] : x[row] - part;
-  }
-}
-
-// One CTA per vector: vector b of v ([N * vps][n_x], position order) belongs
-// to scenario b / vps (vps vectors per scenario share its factors).
-// phase (large trailing block, S.big): 1 = the forward sparse rows and the
-// sparse part of the trailing rows only, 2 = the backward sparse rows only
-// (the dense block between them by the batched kernels of kernels_big.cu);
-// 0 = all.
-__global__ void __launch_bounds__(1024) k_solve1(DevSym S, const double *__restrict__ LU, const double *__restrict__ rd,
-                                                double *v, int trans, int in_smem, int vps, int phase) {
-  extern __shared__ double xsm[];
-  __shared__ double blk[32][33];
-  const int sc = blockIdx.x / vps, tid = threadIdx.x, bd = blockDim.x;
-  const int lane = tid & 31, warp = tid >> 5;
-  const int nx = S.nx, t0 = S.t0, nd = S.nd;
-  const double *A = LU + (size_t)sc * S.nnzLU;
-  const double *r = rd + (size_t)sc * nx;
-  double *vs = v + (size_t)blockIdx.x * nx;
-  // the solution vector of this scenario lives in shared memory when it fits
-  double *x = in_smem ? xsm : vs;
-  if (in_smem) {
-    for (int i = tid; i < nx; i += bd) x[i] = vs[i];
-    __syncthreads();
-  }
-  // forward sparse rows (few entries each): four lanes per row
-  for (int l = 0; l < (phase == 2 ? 0 : S.nlev_fs); ++l) {
-    solve_level<4>(S.fs4, S.fs_lev_ptr[l], S.fs_lev_ptr[l + 1], S.fr4, trans != 0, A, r, trans != 0, x);
-    __syncthreads();
-  }
-  if (nd > 0 && phase != 2) {
-    const int *ts = S.tail_slot;
-    double *tv = x + t0;
-    // sparse part of the trailing rows (their columns < t0), eight lanes per row
-    {
-      const int grp = tid / 8, sub = tid % 8, ngrp = bd / 8;
-      for (int ib = 0; ib < nd; ib += ngrp) {
-        const int i = ib + grp;
-        double part = 0.0;
-        if (i < nd) {
-          const int row = t0 + i;
-          for (int f = S.fr_ptr[row] + sub; f < S.fr_ptr[row + 1]; f += 8) {
-            const int4 P = S.fr4[f];
-            if (P.x < t0) part = fma(A[trans ? P.z : P.y], x[P.x], part);
-          }
-        }
-        part = group_sum<8>(part);
-        if (sub == 0 && i < nd) tv[i] -= part;
-      }
-    }
-    __syncthreads();
-    if (phase == 1) {
-      if (in_smem)
-        for (int i = tid; i < nx; i += bd) vs[i] = x[i];
-      return;
-    }
-    // Dense trailing block, blocked by 32: one warp per 32 x 32 diagonal
-    // block (lane = row, shuffles), all threads for the off-diagonal updates
-    // (four partial sums).  Column c of the block is contiguous in LU
-    // storage: entry (a, c) sits at tail_slot[c] + a.  Forward: T = L (unit)
-    // or U^T (diagonal u_kk); backward: T = U or L^T.  Where T has the
-    // diagonal u_kk the block multipliers are pre-scaled by 1/u_kk, so each
-    // step of the diagonal solve is one shuffle and one multiply-add.
-    for (int kb = 0; kb < nd; kb += 32) {
-      const int w = min(32, nd - kb);
-      for (int e = tid; e < 32 * 32; e += bd) {
-        const int rr = e >> 5, cc = e & 31;
-        double bv = 0.0;
-        if (rr < w && cc < rr) bv = trans ? A[ts[kb + rr] + kb + cc] * r[t0 + kb + cc] : A[ts[kb + cc] + kb + rr];
-        blk[rr][cc] = bv;
-      }
-      __syncthreads();
-      if (warp == 0) {
-        double xv = lane < w ? tv[kb + lane] : 0.0;
-        for (int jj = 0; jj < w; ++jj) {
-          const double xj = __shfl_sync(0xffffffffu, xv, jj);
-          if (lane > jj) xv = fma(-blk[lane][jj], xj, xv);
-        }
-        if (lane < w) tv[kb + lane] = trans ? xv * r[t0 + kb + lane] : xv;
-      }
-      __syncthreads();
-      for (int i = kb + w + tid; i < nd; i += bd) {
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-        int j = 0;
-        if (trans) {
-          const double *col = A + ts[i] + kb;  // U(kb + j, i), j = 0..w-1
-          for (; j + 4 <= w; j += 4) {
-            s0 = fma(col[j], tv[kb + j], s0);
-            s1 = fma(col[j + 1], tv[kb + j + 1], s1);
-            s2 = fma(col[j + 2], tv[kb + j + 2], s2);
-            s3 = fma(col[j + 3], tv[kb + j + 3], s3);
-          }
-          for (; j < w; ++j) s0 = fma(col[j], tv[kb + j], s0);
-        } else {
-          for (; j + 4 <= w; j += 4) {
-            s0 = fma(A[ts[kb + j] + i], tv[kb + j], s0);
-            s1 = fma(A[ts[kb + j + 1] + i], tv[kb + j + 1], s1);
-            s2 = fma(A[ts[kb + j + 2] + i], tv[kb + j + 2], s2);
-            s3 = fma(A[ts[kb + j + 3] + i], tv[kb + j + 3], s3);
-          }
-          for (; j < w; ++j) s0 = fma(A[ts[kb + j] + i], tv[kb + j], s0);
-        }
-        tv[i] -= (s0 + s1) + (s2 + s3);
-      }
-      __syncthreads();
-    }
-    for (int kb = ((nd - 1) / 32) * 32; kb >= 0; kb -= 32) {
-      const int w = min(32, nd - kb);
-      for (int e = tid; e < 32 * 32; e += bd) {
-        const int rr = e >> 5, cc = e & 31;
-        double bv = 0.0;
-        if (rr < w && cc < w && cc > rr) bv = trans ? A[ts[kb + rr] + kb + cc] : A[ts[kb + cc] + kb + rr] * r[t0 + kb + cc];
-        blk[rr][cc] = bv;
-      }
-      __syncthreads();
-      if (warp == 0) {
-        double xv = lane < w ? tv[kb + lane] : 0.0;
-        for (int jj = w - 1; jj >= 0; --jj) {
-          const double xj = __shfl_sync(0xffffffffu, xv, jj);
-          if (lane < jj) xv = fma(-blk[lane][jj], xj, xv);
-        }
-        if (lane < w) tv[kb + lane] = trans ? xv : xv * r[t0 + kb + lane];
-      }
-      __syncthreads();
-      for (int i = tid; i < kb; i += bd) {
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-        int j = 0;
-        if (trans) {
-          const double *col = A + ts[i] + kb;  // L(kb + j, i), j = 0..w-1
-          for (; j + 4 <= w; j += 4) {
-            s0 = fma(col[j], tv[kb + j], s0);
-            s1 = fma(col[j + 1], tv[kb + j + 1], s1);
-            s2 = fma(col[j + 2], tv[kb + j + 2], s2);
-            s3 = fma(col[j + 3], tv[kb + j + 3], s3);
-          }
-          for (; j < w; ++j) s0 = fma(col[j], tv[kb + j], s0);
-        } else {
-          for (; j + 4 <= w; j += 4) {
-            s0 = fma(A[ts[kb + j] + i], tv[kb + j], s0);
-            s1 = fma(A[ts[kb + j + 1] + i], tv[kb + j + 1], s1);
-            s2 = fma(A[ts[kb + j + 2] + i], tv[kb + j + 2], s2);
-            s3 = fma(A[ts[kb + j + 3] + i], tv[kb + j + 3], s3);
-          }
-          for (; j < w; ++j) s0 = fma(A[ts[kb + j] + i], tv[kb + j], s0);
-        }
-        tv[i] -= (s0 + s1) + (s2 + s3);
-      }
-      __syncthreads();
-    }
-  }
-  if (phase == 1) {  // (no trailing block)
-    if (in_smem)
-      for (int i = tid; i < nx; i += bd) vs[i] = x[i];
-    return;
-  }
-  // backward sparse rows: eight lanes per row
-  for (int l = 0; l < S.nlev_bs; ++l) {
-    solve_level<8>(S.bs4, S.bs_lev_ptr[l], S.bs_lev_ptr[l + 1], S.br4, trans != 0, A, r, trans == 0, x);
-    __syncthreads();
-  }
-  if (in_smem)
-    for (int i = tid; i < nx; i += bd) vs[i] = x[i];
-}
-
-
 // The same factorization by a cluster of two CTAs per scenario (two SMs'
 // FP64 units): the sparse part shared by index parity; the nd x nd
 // trailing block is then split by column panels of 16, panel q
@@ -1028,6 +825,7 @@ void launch_lu_factor(const DevSym &S, int nL, const double *J, double *LU, doub
     // sparse part (one CTA per scenario), then the block by the batched kernels
     k_lu_factor<<<S.N, 512, 0, st>>>(S, nL, J, LU, rd, flags, 1e-14, 0); ipm_count_launch();
     launch_big_lu_dense(S, LU, rd, S.lu_amax, flags, st, emu_lu);
+    launch_diag_inverse(S, LU, rd, st);
     return;
   }
   const int np = (S.nd + 15) / 16, ldl = ((np + 1) / 2) * 16;
@@ -1035,6 +833,7 @@ void launch_lu_factor(const DevSym &S, int nL, const double *J, double *LU, doub
   if (allow_pair && S.nd > 0 && pair_smem <= pair_cap) {
     k_lu_factor_pair<<<2 * S.N, 512, pair_smem, st>>>(S, nL, J, LU, rd, flags, 1e-14);
     ipm_count_launch();
+    launch_diag_inverse(S, LU, rd, st);
     return;
   }
   const int ns = S.nd < ns_max ? S.nd : ns_max;
@@ -1042,6 +841,7 @@ void launch_lu_factor(const DevSym &S, int nL, const double *J, double *LU, doub
   static const bool cap = raise_smem_cap(k_lu_factor);
   (void)cap;
   k_lu_factor<<<S.N, 512, smem, st>>>(S, nL, J, LU, rd, flags, 1e-14, ns); ipm_count_launch();
+  launch_diag_inverse(S, LU, rd, st);
 }
 // b rides along unless the trailing block has kernels of its own
 bool zsolve64_folds_b(const DevSym &S) { return !S.big; }
@@ -1145,45 +945,4 @@ void launch_zsolve32(const DevSym &S, const double *LU, const double *rd, const 
     case 16: zsolve32_launch<8, 2>(S, f, J, K, work, Z, Y, Yu, st, threads, 0); break;
     default: zsolve32_launch<8, 4>(S, f, J, K, work, Z, Y, Yu, st, threads, 0);
   }
-}
-void launch_solve1(const DevSym &S, const double *LU, const double *rd, double *v, int trans,
-                   cudaStream_t st) {
-  // the scenario's vector in shared memory when it fits next to the
-  // kernel's static shared memory
-  static const size_t cap = [] {
-    int dev = 0, optin = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    cudaFuncAttributes fa;
-    cudaFuncGetAttributes(&fa, k_solve1);
-    return raise_smem_cap(k_solve1) ? (size_t)optin - fa.sharedSizeBytes : (size_t)0;
-  }();
-  const int sm = (size_t)S.nx * sizeof(double) <= cap ? 1 : 0;
-  const size_t bytes = sm ? (size_t)S.nx * sizeof(double) : 0;
-  if (S.big) {
-    // sparse rows in one CTA of 1,024 threads per scenario (the level sweeps
-    // of the large networks are long: more rows in flight per round); the
-    // dense block by the batched single-vector kernels (many CTAs per scenario)
-    k_solve1<<<S.N, 1024, bytes, st>>>(S, LU, rd, v, trans, sm, 1, 1); ipm_count_launch();
-    launch_big_trsv(S, LU, rd, v, trans, st);
-    k_solve1<<<S.N, 1024, bytes, st>>>(S, LU, rd, v, trans, sm, 1, 2); ipm_count_launch();
-    return;
-  }
-  k_solve1<<<S.N, 512, bytes, st>>>(S, LU, rd, v, trans, sm, 1, 0); ipm_count_launch();
-}
-
-void launch_solve1_batched(const DevSym &S, const double *LU, const double *rd, double *v, int trans, int vps,
-                           int threads, cudaStream_t st) {
-  static const size_t cap = [] {
-    int dev = 0, optin = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    cudaFuncAttributes fa;
-    cudaFuncGetAttributes(&fa, k_solve1);
-    return raise_smem_cap(k_solve1) ? (size_t)optin - fa.sharedSizeBytes : (size_t)0;
-  }();
-  const int sm = (size_t)S.nx * sizeof(double) <= cap ? 1 : 0;
-  const size_t bytes = sm ? (size_t)S.nx * sizeof(double) : 0;
-  const long long nb = (long long)S.N * vps;
-  k_solve1<<<(unsigned)nb, threads, bytes, st>>>(S, LU, rd, v, trans, sm, vps, 0); ipm_count_launch();
 }

@@ -79,6 +79,99 @@ void min_degree(int nv, std::vector<std::vector<int>> adj, std::vector<int> &ord
 
 }  // namespace
 
+// The units of the single-vector sweeps (layout in ipm_internal.h).  A level's
+// rows are taken longest first, so that rows packed into a unit are of about
+// one length and the long ones start early.
+static void build_sweeps(Sym &S) {
+  struct Prod {
+    int col, slot, tslot;
+  };
+  struct Level {
+    std::vector<std::pair<int, std::vector<Prod>>> rows;
+  };
+  // extra units follow all scheduled ones; they are kept aside until then
+  std::vector<std::array<int, 3>> long_rows;  // (unit, level list index, row index) of rows of more than one unit
+  std::vector<Level> levels;
+  const auto add = [&](const std::vector<int> &rows, size_t e0, size_t e1, bool fwd, int below) {
+    Level L;
+    for (size_t e = e0; e < e1; ++e) {
+      const int i = rows[e];
+      std::vector<Prod> ps;
+      const std::vector<int> &ptr = fwd ? S.fr_ptr : S.br_ptr, &col = fwd ? S.fr_col : S.br_col;
+      const std::vector<int> &slot = fwd ? S.fr_lslot : S.br_uslot, &tslot = fwd ? S.fr_uslot : S.br_lslot;
+      for (int f = ptr[i]; f < ptr[i + 1]; ++f)
+        if (col[f] < below) ps.push_back({col[f], slot[f], tslot[f]});
+      L.rows.push_back({i, std::move(ps)});
+    }
+    std::stable_sort(L.rows.begin(), L.rows.end(),
+                     [](const auto &a, const auto &b) { return a.second.size() > b.second.size(); });
+    levels.push_back(std::move(L));
+  };
+  for (int l = 0; l < S.nlev_fs; ++l) add(S.fs_rows, S.fs_lev_ptr[l], S.fs_lev_ptr[l + 1], true, S.nx);
+  std::vector<int> tail(S.nd);
+  for (int a = 0; a < S.nd; ++a) tail[a] = S.t0 + a;
+  if (S.nd > 0) add(tail, 0, tail.size(), true, S.t0);
+  const size_t nf = levels.size();
+  for (int l = 0; l < S.nlev_bs; ++l) add(S.bs_rows, S.bs_lev_ptr[l], S.bs_lev_ptr[l + 1], false, S.nx);
+  // one unit: P products per lane, 2^lg lanes per row
+  constexpr int P = 4, FULL = 32 * P;
+  std::vector<int> titem;
+  const auto put = [&](const std::vector<std::pair<int, const Prod *>> &rows, const std::vector<int> &n, int lg, int code) {
+    const int g = 1 << lg;
+    for (int h = 0; h < P; ++h)
+      for (int lane = 0; lane < 32; ++lane) {
+        const size_t q = (size_t)(lane / g);
+        const int f = h * g + lane % g;
+        const bool on = q < rows.size() && f < n[q];
+        const Prod p = on ? rows[q].second[f] : Prod{0, -1, -1};
+        S.sw_item.insert(S.sw_item.end(), {p.col, p.slot});
+        titem.insert(titem.end(), {p.col, p.tslot});
+      }
+    for (int lane = 0; lane < 32; ++lane) {
+      const size_t q = (size_t)(lane / g);
+      S.sw_row.push_back(q < rows.size() ? rows[q].first | code << 26 : -1);
+    }
+  };
+  int units = 0;
+  const auto lanes_lg = [](size_t n) {
+    int lg = 0;
+    while (lg < 5 && (size_t)(P << lg) < n) ++lg;
+    return lg;
+  };
+  for (size_t l = 0; l < levels.size(); ++l) {
+    std::vector<int> &lev = l < nf ? S.swf_lev : S.swb_lev;
+    if (lev.empty()) lev.push_back(units);
+    const auto &rows = levels[l].rows;
+    for (size_t e = 0; e < rows.size();) {
+      const int lg = lanes_lg(rows[e].second.size());
+      std::vector<std::pair<int, const Prod *>> rs;
+      std::vector<int> n;
+      const bool over = rows[e].second.size() > FULL;
+      if (over) long_rows.push_back({units, (int)l, (int)e});
+      for (; e < rows.size() && rs.size() < (size_t)(32 >> lg) && lanes_lg(rows[e].second.size()) == lg; ++e) {
+        rs.push_back({rows[e].first, rows[e].second.data()});
+        n.push_back((int)std::min<size_t>(rows[e].second.size(), FULL));
+      }
+      put(rs, n, lg, lg | (over ? 8 : 0));
+      ++units;
+    }
+    lev.push_back(units);
+  }
+  if (S.swf_lev.empty()) S.swf_lev.assign(1, units);
+  if (S.swb_lev.empty()) S.swb_lev.assign(1, units);
+  S.sw_extra.assign((size_t)std::max(units, 1) * 2, 0);
+  int next = units;
+  for (const auto &lr : long_rows) {
+    const auto &row = levels[lr[1]].rows[lr[2]];
+    S.sw_extra[(size_t)lr[0] * 2] = next;
+    for (size_t f = FULL; f < row.second.size(); f += FULL, ++next) {
+      put({{row.first, row.second.data() + f}}, {(int)std::min<size_t>(row.second.size() - f, FULL)}, 5, 5 | 8);
+      ++S.sw_extra[(size_t)lr[0] * 2 + 1];
+    }
+  }
+  S.sw_item.insert(S.sw_item.end(), titem.begin(), titem.end());
+}
+
 bool build_symbolic(const HostNet &net, int N, Sym &S, std::string &err, int big) {
   const int n = net.n, L = net.L, ng = net.ng;
   if (n < 2 || L < 1 || ng < 1 || N < 1) { err = "bad sizes"; return false; }
@@ -545,18 +638,30 @@ bool build_symbolic(const HostNet &net, int N, Sym &S, std::string &err, int big
       if (any) S.fs_lev_ptr.push_back((int)S.fs_rows.size());
     }
     S.nlev_fs = (int)S.fs_lev_ptr.size() - 1;
-    S.bs_lev_ptr.assign(1, 0);
-    for (int l = 0; l < nlevb; ++l) {
-      bool any = false;
-      for (int i : bl[l])
-        if (i < S.t0) { S.bs_rows.push_back(i); any = true; }
-      if (any) S.bs_lev_ptr.push_back((int)S.bs_rows.size());
+    // (backward: by the dependence among the sparse rows alone, the block
+    // being done before them; with the block's own chain counted, rows of one
+    // such level fell into levels as many as the block has rows: 817 instead
+    // of 25 on a 10,000-bus network)
+    {
+      std::vector<int> bl2(S.t0, 0);
+      int nl = S.t0 > 0 ? 1 : 0;
+      for (int i = S.t0 - 1; i >= 0; --i)
+        for (int k : pat[i])
+          if (k < S.t0) {
+            bl2[i] = std::max(bl2[i], bl2[k] + 1);
+            nl = std::max(nl, bl2[i] + 1);
+          }
+      std::vector<std::vector<int>> rows(nl);
+      for (int i = 0; i < S.t0; ++i) rows[bl2[i]].push_back(i);
+      S.bs_lev_ptr.assign(1, 0);
+      for (int l = 0; l < nl; ++l) {
+        S.bs_rows.insert(S.bs_rows.end(), rows[l].begin(), rows[l].end());
+        S.bs_lev_ptr.push_back((int)S.bs_rows.size());
+      }
     }
     S.nlev_bs = (int)S.bs_lev_ptr.size() - 1;
-    for (int i : S.fs_rows) S.fs4.insert(S.fs4.end(), {i, S.fr_ptr[i], S.fr_ptr[i + 1], 0});
     for (int i : S.bs_rows) S.bs4.insert(S.bs4.end(), {i, S.br_ptr[i], S.br_ptr[i + 1], 0});
-    for (size_t f = 0; f < S.fr_col.size(); ++f) S.fr4.insert(S.fr4.end(), {S.fr_col[f], S.fr_lslot[f], S.fr_uslot[f], 0});
-    for (size_t f = 0; f < S.br_col.size(); ++f) S.br4.insert(S.br4.end(), {S.br_col[f], S.br_uslot[f], S.br_lslot[f], 0});
+    build_sweeps(S);
   }
   // ---- G_u (rows: positions) and its transpose (rows: u) ----
   const int nu = S.nu;
