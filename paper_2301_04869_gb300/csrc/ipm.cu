@@ -364,7 +364,9 @@ ipm_status alloc_work(ipm_ctx *c) {
   TRY(dalloc(c, &c->xt, N * nx)); TRY(dalloc(c, &c->ut, nu)); TRY(dalloc(c, &c->st, N * m));
   TRY(dalloc(c, &c->gt, N * nx)); TRY(dalloc(c, &c->ht, N * m)); TRY(dalloc(c, &c->fst, N));
   TRY(dalloc(c, &c->Pt, N * n)); TRY(dalloc(c, &c->Qt, N * n));
-  TRY(dalloc(c, &c->red_partial, 152 * 8)); TRY(dalloc(c, &c->red_out, 16));
+  // partial values of the reductions, then the count of CTAs that left theirs
+  TRY(dalloc(c, &c->red_partial, 152 * 8 + 1)); TRY(dalloc(c, &c->red_out, 16));
+  CK(cudaMemset(c->red_partial + 152 * 8, 0, sizeof(double)));
   CK(cudaMallocHost(&c->h_red, 16 * sizeof(double)));
   CK(cudaMallocHost(&c->h_flags, FLAG_COUNT * sizeof(int)));
   CK(cudaMallocHost(&c->h_mu, sizeof(double)));

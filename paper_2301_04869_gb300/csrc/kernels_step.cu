@@ -26,14 +26,22 @@ __device__ __forceinline__ double warp_op(int op, double v) {
   return v;
 }
 
+// One launch per reduction: every CTA leaves its partial values, and the one
+// that counts last joins them, a warp per value (lane l takes CTAs l, l + 32,
+// ..., then the lanes in a fixed tree), and sets the count back.  Joining the
+// 152 partial values one after the other in a launch of its own took 40 us
+// for the optimality error's seven (dependent FP64 additions), 11 for the
+// merit's three.
 template <class F>
-__global__ void __launch_bounds__(256) k_reduce(F f, long long n, double *partial) {
+__global__ void __launch_bounds__(256) k_reduce(F f, long long n, double *partial, double *out, unsigned *count) {
+  static_assert(F::NV <= 8, "a warp of the CTA per value");
   double acc[F::NV];
 #pragma unroll
   for (int i = 0; i < F::NV; ++i) acc[i] = op_init(F::op(i));
   for (long long t = (long long)blockIdx.x * 256 + threadIdx.x; t < n; t += (long long)gridDim.x * 256)
     f(t, acc);
   __shared__ double sh[F::NV][8];
+  __shared__ bool last;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
   for (int i = 0; i < F::NV; ++i) {
@@ -41,27 +49,36 @@ __global__ void __launch_bounds__(256) k_reduce(F f, long long n, double *partia
     if (lane == 0) sh[i][w] = v;
   }
   __syncthreads();
-  if (threadIdx.x < F::NV) {
-    const int i = threadIdx.x;
-    double v = sh[i][0];
-    for (int q = 1; q < 8; ++q) v = op_comb(F::op(i), v, sh[i][q]);
-    partial[(size_t)blockIdx.x * F::NV + i] = v;
+  double v = op_init(OP_SUM);
+  if (w < F::NV) {
+    v = lane < 8 ? sh[w][lane] : op_init(F::op(w));
+    v = warp_op(F::op(w), v);
+    if (lane == 0) {
+      (gridDim.x == 1 ? out : partial + (size_t)blockIdx.x * F::NV)[w] = v;
+      __threadfence();
+    }
   }
-}
-
-template <class F>
-__global__ void k_reduce_final(int nb, const double *partial, double *out) {
-  const int i = threadIdx.x;
-  if (i >= F::NV) return;
-  double v = partial[i];
-  for (int b = 1; b < nb; ++b) v = op_comb(F::op(i), v, partial[(size_t)b * F::NV + i]);
-  out[i] = v;
+  if (gridDim.x == 1) return;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const unsigned c = atomicAdd(count, 1u);
+    last = c == gridDim.x - 1;
+    if (last) *count = 0u;
+  }
+  __syncthreads();
+  if (!last || w >= F::NV) return;
+  __threadfence();
+  v = op_init(F::op(w));
+  for (int b = lane; b < (int)gridDim.x; b += 32) v = op_comb(F::op(w), v, __ldcg(&partial[(size_t)b * F::NV + w]));
+  v = warp_op(F::op(w), v);
+  if (lane == 0) out[w] = v;
 }
 
 template <class F>
 void run_reduce(const F &f, long long n, double *partial, double *out, cudaStream_t st) {
-  k_reduce<F><<<RED_BLOCKS, 256, 0, st>>>(f, n, partial); ipm_count_launch();
-  k_reduce_final<F><<<1, 32, 0, st>>>(RED_BLOCKS, partial, out); ipm_count_launch();
+  const int nb = (int)((n + 255) / 256 < RED_BLOCKS ? (n + 255) / 256 : RED_BLOCKS);
+  k_reduce<F><<<nb, 256, 0, st>>>(f, n, partial, out, reinterpret_cast<unsigned *>(partial + RED_BLOCKS * 8));
+  ipm_count_launch();
 }
 
 __device__ __forceinline__ double bgrad(double w, double l, double b, double mu) {
