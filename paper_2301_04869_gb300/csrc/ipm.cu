@@ -300,13 +300,14 @@ ipm_status alloc_work(ipm_ctx *c) {
     }
   c->ntiles = (int)tl.size();
   // split the N*nx contraction rows into equal chunks so that tiles x chunks
-  // fills one wave (3 CTAs of 256 threads per SM, 152 SMs); the buffer of
-  // partial tiles has room for the autotuner's largest candidate (4x)
+  // fills four waves (3 CTAs of 256 threads per SM, 152 SMs): tiles at the
+  // diagonal and the ragged edge do less work, and more waves level that out
+  // (1,000 buses x 64, assembly included: one wave 12.1 ms, two 11.4, three
+  // 10.9, four 10.6)
   {
     const long long G0 = std::max(1, (3 * 152) / c->ntiles);
     set_groups(c, 4 * G0);
     c->max_groups = c->ngroups;
-    set_groups(c, G0);
   }
   {
     // the multi-RHS solve's panels in flight; a mixed context also runs the FP64 solve (fallback iterations)
