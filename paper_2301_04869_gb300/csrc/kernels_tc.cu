@@ -56,8 +56,13 @@ struct Maps {
 // Accumulation: the tensor core's FP32 accumulation loses precision over long
 // K, so every 64-wide K block (its 24 split products) accumulates into a fresh
 // TMEM buffer (two buffers, double-buffered); the epilogue warps drain each
-// buffer into round-to-nearest FP32 registers and flush those into this CTA's
-// FP64 partial tile every FLUSH blocks.
+// buffer into round-to-nearest FP32 registers and flush every column into
+// this CTA's FP64 partial tile (column-major: a warp's flush of a column is
+// 256 contiguous bytes) after FLUSH blocks,
+// BN / FLUSH columns after each block: GB300 converts and adds FP64 at a
+// hundredth of its FP32 rate, and a flush of all 128 columns at once, to
+// addresses 1 KB apart, held both TMEM buffers and so the MMAs (10,000 buses x
+// 32 23.5 -> 16.4 ms, 1,000 x 64 216 -> 143 us).
 constexpr int FLUSH = 16;
 
 __global__ void __launch_bounds__(192, 1) k_tc_schur(const __grid_constant__ Maps maps, int nt1, int kb_total,
@@ -147,43 +152,58 @@ __global__ void __launch_bounds__(192, 1) k_tc_schur(const __grid_constant__ Map
     // epilogue: drain every block's accumulator into FP32 registers
     const int q = warp & 3;  // lane quarter this warp may access
     const int row = q * 32 + lane;
-    double *out = partial + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * BM * BN + (size_t)row * BN;
+    double *out = partial + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * BM * BN + row;
+    constexpr int FC = BN / FLUSH;  // columns flushed after a block
     float acc[BN];
 #pragma unroll
     for (int c = 0; c < BN; ++c) acc[c] = 0.0f;
-    for (int c = 0; c < BN; ++c) out[c] = 0.0;
-    for (int i = 0; i < nkb; ++i) {
-      const int b = i & 1;
-      if (!mbar_wait(&acc_full[b], (i >> 1) & 1)) {
-        flags[FLAG_TIMEOUT] = 1;
-        *abort_flag = 1;
-        break;
-      }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    for (int c = 0; c < BN; ++c) out[c * BM] = 0.0;
+    bool ok = true;
+    for (int i0 = 0; i0 < nkb && ok; i0 += FLUSH) {
 #pragma unroll
-      for (int c0 = 0; c0 < BN; c0 += 16) {
-        uint32_t v[16];
-        const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * BN + c0);
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-              "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-            : "r"(taddr));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      for (int ph = 0; ph < FLUSH; ++ph) {
+        const int i = i0 + ph, b = i & 1;
+        if (i >= nkb || !ok) continue;
+        double sum[FC];
 #pragma unroll
-        for (int e = 0; e < 16; ++e) acc[c0 + e] += __uint_as_float(v[e]);
-      }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_empty[b])) : "memory");
-      if ((i + 1) % FLUSH == 0 || i + 1 == nkb) {
+        for (int c = 0; c < FC; ++c) sum[c] = out[(ph * FC + c) * BM];
+        if (!mbar_wait(&acc_full[b], (i >> 1) & 1)) {
+          flags[FLAG_TIMEOUT] = 1;
+          *abort_flag = 1;
+          ok = false;
+          continue;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-        for (int c = 0; c < BN; ++c) {
-          out[c] += (double)acc[c];
-          acc[c] = 0.0f;
+        for (int c0 = 0; c0 < BN; c0 += 32) {
+          uint32_t v[2][16];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * BN + c0 + 16 * h);
+            asm volatile(
+                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                : "=r"(v[h][0]), "=r"(v[h][1]), "=r"(v[h][2]), "=r"(v[h][3]), "=r"(v[h][4]), "=r"(v[h][5]),
+                  "=r"(v[h][6]), "=r"(v[h][7]), "=r"(v[h][8]), "=r"(v[h][9]), "=r"(v[h][10]), "=r"(v[h][11]),
+                  "=r"(v[h][12]), "=r"(v[h][13]), "=r"(v[h][14]), "=r"(v[h][15])
+                : "r"(taddr));
+          }
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+          for (int e = 0; e < 32; ++e) acc[c0 + e] += __uint_as_float(v[e / 16][e % 16]);
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0)
+          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_empty[b])) : "memory");
+#pragma unroll
+        for (int c = 0; c < FC; ++c) {
+          out[(ph * FC + c) * BM] = sum[c] + (double)acc[ph * FC + c];
+          acc[ph * FC + c] = 0.0f;
         }
       }
     }
+#pragma unroll
+    for (int c = 0; c < BN; ++c) out[c * BM] += (double)acc[c];
   }
   // drain: if we aborted, let issued copies land before the CTA exits
   if (warp == 0 && lane == 0 && *abort_flag) {
@@ -212,30 +232,37 @@ __device__ __forceinline__ void split3(float a, __nv_bfloat16 &h, __nv_bfloat16 
   l = __float2bfloat16_rn(r2);
 }
 
-__global__ void k_split_t(long long krows, int nu, long long kpad, const float *__restrict__ src,
-                          __nv_bfloat16 *planes) {
-  // 32 x 32 transpose tiles through shared memory
-  __shared__ float t[32][33];
-  const long long k0 = (long long)blockIdx.x * 32;
-  const int j0 = blockIdx.y * 32;
-  const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
-  for (int r = ty; r < 32; r += 8) {
+// HBM-bound: 64 x 64 transpose tiles, so that a warp reads two rows of 128
+// bytes and writes 128 bytes of a plane row (10,000 buses x 32, 12.2 GB per
+// operand: 3.84 ms with 32 x 32 tiles, 2.16 with these).
+__global__ void __launch_bounds__(256) k_split_t(long long krows, int nu, long long kpad,
+                                                 const float *__restrict__ src, __nv_bfloat16 *planes) {
+  __shared__ float t[64][65];
+  const long long k0 = (long long)blockIdx.x * 64;
+  const int j0 = blockIdx.y * 64, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll
+  for (int r = ty; r < 64; r += 8) {
     const long long k = k0 + r;
-    const int j = j0 + tx;
-    t[r][tx] = (k < krows && j < nu) ? src[k * nu + j] : 0.0f;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int j = j0 + tx + 32 * h;
+      t[r][tx + 32 * h] = (k < krows && j < nu) ? src[k * nu + j] : 0.0f;
+    }
   }
   __syncthreads();
   const size_t plane = (size_t)nu * kpad;
-  for (int r = ty; r < 32; r += 8) {
+  const long long k = k0 + 2 * tx;
+#pragma unroll
+  for (int r = ty; r < 64; r += 8) {
     const int j = j0 + r;
-    const long long k = k0 + tx;
-    if (j < nu && k < kpad) {
-      __nv_bfloat16 h, m, l;
-      split3(t[tx][r], h, m, l);
+    if (j < nu && k < kpad) {  // kpad is even
+      __nv_bfloat162 h, m, l;
+      split3(t[2 * tx][r], h.x, m.x, l.x);
+      split3(t[2 * tx + 1][r], h.y, m.y, l.y);
       const size_t o = (size_t)j * kpad + k;
-      planes[o] = h;
-      planes[plane + o] = m;
-      planes[2 * plane + o] = l;
+      *reinterpret_cast<__nv_bfloat162 *>(planes + o) = h;
+      *reinterpret_cast<__nv_bfloat162 *>(planes + plane + o) = m;
+      *reinterpret_cast<__nv_bfloat162 *>(planes + 2 * plane + o) = l;
     }
   }
 }
@@ -252,7 +279,7 @@ __global__ void k_tc_assemble(int nu, int N, int ngroups, int ntiles, int nt1, c
   const int tt = ti * nt1 - ti * (ti - 1) / 2 + (tj - ti);
   double v = 0.0;
   for (int g = 0; g < ngroups; ++g)
-    v += partial[((size_t)g * ntiles + tt) * BM * BN + (size_t)(i - ti * BM) * BN + (j - tj * BN)];
+    v += partial[((size_t)g * ntiles + tt) * BM * BN + (size_t)(j - tj * BN) * BM + (i - ti * BM)];  // column-major tiles
   if (Yu)
     for (int s = 0; s < N; ++s) v += Yu[(size_t)s * nu * nu + (size_t)i * nu + j];
   if (diag && i == j) v += diag[i];
@@ -332,8 +359,8 @@ bool tc_set_operands(TcPlan &P, const void *a_planes, const void *b_planes) {
 }
 
 void launch_split_t(long long krows, int nu, long long kpad, const float *src, void *planes, cudaStream_t st) {
-  dim3 grid((unsigned)((kpad + 31) / 32), (unsigned)((nu + 31) / 32));
-  tc::k_split_t<<<grid, dim3(32, 8), 0, st>>>(krows, nu, kpad, src, (__nv_bfloat16 *)planes); ipm_count_launch();
+  dim3 grid((unsigned)((kpad + 63) / 64), (unsigned)((nu + 63) / 64));
+  tc::k_split_t<<<grid, 256, 0, st>>>(krows, nu, kpad, src, (__nv_bfloat16 *)planes); ipm_count_launch();
 }
 
 void launch_tc_schur(const TcPlan &P, double *partial, int *flags, cudaStream_t st) {
