@@ -229,12 +229,9 @@ void launch_emu_split_pair(const EmuPlan &P, const double *Z, const double *Y, c
 void launch_emu_schur(const EmuPlan &P, double *partial, int *flags, cudaStream_t st);
 void launch_emu_assemble(const EmuPlan &P, int N, const double *partial, const double *Yu, const double *diag,
                          double *Khat, cudaStream_t st);
-// the large-block LU's updates at FP64 grade on the tensor cores, rows
-// [a0, a0 + na) and columns [b0, b0 + nb) of the block by its columns and rows
-// [kb, ke) (at most EMU_LU_K): slices of the N scenarios' rows of L and columns
-// of U stacked with stride Mp (nd rounded up to 128), planes
-// [8][N Mp][EMU_LU_K] each
-constexpr int EMU_LU_K = 256;
+// the large-block LU's trailing update A22 -= L21 U12 at FP64 grade on the
+// tensor cores: slices of the N scenarios' L21 rows and U12 columns stacked
+// with stride Mp (nd rounded up to 128), planes [8][N Mp][64] each
 struct EmuLuPlan {
   int N = 0, nd = 0, Mp = 0;
   void *a_planes = nullptr, *b_planes = nullptr;
@@ -243,8 +240,8 @@ struct EmuLuPlan {
 };
 size_t emu_lu_planes_bytes(int N, int nd);
 bool emu_lu_plan(EmuLuPlan &P, int N, int nd, void *a_planes, void *b_planes, int *exp_a, int *exp_b);
-void launch_emu_lu_update(const EmuLuPlan &P, double *LU, long long nnzlu, int dense_base, int kb, int ke, int a0,
-                          int na, int b0, int nb, int *flags, cudaStream_t st);
+void launch_emu_lu_update(const EmuLuPlan &P, double *LU, long long nnzlu, int dense_base, int kb, int ke, int *flags,
+                          cudaStream_t st);
 // kernels_tcsolve.cu: the mixed path's solve through the large trailing
 // block with its updates as BF16x3 products on the tensor cores; planes of
 // the factor block [3][N ndp][kpl] then of the finished rows [3][N nup][kpl]

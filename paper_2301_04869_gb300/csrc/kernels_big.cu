@@ -110,10 +110,10 @@ __global__ void __launch_bounds__(128) k_blu_l21(int nd, int nx, int t0, long lo
     if (c < pb) A[(size_t)(kb + c) * nd + i] = a[c];
 }
 
-// U12 = L11^{-1} A12: columns [c0, c1) of rows [kb, ke); a warp per column,
+// U12 = L11^{-1} A12: columns [ke, nd) of rows [kb, ke); a warp per column,
 // lane l holding rows kb + l and kb + 32 + l; L11 staged in shared memory.
 __global__ void __launch_bounds__(256) k_blu_trsm(int nd, long long nnzlu, int dense_base, double *LU, int kb,
-                                                  int ke, int c0, int c1) {
+                                                  int ke) {
   __shared__ double L11[PB][PB + 1];
   const int sc = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   double *A = LU + (size_t)sc * nnzlu + dense_base;
@@ -123,8 +123,8 @@ __global__ void __launch_bounds__(256) k_blu_trsm(int nd, long long nnzlu, int d
     L11[i][k] = A[(size_t)(kb + k) * nd + kb + i];
   }
   __syncthreads();
-  const int j = c0 + blockIdx.x * 8 + warp;
-  if (j >= c1) return;
+  const int j = ke + blockIdx.x * 8 + warp;
+  if (j >= nd) return;
   double *col = A + (size_t)j * nd + kb;
   double x0 = lane < pb ? col[lane] : 0.0;
   double x1 = lane + 32 < pb ? col[lane + 32] : 0.0;
@@ -360,57 +360,24 @@ void launch_big_lu_dense(const DevSym &S, double *LU, double *rd, const double *
                                                (int)gemm_smem()) == cudaSuccess;
   (void)cap;
   const int nd = S.nd;
-  const auto panel = [&](int kb, int ke) {  // columns [kb, ke), up to date: L11, U11, L21
+  for (int kb = 0; kb < nd; kb += PB) {
+    const int ke = kb + PB < nd ? kb + PB : nd;
     k_blu_diag<<<S.N, 256, 0, st>>>(nd, S.nx, S.t0, S.nnzLU, S.dense_base, LU, rd, amax, 1e-14, flags, kb, ke);
     ipm_count_launch();
-    if (ke >= nd) return;
+    if (ke >= nd) break;
     k_blu_l21<<<dim3((nd - ke + 127) / 128, S.N), 128, 0, st>>>(nd, S.nx, S.t0, S.nnzLU, S.dense_base, LU, rd, kb,
                                                                  ke);
     ipm_count_launch();
-  };
-  const auto trsm = [&](int kb, int ke, int c0, int c1) {  // U12 of columns [c0, c1)
-    k_blu_trsm<<<dim3((c1 - c0 + 7) / 8, S.N), 256, 0, st>>>(nd, S.nnzLU, S.dense_base, LU, kb, ke, c0, c1);
+    k_blu_trsm<<<dim3((nd - ke + 7) / 8, S.N), 256, 0, st>>>(nd, S.nnzLU, S.dense_base, LU, kb, ke);
     ipm_count_launch();
-  };
-  if (emu_lu) {
-    // Updates at FP64 grade on the tensor cores (exact 7-bit slices).  Their
-    // time is the epilogue (five FP64-unit operations per entry, ~19 cycles
-    // each per warp) however deep the product is, so the trailing block is
-    // updated once per EMU_LU_K columns: within such a block column, panels
-    // of PB and updates of its own columns only; then its rows of U, each PB
-    // of them by the ones before in one product; then the rest of the
-    // matrix.  1,776 states x 32 scenarios: 9.2e6 updated entries per
-    // scenario instead of 25e6, their products 26.4 -> 12.6 ms.
-    constexpr int OB = EMU_LU_K;
-    const auto update = [&](int kb, int ke, int a0, int a1, int b0, int b1) {
-      launch_emu_lu_update(*emu_lu, LU, S.nnzLU, S.dense_base, kb, ke, a0, a1 - a0, b0, b1 - b0, flags, st);
-    };
-    for (int ob = 0; ob < nd; ob += OB) {
-      const int oe = ob + OB < nd ? ob + OB : nd;
-      for (int kb = ob; kb < oe; kb += PB) {
-        const int ke = kb + PB < oe ? kb + PB : oe;
-        panel(kb, ke);
-        if (ke >= oe) break;
-        trsm(kb, ke, ke, oe);
-        update(kb, ke, ke, nd, ke, oe);
-      }
-      if (oe >= nd) break;
-      for (int kb = ob; kb < oe; kb += PB) {
-        if (kb > ob) update(ob, kb, kb, kb + PB, oe, nd);
-        trsm(kb, kb + PB, oe, nd);
-      }
-      update(ob, oe, oe, nd, oe, nd);
+    if (emu_lu) {
+      // FP64-grade on the tensor cores (exact 7-bit slices of L21, U12)
+      launch_emu_lu_update(*emu_lu, LU, S.nnzLU, S.dense_base, kb, ke, flags, st);
+    } else {
+      const int nt = (nd - ke + TT - 1) / TT;
+      k_blu_gemm<<<dim3(nt * nt, S.N), 256, gemm_smem(), st>>>(nd, S.nnzLU, S.dense_base, LU, kb, ke, nt);
+      ipm_count_launch();
     }
-    return;
-  }
-  for (int kb = 0; kb < nd; kb += PB) {
-    const int ke = kb + PB < nd ? kb + PB : nd;
-    panel(kb, ke);
-    if (ke >= nd) break;
-    trsm(kb, ke, ke, nd);
-    const int nt = (nd - ke + TT - 1) / TT;
-    k_blu_gemm<<<dim3(nt * nt, S.N), 256, gemm_smem(), st>>>(nd, S.nnzLU, S.dense_base, LU, kb, ke, nt);
-    ipm_count_launch();
   }
 }
 

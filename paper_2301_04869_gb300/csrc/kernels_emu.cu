@@ -275,11 +275,9 @@ __device__ __forceinline__ void tile_of_index(const int2 *tiles, int t, int &ti,
   tj = v.y;
 }
 
-constexpr int LU_K = EMU_LU_K;  // widest panel of the large-block LU's updates
-
 // Batched updates C -= A B (MODE 1, 2): the operands are the scenarios' A
 // rows and B columns stacked with fixed strides mpa, mpb (multiples of 128)
-// per scenario, the contraction is one group of 32 KPG (64 .. LU_K),
+// per scenario, the contraction is one 64-wide block (KPG = 2: one group),
 // and the epilogue subtracts the tile from the scenario's output instead of
 // writing a partial tile: MODE 1 a column-major FP64 block (the large-block
 // LU's trailing update), MODE 2 a row-major FP32 block (the multi-RHS
@@ -491,36 +489,35 @@ __global__ void __launch_bounds__(320, 1) k_emu_mma(const __grid_constant__ Maps
   }
 }
 
-// Slices of the operands of one update of the large-block LU, rows
-// [a0, a0 + na) and columns [b0, b0 + nb) by the columns [kb, ke) of L (side 0)
-// and the rows [kb, ke) of U (side 1), at most LU_K of them: stacked row
-// r = s Mp + m is row a0 + m of L or column b0 + m of U, a warp per row: its
+// Slices of the trailing update's operands for one panel [kb, ke) of the
+// large-block LU: stacked row r = s Mp + m (m < M = nd - ke) is row m of
+// L21 (side 0: L(ke + m, kb + k)) or column m of U12 (side 1:
+// U(kb + k, ke + m)), k = 0 .. ke - kb - 1 (at most 64); a warp per row: its
 // exponent e = ilogb(max |x|) + 2 and eight 7-bit digits per entry as in
-// k_emu_split, planes [NS][N Mp][LU_K] (K-major); rows past na (nb) up to the
-// next tile boundary are zero.
+// k_emu_split, planes [NS][N Mp][64] (K-major); rows m >= M are zero.
 __global__ void __launch_bounds__(256) k_emu_lu_split(const double *__restrict__ LU, long long nnzlu, int dense_base,
-                                                      int nd, int kb, int ke, int a0, int na, int b0, int nb, int Mp,
-                                                      int N, __nv_bfloat16 *pa, __nv_bfloat16 *pb, int *ea, int *eb) {
-  const int lane = threadIdx.x & 31, side = blockIdx.y, sc = blockIdx.z, K = ke - kb;
-  const int m = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), M = side == 0 ? na : nb;
-  if (m >= (M + BM - 1) / BM * BM) return;
-  const long long r = (long long)sc * Mp + m;
+                                                      int nd, int kb, int ke, int Mp, int N,
+                                                      __nv_bfloat16 *pa, __nv_bfloat16 *pb, int *ea, int *eb) {
+  const long long r = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31, side = blockIdx.y;
+  if (r >= (long long)N * Mp) return;
+  const int sc = (int)(r / Mp), m = (int)(r - (long long)sc * Mp), M = nd - ke, pbw = ke - kb;
   const double *A = LU + (size_t)sc * nnzlu + dense_base;
-  double x[LU_K / 32];
+  double x[2] = {0.0, 0.0};
+  if (m < M)
 #pragma unroll
-  for (int h = 0; h < LU_K / 32; ++h) {
-    const int k = lane + 32 * h;
-    x[h] = 0.0;
-    if (k < K && m < M) x[h] = side == 0 ? A[(size_t)(kb + k) * nd + a0 + m] : A[(size_t)(b0 + m) * nd + kb + k];
-  }
+    for (int h = 0; h < 2; ++h) {
+      const int k = lane + 32 * h;
+      if (k < pbw) x[h] = side == 0 ? A[(size_t)(kb + k) * nd + ke + m] : A[(size_t)(ke + m) * nd + kb + k];
+    }
   unsigned long long key = 0;
+  int E[2];
+  long long mt[2];
+  bool neg[2];
 #pragma unroll
-  for (int h = 0; h < LU_K / 32; ++h) {
-    int E;
-    long long mt;
-    bool neg;
-    dsplit_bits(x[h], E, mt, neg);
-    if (mt) key = max(key, ((unsigned long long)E << 53) | (unsigned long long)mt);
+  for (int h = 0; h < 2; ++h) {
+    dsplit_bits(x[h], E[h], mt[h], neg[h]);
+    if (mt[h]) key = max(key, ((unsigned long long)E[h] << 53) | (unsigned long long)mt[h]);
   }
   for (int o = 16; o > 0; o >>= 1) {
     const unsigned long long ok = __shfl_xor_sync(0xffffffffu, key, o);
@@ -529,15 +526,10 @@ __global__ void __launch_bounds__(256) k_emu_lu_split(const double *__restrict__
   const int e = key > 0 ? (int)(key >> 53) - 1023 + 2 : 0;
   __nv_bfloat16 *planes = side == 0 ? pa : pb;
   if (lane == 0) (side == 0 ? ea : eb)[r] = e;
-  const size_t plane = (size_t)N * Mp * LU_K;
+  const size_t plane = (size_t)N * Mp * 64;
 #pragma unroll
-  for (int h = 0; h < LU_K / 32; ++h) {
-    if (32 * h >= K) break;
-    int E;
-    long long mt;
-    bool neg;
-    dsplit_bits(x[h], E, mt, neg);
-    const long long X = mt ? fixed56(E, mt, neg, e) : 0;
+  for (int h = 0; h < 2; ++h) {
+    const long long X = mt[h] ? fixed56(E[h], mt[h], neg[h], e) : 0;
     const unsigned long long Y = (unsigned long long)(X + DIGIT_OFFSET);
     const uint32_t lo = (uint32_t)Y, hi = (uint32_t)(Y >> 32);
     uint32_t d[NS];
@@ -549,7 +541,7 @@ __global__ void __launch_bounds__(256) k_emu_lu_split(const double *__restrict__
     d[5] = digit_bf16((int)((lo >> 14) & 127) - 64);
     d[6] = digit_bf16((int)((lo >> 7) & 127) - 64);
     d[7] = digit_bf16((int)(lo & 127) - 64);
-    uint16_t *dst = reinterpret_cast<uint16_t *>(planes) + (size_t)r * LU_K + lane + 32 * h;
+    uint16_t *dst = reinterpret_cast<uint16_t *>(planes) + (size_t)r * 64 + lane + 32 * h;
 #pragma unroll
     for (int t = 0; t < NS; ++t) dst[t * plane] = (uint16_t)d[t];
   }
@@ -790,8 +782,8 @@ done:
 }
 
 // ---------------------------------------------------------------------------
-// The updates of the large-block LU at FP64 grade on the tensor cores (the
-// emulated product above with one row group of 64 to LU_K).
+// The trailing update A22 -= L21 U12 of the large-block LU at FP64 grade on
+// the tensor cores (the emulated product above with one 64-row group).
 bool emu_lu_plan(EmuLuPlan &P, int N, int nd, void *a_planes, void *b_planes, int *exp_a, int *exp_b) {
   P.N = N;
   P.nd = nd;
@@ -803,11 +795,11 @@ bool emu_lu_plan(EmuLuPlan &P, int N, int nd, void *a_planes, void *b_planes, in
   const long long rows = (long long)N * P.Mp;
   if (rows > 0x7fffffffLL) return false;
   emu::Maps m;
-  const size_t plane = (size_t)rows * emu::LU_K * 2;
+  const size_t plane = (size_t)rows * 64 * 2;
   for (int p = 0; p < emu::NS; ++p) {
-    if (!tc_make_kmajor_map_box(&m.a[p], (const char *)a_planes + p * plane, (int)rows, emu::LU_K, emu::BM, emu::BK))
+    if (!tc_make_kmajor_map_box(&m.a[p], (const char *)a_planes + p * plane, (int)rows, 64, emu::BM, emu::BK))
       return false;
-    if (!tc_make_kmajor_map_box(&m.b[p], (const char *)b_planes + p * plane, (int)rows, emu::LU_K, emu::BN, emu::BK))
+    if (!tc_make_kmajor_map_box(&m.b[p], (const char *)b_planes + p * plane, (int)rows, 64, emu::BN, emu::BK))
       return false;
   }
   static_assert(sizeof(emu::Maps) <= sizeof(P.maps), "map storage");
@@ -817,38 +809,29 @@ bool emu_lu_plan(EmuLuPlan &P, int N, int nd, void *a_planes, void *b_planes, in
 
 size_t emu_lu_planes_bytes(int N, int nd) {
   const long long Mp = (nd + emu::BM - 1) / emu::BM * emu::BM;
-  return (size_t)emu::NS * N * Mp * emu::LU_K * 2;
+  return (size_t)emu::NS * N * Mp * 64 * 2;
 }
 
-template <int KPG>
-static void emu_lu_mma(const EmuLuPlan &P, const emu::TileOut &lo, int *flags, cudaStream_t st) {
-  auto kern = emu::k_emu_mma<KPG, 1>;
+void launch_emu_lu_update(const EmuLuPlan &P, double *LU, long long nnzlu, int dense_base, int kb, int ke, int *flags,
+                          cudaStream_t st) {
+  const int M = P.nd - ke;
+  if (M <= 0) return;
+  const long long rows = (long long)P.N * P.Mp;
+  emu::k_emu_lu_split<<<dim3((unsigned)((rows * 32 + 255) / 256), 2), 256, 0, st>>>(
+      LU, nnzlu, dense_base, P.nd, kb, ke, P.Mp, P.N, (__nv_bfloat16 *)P.a_planes, (__nv_bfloat16 *)P.b_planes,
+      P.exp_a, P.exp_b);
+  ipm_count_launch();
+  auto kern = emu::k_emu_mma<2, 1>;
   static const bool attr =
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, emu::SMEM_BYTES) == cudaSuccess;
   (void)attr;
   emu::Maps m;
   memcpy(&m, P.maps, sizeof(m));
+  // C = the dense block, column-major: (ke + m, ke + n) at dense_base + (ke + n) nd + ke + m
+  emu::TileOut lo{LU + dense_base, nnzlu, 1, P.nd, ke, ke, M, M, P.Mp, P.Mp,
+                  (M + emu::BM - 1) / emu::BM, (M + emu::BN - 1) / emu::BN};
   const long long grid = (long long)P.N * lo.na * lo.nb;
-  kern<<<dim3((unsigned)grid, 1), 320, emu::SMEM_BYTES, st>>>(m, nullptr, P.N * P.Mp, KPG, KPG, P.exp_a, P.exp_b,
-                                                             nullptr, flags, lo);
+  kern<<<dim3((unsigned)grid, 1), 320, emu::SMEM_BYTES, st>>>(m, nullptr, (int)rows, 2, 2, P.exp_a, P.exp_b, nullptr,
+                                                             flags, lo);
   ipm_count_launch();
-}
-
-void launch_emu_lu_update(const EmuLuPlan &P, double *LU, long long nnzlu, int dense_base, int kb, int ke, int a0,
-                          int na, int b0, int nb, int *flags, cudaStream_t st) {
-  if (na <= 0 || nb <= 0) return;
-  const int mt = ((na > nb ? na : nb) + emu::BM - 1) / emu::BM * emu::BM;
-  emu::k_emu_lu_split<<<dim3(mt / 8, 2, P.N), 256, 0, st>>>(
-      LU, nnzlu, dense_base, P.nd, kb, ke, a0, na, b0, nb, P.Mp, P.N, (__nv_bfloat16 *)P.a_planes,
-      (__nv_bfloat16 *)P.b_planes, P.exp_a, P.exp_b);
-  ipm_count_launch();
-  // C = the dense block, column-major: (a0 + m, b0 + n) at dense_base + (b0 + n) nd + a0 + m
-  const emu::TileOut lo{LU + dense_base, nnzlu, 1, P.nd, a0, b0, na, nb, P.Mp, P.Mp,
-                        (na + emu::BM - 1) / emu::BM, (nb + emu::BN - 1) / emu::BN};
-  switch ((ke - kb + 63) / 64) {  // (a short last panel is padded with zeros)
-    case 1: emu_lu_mma<2>(P, lo, flags, st); break;
-    case 2: emu_lu_mma<4>(P, lo, flags, st); break;
-    case 3: emu_lu_mma<6>(P, lo, flags, st); break;
-    default: emu_lu_mma<8>(P, lo, flags, st);
-  }
 }
