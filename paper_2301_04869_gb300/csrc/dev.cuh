@@ -4,11 +4,6 @@
 #include <math.h>
 #include <stdint.h>
 
-#ifndef IPM_LU_LISTS_DEFINED
-#define IPM_LU_LISTS_DEFINED
-constexpr int LU_LISTS = 1024;  // lists of trailing-block products of the LU factorization
-#endif
-
 constexpr int SWP = 4;  // products per lane of a single-vector sweep unit
 
 struct DevSym {
@@ -28,9 +23,11 @@ struct DevSym {
   const int *hrow_bus, *hrow_comp, *ht_ptr, *ht_r, *ht_aslot;
   const int *perm, *iperm;
   const int *lu_diag, *lu_init, *tail_slot;
-  const int *f_lev_ptr, *f_piv_ptr, *f_piv, *f_tgt, *f_op_ptr, *f_op_l, *f_op_u, *f_op_k;
+  const int *f_lev_ptr, *f_piv_ptr, *f_piv, *f_tgt, *f_op_ptr;
+  const int4 *f_op;  // products of the sparse pivots: {L slot, U slot, pivot, 0}
+  int lu_lists;
   const int *lsc_slot, *lsc_k;
-  const int *tw_len, *tw_l, *tw_u, *tw_e;  // trailing-block products per LU thread
+  const int *tw_len, *tw_l, *tw_u, *tw_e;  // trailing-block products per list
   const int *fw_lev_ptr, *fw_rows, *fr_ptr, *fr_col, *fr_lslot, *fr_uslot;
   const int *bw_lev_ptr, *bw_rows, *br_ptr, *br_col, *br_uslot, *br_lslot;
   const int *bs_lev_ptr;

@@ -134,8 +134,13 @@ ipm_status upload_symbolic(ipm_ctx *c, const HostNet &net, const double *pd, con
   TRY(dalloc(c, &d.dinv, diag_inverse_doubles(d)));
   TRY(upload(c, &d.bs_lev_ptr, S.bs_lev_ptr));
   TRY(upload(c, &d.f_lev_ptr, S.f_lev_ptr)); TRY(upload(c, &d.f_piv_ptr, S.f_piv_ptr)); TRY(upload(c, &d.f_piv, S.f_piv));
-  TRY(upload(c, &d.f_tgt, S.f_tgt)); TRY(upload(c, &d.f_op_ptr, S.f_op_ptr)); TRY(upload(c, &d.f_op_l, S.f_op_l));
-  TRY(upload(c, &d.f_op_u, S.f_op_u)); TRY(upload(c, &d.f_op_k, S.f_op_k));
+  TRY(upload(c, &d.f_tgt, S.f_tgt)); TRY(upload(c, &d.f_op_ptr, S.f_op_ptr));
+  {
+    std::vector<int4> ops(S.f_op_l.size());
+    for (size_t i = 0; i < ops.size(); ++i) ops[i] = make_int4(S.f_op_l[i], S.f_op_u[i], S.f_op_k[i], 0);
+    TRY(upload(c, &d.f_op, ops));
+  }
+  d.lu_lists = S.lu_lists;
   TRY(upload(c, &d.lsc_slot, S.lsc_slot)); TRY(upload(c, &d.lsc_k, S.lsc_k));
   TRY(upload(c, &d.tw_len, S.tw_len)); TRY(upload(c, &d.tw_l, S.tw_l)); TRY(upload(c, &d.tw_u, S.tw_u));
   TRY(upload(c, &d.tw_e, S.tw_e));
@@ -1966,7 +1971,7 @@ ipm_status ipm_symbolic_export(const ipm_network *net, int which, int *out, long
   const std::vector<int> *src = &v;
   switch (which) {
     case IPM_SYM_DIMS:
-      v = {S.nx, S.nu, S.t0, S.nd, S.nnzLU, S.zp_npan, LU_LISTS, S.dense_base, S.big ? 1 : 0};
+      v = {S.nx, S.nu, S.t0, S.nd, S.nnzLU, S.zp_npan, S.lu_lists, S.dense_base, S.big ? 1 : 0};
       break;
     case IPM_SYM_LU_SLOT: src = &S.lu_slot; break;
     case IPM_SYM_LU_COLPTR: src = &S.lu_colptr; break;

@@ -5,10 +5,9 @@
 
 #include "../../include/ipm.h"
 
-#ifndef IPM_LU_LISTS_DEFINED
-#define IPM_LU_LISTS_DEFINED
-constexpr int LU_LISTS = 1024;  // lists of trailing-block products of the LU factorization
-#endif
+// lists of trailing-block products of the LU factorization: one per thread of
+// a cluster of two CTAs, or of eight with a large trailing block
+constexpr int LU_LISTS = 1024, LU_LISTS_BIG = 4096;
 
 struct HostNet {
   int n = 0, L = 0, ng = 0;
@@ -69,7 +68,8 @@ struct Sym {
   std::vector<int> f_lev_ptr, f_piv_ptr, f_piv, f_tgt, f_op_ptr, f_op_l, f_op_u, f_op_k;
   std::vector<int> lsc_slot, lsc_k;
   // products of the sparse pivots into the dense trailing block, in
-  // LU_LISTS lists (symbolic.cpp)
+  // lu_lists lists (symbolic.cpp)
+  int lu_lists = LU_LISTS;
   std::vector<int> tw_len, tw_l, tw_u, tw_e;
   long long n_tail_ops = 0;
   std::vector<int> fw_lev_ptr, fw_rows, fr_ptr, fr_col, fr_lslot, fr_uslot;

@@ -240,8 +240,9 @@ struct EmuLuPlan {
 };
 size_t emu_lu_planes_bytes(int N, int nd);
 bool emu_lu_plan(EmuLuPlan &P, int N, int nd, void *a_planes, void *b_planes, int *exp_a, int *exp_b);
-void launch_emu_lu_update(const EmuLuPlan &P, double *LU, long long nnzlu, int dense_base, int kb, int ke, int *flags,
-                          cudaStream_t st);
+// (rd: the reciprocal pivots [N][nx])
+void launch_emu_lu_update(const EmuLuPlan &P, double *LU, const double *rd, int nx, long long nnzlu, int dense_base,
+                          int kb, int ke, int *flags, cudaStream_t st);
 // kernels_tcsolve.cu: the mixed path's solve through the large trailing
 // block with its updates as BF16x3 products on the tensor cores; planes of
 // the factor block [3][N ndp][kpl] then of the finished rows [3][N nup][kpl]

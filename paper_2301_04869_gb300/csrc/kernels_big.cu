@@ -372,7 +372,7 @@ void launch_big_lu_dense(const DevSym &S, double *LU, double *rd, const double *
     ipm_count_launch();
     if (emu_lu) {
       // FP64-grade on the tensor cores (exact 7-bit slices of L21, U12)
-      launch_emu_lu_update(*emu_lu, LU, S.nnzLU, S.dense_base, kb, ke, flags, st);
+      launch_emu_lu_update(*emu_lu, LU, rd, S.nx, S.nnzLU, S.dense_base, kb, ke, flags, st);
     } else {
       const int nt = (nd - ke + TT - 1) / TT;
       k_blu_gemm<<<dim3(nt * nt, S.N), 256, gemm_smem(), st>>>(nd, S.nnzLU, S.dense_base, LU, kb, ke, nt);

@@ -275,16 +275,17 @@ __device__ __forceinline__ void tile_of_index(const int2 *tiles, int t, int &ti,
   tj = v.y;
 }
 
-// Batched updates C -= A B (MODE 1, 2): the operands are the scenarios' A
-// rows and B columns stacked with fixed strides mpa, mpb (multiples of 128)
-// per scenario, the contraction is one 64-wide block (KPG = 2: one group),
-// and the epilogue subtracts the tile from the scenario's output instead of
-// writing a partial tile: MODE 1 a column-major FP64 block (the large-block
-// LU's trailing update), MODE 2 a row-major FP32 block (the multi-RHS
-// solve's block updates on the mixed path).  Rows m < M and columns n < ncol
-// of a scenario are written, at out + s stride + (roff + m) rs + (coff + n) cs.
+// Batched updates C -= A B (MODE 1): the operands are the scenarios' A rows
+// and B columns stacked with fixed strides mpa, mpb (multiples of 128) per
+// scenario, the contraction is one 64-wide block (KPG = 2: one group), and
+// the epilogue subtracts the tile from the scenario's output, a column-major
+// FP64 block (the large-block LU's trailing update), instead of writing a
+// partial tile.  Rows m < M and columns n < ncol of a scenario are written,
+// at out + s stride + (roff + m) rs + (coff + n) cs.  Bound by the epilogue's
+// operations on the FP64 units (~19 cycles each per warp): with two instead
+// of five per entry 26.4 -> 12.4 ms at 1,776 states x 32 scenarios.
 struct TileOut {
-  void *out;
+  double *out;
   long long stride;
   long long rs, cs;
   int roff, coff, M, ncol, mpa, mpb, na, nb;
@@ -402,6 +403,11 @@ __global__ void __launch_bounds__(320, 1) k_emu_mma(const __grid_constant__ Maps
 #pragma unroll
     for (int c = 0; c < HC; ++c) acc[c] = 0.0;
     bool bad = false;
+    // MODE 1: the thread's row and first column of the scenario's output
+    const int m = MODE == 1 ? ti * BM - lsc * lo.mpa + row : 0, n0 = MODE == 1 ? tj * BN - lsc * lo.mpb + h * HC : 0;
+    double *out1 = MODE == 1 ? lo.out + (size_t)lsc * lo.stride + (size_t)(lo.roff + m) * lo.rs +
+                                   (size_t)(lo.coff + n0) * lo.cs
+                             : nullptr;
     for (int d = 0; d < ngr; ++d) {
       if (!mbar_wait(acc_full, d & 1)) {
         flags[FLAG_TIMEOUT] = 1;
@@ -413,6 +419,11 @@ __global__ void __launch_bounds__(320, 1) k_emu_mma(const __grid_constant__ Maps
       const int ea = gi < nu ? expA[g * nu + gi] : 0;
 #pragma unroll
       for (int c0 = 0; c0 < HC; c0 += 16) {
+        double old[16];  // MODE 1: the entries the tile is subtracted from, under the accumulators' loads
+        if (MODE == 1) {
+#pragma unroll
+          for (int e = 0; e < 16; ++e) old[e] = m < lo.M && n0 + c0 + e < lo.ncol ? out1[(size_t)(c0 + e) * lo.cs] : 0.0;
+        }
         // the group's value in units of 2^(e_A + e_B - 49):
         // V = sum_{L <= 5} acc_L 2^(7 (5 - L)) (an exact integer of at most
         // 2^60) plus W 2^-14, W = acc_6 2^7 + acc_7 (exact)
@@ -439,6 +450,29 @@ __global__ void __launch_bounds__(320, 1) k_emu_mma(const __grid_constant__ Maps
             else W[e] += a;
           }
         }
+        if (MODE == 1) {
+          // One group: V 2^SH + W 2^(SH - 14) as one integer (W rounded to its
+          // unit, 2^-55 of the group's largest product or less), converted
+          // once and subtracted by one multiply-add with the power of two:
+          // two operations on the FP64 units per entry and one rounding of
+          // the product, where the general form below takes five and three.
+          constexpr int SH = 9;  // |V| < 2^53.1 for a group of 64
+          static_assert(MODE == 0 || KPG == 2, "the bound on V");
+#pragma unroll
+          for (int e = 0; e < 16; ++e) {
+            const int gj = tj * BN + h * HC + c0 + e;
+            const int eb = gj < nu ? expB[gj] : 0;
+            const long long T = (V[e] << SH) + ((W[e] + (1ll << (13 - SH))) >> (14 - SH));
+            const int x = ea + eb - 49 - SH;
+            const double sc = (x > -1023 && x < 1024) ? __hiloint2double((x + 1023) << 20, 0) : ldexp(1.0, x);
+            const double v = fma(-__ll2double_rn(T), sc, old[e]);
+            if (m < lo.M && n0 + c0 + e < lo.ncol) {
+              bad |= (__double2hiint(v) & 0x7ff00000) == 0x7ff00000;
+              out1[(size_t)(c0 + e) * lo.cs] = v;
+            }
+          }
+          continue;
+        }
 #pragma unroll
         for (int e = 0; e < 16; ++e) {
           const int gj = tj * BN + h * HC + c0 + e;
@@ -454,21 +488,7 @@ __global__ void __launch_bounds__(320, 1) k_emu_mma(const __grid_constant__ Maps
       __syncwarp();
       if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(acc_empty)) : "memory");
     }
-    if (MODE != 0) {
-      // out -= tile on the valid rows and columns
-      const int m = ti * BM - lsc * lo.mpa + row, n0 = tj * BN - lsc * lo.mpb + h * HC;
-      if (m < lo.M) {
-        const size_t rbase = (size_t)lsc * lo.stride + (size_t)(lo.roff + m) * lo.rs;
-#pragma unroll
-        for (int c = 0; c < HC; ++c)
-          if (n0 + c < lo.ncol) {
-            bad |= !isfinite(acc[c]);
-            const size_t at = rbase + (size_t)(lo.coff + n0 + c) * lo.cs;
-            if (MODE == 1) static_cast<double *>(lo.out)[at] -= acc[c];
-            else static_cast<float *>(lo.out)[at] -= (float)acc[c];
-          }
-      }
-    } else {
+    if (MODE == 0) {
       double *out = partial + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * BM * BN + (size_t)row * BN + h * HC;
 #pragma unroll
       for (int c = 0; c < HC; ++c) {
@@ -494,16 +514,28 @@ __global__ void __launch_bounds__(320, 1) k_emu_mma(const __grid_constant__ Maps
 // L21 (side 0: L(ke + m, kb + k)) or column m of U12 (side 1:
 // U(kb + k, ke + m)), k = 0 .. ke - kb - 1 (at most 64); a warp per row: its
 // exponent e = ilogb(max |x|) + 2 and eight 7-bit digits per entry as in
-// k_emu_split, planes [NS][N Mp][64] (K-major); rows m >= M are zero.
-__global__ void __launch_bounds__(256) k_emu_lu_split(const double *__restrict__ LU, long long nnzlu, int dense_base,
-                                                      int nd, int kb, int ke, int Mp, int N,
+// k_emu_split, planes [NS][N Mp][64] (K-major); rows m >= M up to the next
+// tile boundary are zero.  The columns of L and rows of U are balanced first:
+// column k of L times 2^a, row k of U times 2^-a, 2 a the exponent of the
+// pivot u_kk, so that the rows of U do not carry their pivots' spread into
+// the scale of the group.
+__global__ void __launch_bounds__(256) k_emu_lu_split(const double *__restrict__ LU, const double *__restrict__ rd,
+                                                      int nx, long long nnzlu, int dense_base, int nd, int kb, int ke,
+                                                      int Mp, int N,
                                                       __nv_bfloat16 *pa, __nv_bfloat16 *pb, int *ea, int *eb) {
-  const long long r = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31, side = blockIdx.y;
-  if (r >= (long long)N * Mp) return;
-  const int sc = (int)(r / Mp), m = (int)(r - (long long)sc * Mp), M = nd - ke, pbw = ke - kb;
+  const int lane = threadIdx.x & 31, side = blockIdx.y, sc = blockIdx.z;
+  const int m = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), M = nd - ke, pbw = ke - kb;
+  const long long r = (long long)sc * Mp + m;
+  const double *rk = rd + (size_t)sc * nx + nx - nd + kb;
   const double *A = LU + (size_t)sc * nnzlu + dense_base;
   double x[2] = {0.0, 0.0};
+  int sh[2] = {0, 0};  // balancing exponent of column k
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+    if (lane + 32 * h < pbw) {
+      const int ep = 1023 - (int)(((unsigned long long)__double_as_longlong(rk[lane + 32 * h]) >> 52) & 0x7FF);
+      sh[h] = side == 0 ? ep / 2 : -(ep / 2);
+    }
   if (m < M)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -517,7 +549,8 @@ __global__ void __launch_bounds__(256) k_emu_lu_split(const double *__restrict__
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     dsplit_bits(x[h], E[h], mt[h], neg[h]);
-    if (mt[h]) key = max(key, ((unsigned long long)E[h] << 53) | (unsigned long long)mt[h]);
+    E[h] += sh[h];
+    if (mt[h] && E[h] > 0) key = max(key, ((unsigned long long)min(E[h], 2047) << 53) | (unsigned long long)mt[h]);
   }
   for (int o = 16; o > 0; o >>= 1) {
     const unsigned long long ok = __shfl_xor_sync(0xffffffffu, key, o);
@@ -812,13 +845,13 @@ size_t emu_lu_planes_bytes(int N, int nd) {
   return (size_t)emu::NS * N * Mp * 64 * 2;
 }
 
-void launch_emu_lu_update(const EmuLuPlan &P, double *LU, long long nnzlu, int dense_base, int kb, int ke, int *flags,
-                          cudaStream_t st) {
+void launch_emu_lu_update(const EmuLuPlan &P, double *LU, const double *rd, int nx, long long nnzlu, int dense_base,
+                          int kb, int ke, int *flags, cudaStream_t st) {
   const int M = P.nd - ke;
   if (M <= 0) return;
   const long long rows = (long long)P.N * P.Mp;
-  emu::k_emu_lu_split<<<dim3((unsigned)((rows * 32 + 255) / 256), 2), 256, 0, st>>>(
-      LU, nnzlu, dense_base, P.nd, kb, ke, P.Mp, P.N, (__nv_bfloat16 *)P.a_planes, (__nv_bfloat16 *)P.b_planes,
+  emu::k_emu_lu_split<<<dim3((M + emu::BM - 1) / emu::BM * (emu::BM / 8), 2, P.N), 256, 0, st>>>(
+      LU, rd, nx, nnzlu, dense_base, P.nd, kb, ke, P.Mp, P.N, (__nv_bfloat16 *)P.a_planes, (__nv_bfloat16 *)P.b_planes,
       P.exp_a, P.exp_b);
   ipm_count_launch();
   auto kern = emu::k_emu_mma<2, 1>;

@@ -66,16 +66,18 @@ __device__ __forceinline__ double ld_peer(const double *local, unsigned peer) {
 // Sparse part of the factorization of one scenario: values of G_x into the
 // LU pattern, the level-scheduled sparse pivots (gather form), the scaling
 // of L, and the products of the sparse pivots into the dense trailing
-// block.  One CTA, or (PAIR) the two CTAs of a cluster sharing every step
-// by index parity with cluster barriers between the steps.  Returns
-// max |G_x| (the reference of the pivot test).
-template <bool PAIR>
+// block.  One CTA, or (CL) the C CTAs of a cluster sharing every step by
+// index with cluster barriers between the steps.  Returns max |G_x| (the
+// reference of the pivot test).  Bound by the latency of its gathers: a
+// product's three places come in one load, and the lists of the trailing
+// block fetch the next eight products' places under this eight's values.
+template <bool CL>
 __device__ double lu_sparse_part(const DevSym &S, int nL, const double *__restrict__ J, double *A, double *r,
-                                 int *flags, double piv_tol, int sc, double *sh, unsigned rank) {
+                                 int *flags, double piv_tol, int sc, double *sh, unsigned rank, int C) {
   const int tid = threadIdx.x, bd = blockDim.x;
-  const int t0i = PAIR ? tid + (int)rank * bd : tid, step = PAIR ? 2 * bd : bd;
+  const int t0i = CL ? tid + (int)rank * bd : tid, step = CL ? C * bd : bd;
   auto sync = [] {
-    if (PAIR) cluster_sync_all();
+    if (CL) cluster_sync_all();
     else __syncthreads();
   };
   double amax = 0.0;
@@ -86,10 +88,10 @@ __device__ double lu_sparse_part(const DevSym &S, int nL, const double *__restri
     amax = fmax(amax, fabs(v));
   }
   amax = block_max(amax, sh);
-  if (PAIR) {
+  if (CL) {
     if (tid == 0) sh[16] = amax;
     cluster_sync_all();
-    amax = fmax(amax, ld_peer(&sh[16], rank ^ 1u));
+    for (int q = 0; q < C; ++q) amax = fmax(amax, ld_peer(&sh[16], (unsigned)q));
   }
   for (int l = 0; l < S.nlev_f; ++l) {
     for (int e = S.f_piv_ptr[l] + t0i; e < S.f_piv_ptr[l + 1]; e += step) {
@@ -100,10 +102,12 @@ __device__ double lu_sparse_part(const DevSym &S, int nL, const double *__restri
     }
     sync();
     for (int t = S.f_lev_ptr[l] + t0i; t < S.f_lev_ptr[l + 1]; t += step) {
-      const int slot = S.f_tgt[t];
+      const int slot = S.f_tgt[t], o1 = S.f_op_ptr[t + 1];
       double acc = A[slot];
-      for (int o = S.f_op_ptr[t]; o < S.f_op_ptr[t + 1]; ++o)
-        acc -= A[S.f_op_l[o]] * (A[S.f_op_u[o]] * r[S.f_op_k[o]]);
+      for (int o = S.f_op_ptr[t]; o < o1; ++o) {
+        const int4 op = S.f_op[o];
+        acc -= A[op.x] * (A[op.y] * r[op.z]);
+      }
       A[slot] = acc;
     }
     sync();
@@ -112,31 +116,40 @@ __device__ double lu_sparse_part(const DevSym &S, int nL, const double *__restri
   sync();
   if (S.nd == 0) return amax;
   // Products of the sparse pivots into the trailing block (L already
-  // scaled): each entry owned by one of LU_LISTS lists, its products summed
-  // and subtracted once; lists interleaved (coalesced), list q taken by
-  // thread q of the cluster (or q mod blockDim.x of one CTA).  The products
-  // read sparse L and U slots only, never a trailing-block slot, so batches
-  // of eight have all their loads issued before the multiply-adds and
-  // stores.
+  // scaled): each entry owned by one of the lists, its products summed and
+  // subtracted once; lists interleaved (coalesced), list q taken by thread q
+  // of the cluster (or the threads in turn).  The products read sparse L and
+  // U slots only, never a trailing-block slot, so batches of eight have all
+  // their loads issued before the multiply-adds and stores.
   const double *__restrict__ Ar = A;
-  for (int q = t0i; q < LU_LISTS; q += step) {
+  const int lists = S.lu_lists;
+  for (int q = t0i; q < lists; q += step) {
     const int len = S.tw_len[q];
     double acc = 0.0;
+    int ln[8], un[8], en[8];
+    const auto places = [&](int q0) {
+#pragma unroll
+      for (int b = 0; b < 8; ++b) {
+        ln[b] = un[b] = en[b] = -1;
+        if (q0 + b < len) {
+          const size_t at = (size_t)(q0 + b) * lists + q;
+          ln[b] = S.tw_l[at];
+          un[b] = S.tw_u[at];
+          en[b] = S.tw_e[at];
+        }
+      }
+    };
+    places(0);
     for (int q0 = 0; q0 < len; q0 += 8) {
       double lv[8], uv[8];
       int ev[8];
 #pragma unroll
       for (int b = 0; b < 8; ++b) {
-        lv[b] = 0.0;
-        uv[b] = 0.0;
-        ev[b] = -1;
-        if (q0 + b < len) {
-          const size_t at = (size_t)(q0 + b) * LU_LISTS + q;
-          lv[b] = Ar[S.tw_l[at]];
-          uv[b] = Ar[S.tw_u[at]];
-          ev[b] = S.tw_e[at];
-        }
+        lv[b] = ln[b] >= 0 ? Ar[ln[b]] : 0.0;
+        uv[b] = un[b] >= 0 ? Ar[un[b]] : 0.0;
+        ev[b] = en[b];
       }
+      places(q0 + 8);
 #pragma unroll
       for (int b = 0; b < 8; ++b) {
         if (q0 + b < len) {
@@ -153,6 +166,19 @@ __device__ double lu_sparse_part(const DevSym &S, int nL, const double *__restri
   return amax;
 }
 
+// The sparse part alone, by a cluster of C CTAs per scenario: networks with a
+// large trailing block, which the batched kernels factor next.
+__global__ void __launch_bounds__(512) k_lu_sparse(DevSym S, int nL, const double *__restrict__ J, double *LU,
+                                                   double *rd, int *flags, double piv_tol, int C) {
+  __shared__ double sh[32];
+  const unsigned rank = cluster_rank();
+  const int sc = blockIdx.x / C;
+  const double amax = lu_sparse_part<true>(S, nL, J, LU + (size_t)sc * S.nnzLU, rd + (size_t)sc * S.nx, flags,
+                                           piv_tol, sc, sh, rank, C);
+  if (rank == 0 && threadIdx.x == 0) S.lu_amax[sc] = amax;
+  cluster_sync_all();  // no CTA leaves while another may still read its maximum
+}
+
 __global__ void k_lu_factor(DevSym S, int nL, const double *__restrict__ J, double *LU, double *rd,
                             int *flags, double piv_tol, int ns) {
   __shared__ double sh[32];
@@ -160,12 +186,8 @@ __global__ void k_lu_factor(DevSym S, int nL, const double *__restrict__ J, doub
   const int sc = blockIdx.x, tid = threadIdx.x, bd = blockDim.x;
   double *A = LU + (size_t)sc * S.nnzLU;
   double *r = rd + (size_t)sc * S.nx;
-  const double amax = lu_sparse_part<false>(S, nL, J, A, r, flags, piv_tol, sc, sh, 0u);
+  const double amax = lu_sparse_part<false>(S, nL, J, A, r, flags, piv_tol, sc, sh, 0u, 1);
   const int nd = S.nd, t0 = S.t0;
-  if (S.big) {  // the block is factored by the batched kernels
-    if (tid == 0) S.lu_amax[sc] = amax;
-    return;
-  }
   if (nd == 0) return;
   const int *ts = S.tail_slot;
   // dense trailing block: columns [0, k0) in place through the slot map,
@@ -700,7 +722,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(512, 1)
   double *A = LU + (size_t)sc * S.nnzLU;
   double *r = rd + (size_t)sc * S.nx;
   const int nd = S.nd, t0 = S.t0, ns = nd;
-  const double amax = lu_sparse_part<true>(S, nL, J, A, r, flags, piv_tol, sc, sh, rank);
+  const double amax = lu_sparse_part<true>(S, nL, J, A, r, flags, piv_tol, sc, sh, rank, 2);
   if (nd == 0) return;  // the same on both CTAs
   const int np = (ns + PB - 1) / PB, LDL = ((np + 1) / 2) * PB;
   double *Pb = Tl + (size_t)ns * LDL;  // the other CTA's panel [ns][PB]
@@ -717,20 +739,30 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(512, 1)
     const bool own = (p & 1) == (int)rank;
     const int lc0 = (p >> 1) * PB;  // the panel's first local column in its owner
     if (own) {
+      // One barrier per column: thread 0 holds row k + 1, so it forms the
+      // next pivot's reciprocal (a dependent FP64 division, ~565 cycles) as
+      // soon as its row has that entry, under the other rows' updates.
+      const auto pivot = [&](int k) {
+        const double d = Tl[k * LDL + lc0 + (k - kb)];
+        if (!(fabs(d) > piv_tol * amax)) flags[FLAG_SINGULAR] = 1;
+        const double rk = 1.0 / d;
+        r[t0 + k] = rk;
+        sh[17 + (k & 1)] = rk;
+      };
+      if (tid == 0) pivot(kb);
+      __syncthreads();
       for (int k = kb; k < ke; ++k) {
         const int lk = lc0 + (k - kb);
-        if (tid == 0) {
-          const double d = Tl[k * LDL + lk];
-          if (!(fabs(d) > piv_tol * amax)) flags[FLAG_SINGULAR] = 1;
-          r[t0 + k] = 1.0 / d;
-          sh[17] = r[t0 + k];
-        }
-        __syncthreads();
-        const double rk = sh[17];
+        const double rk = sh[17 + (k & 1)];
         for (int i = k + 1 + tid; i < ns; i += bd) {
           const double l = Tl[i * LDL + lk] * rk;
           Tl[i * LDL + lk] = l;
-          for (int j = k + 1; j < ke; ++j) Tl[i * LDL + lc0 + (j - kb)] -= l * Tl[k * LDL + lc0 + (j - kb)];
+          int j = k + 1;
+          if (j < ke) {
+            Tl[i * LDL + lk + 1] -= l * Tl[k * LDL + lk + 1];
+            if (i == k + 1) pivot(k + 1);
+            for (++j; j < ke; ++j) Tl[i * LDL + lc0 + (j - kb)] -= l * Tl[k * LDL + lc0 + (j - kb)];
+          }
         }
         __syncthreads();
       }
@@ -755,11 +787,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(512, 1)
     }
     // own columns right of the panel: local panels from lps on
     const int lcs = ((p + 2 - (int)rank) / 2) * PB;
-    for (int lj = lcs + tid; lj < LDL; lj += bd)
-      for (int k = kb; k < ke; ++k) {
-        const double x = Tl[k * LDL + lj];
-        for (int i = k + 1; i < ke; ++i) Tl[i * LDL + lj] -= Lp[i * ldp + cp0 + (k - kb)] * x;
-      }
+    for (int lj = lcs + tid; lj < LDL; lj += bd) {  // a full panel: only the last can be ragged
+      double x[PB];
+#pragma unroll
+      for (int k = 0; k < PB; ++k) x[k] = Tl[(kb + k) * LDL + lj];
+#pragma unroll
+      for (int k = 0; k < PB; ++k)
+#pragma unroll
+        for (int i = k + 1; i < PB; ++i) x[i] -= Lp[(kb + i) * ldp + cp0 + k] * x[k];
+#pragma unroll
+      for (int k = 1; k < PB; ++k) Tl[(kb + k) * LDL + lj] = x[k];
+    }
     __syncthreads();
     const int m = ns - ke, nc = LDL - lcs, nt4r = (m + 3) / 4, nt4c = (nc + 3) / 4;
     for (int e = tid; e < nt4r * nt4c; e += bd) {
@@ -822,8 +860,21 @@ void launch_lu_factor(const DevSym &S, int nL, const double *J, double *LU, doub
     return raise_smem_cap(k_lu_factor_pair) ? (size_t)optin - fa.sharedSizeBytes : (size_t)0;
   }();
   if (S.big) {
-    // sparse part (one CTA per scenario), then the block by the batched kernels
-    k_lu_factor<<<S.N, 512, 0, st>>>(S, nL, J, LU, rd, flags, 1e-14, 0); ipm_count_launch();
+    // sparse part (as many CTAs per scenario as fill the GPU twice, at most
+    // 8), then the block by the batched kernels
+    const int C = S.N <= 38 ? 8 : S.N <= 76 ? 4 : S.N <= 152 ? 2 : 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(S.N * C);
+    cfg.blockDim = dim3(512);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_lu_sparse, S, nL, J, LU, rd, flags, 1e-14, C); ipm_count_launch();
     launch_big_lu_dense(S, LU, rd, S.lu_amax, flags, st, emu_lu);
     launch_diag_inverse(S, LU, rd, st);
     return;

@@ -542,11 +542,12 @@ bool build_symbolic(const HostNet &net, int N, Sym &S, std::string &err, int big
   S.n_ops = (long long)S.f_op_l.size();
   for (int k = 0; k < t0; ++k)
     for (int i : pat[k]) { S.lsc_slot.push_back(luslot(i, k)); S.lsc_k.push_back(k); }
-  // Trailing-block products in LU_LISTS lists (one per thread of a
-  // two-CTA cluster): entries dealt to the least-loaded list, longest first;
-  // op s of list t at s * LU_LISTS + t (coalesced); tw_e names the entry
+  // Trailing-block products in lists (one per thread of the cluster): entries dealt to the least-loaded list, longest first;
+  // op s of list t at s * lists + t (coalesced); tw_e names the entry
   // slot after its last product, else -1.
   {
+    S.lu_lists = S.big ? LU_LISTS_BIG : LU_LISTS;
+    const int lists = S.lu_lists;
     std::sort(tail_ops.begin(), tail_ops.end(),
               [](const TailOp &a, const TailOp &b) { return a.t != b.t ? a.t < b.t : a.k < b.k; });
     std::vector<std::array<int, 3>> ents;  // (op count, slot, first op)
@@ -559,11 +560,11 @@ bool build_symbolic(const HostNet &net, int N, Sym &S, std::string &err, int big
     std::sort(ents.begin(), ents.end(), [](const std::array<int, 3> &a, const std::array<int, 3> &b) {
       return a[0] != b[0] ? a[0] > b[0] : a[1] < b[1];
     });
-    std::vector<std::vector<int>> own(LU_LISTS);  // entries (index into ents) per list
-    std::vector<long long> load(LU_LISTS, 0);
+    std::vector<std::vector<int>> own(lists);  // entries (index into ents) per list
+    std::vector<long long> load(lists, 0);
     // least-loaded list first (ties: the lower list)
     std::set<std::pair<long long, int>> heap;
-    for (int q = 0; q < LU_LISTS; ++q) heap.insert({0LL, q});
+    for (int q = 0; q < lists; ++q) heap.insert({0LL, q});
     for (size_t e = 0; e < ents.size(); ++e) {
       const auto top = *heap.begin();
       heap.erase(heap.begin());
@@ -572,17 +573,17 @@ bool build_symbolic(const HostNet &net, int N, Sym &S, std::string &err, int big
       load[top.second] += ents[e][0];
     }
     long long M = 0;
-    for (int q = 0; q < LU_LISTS; ++q) M = std::max(M, load[q]);
-    S.tw_len.assign(LU_LISTS, 0);
-    S.tw_l.assign((size_t)M * LU_LISTS, 0);
-    S.tw_u.assign((size_t)M * LU_LISTS, 0);
-    S.tw_e.assign((size_t)M * LU_LISTS, -1);
-    for (int q = 0; q < LU_LISTS; ++q) {
+    for (int q = 0; q < lists; ++q) M = std::max(M, load[q]);
+    S.tw_len.assign(lists, 0);
+    S.tw_l.assign((size_t)M * lists, 0);
+    S.tw_u.assign((size_t)M * lists, 0);
+    S.tw_e.assign((size_t)M * lists, -1);
+    for (int q = 0; q < lists; ++q) {
       int s_ = 0;
       for (int ei : own[q]) {
         const auto &en = ents[ei];
         for (int o = 0; o < en[0]; ++o, ++s_) {
-          const size_t at = (size_t)s_ * LU_LISTS + q;
+          const size_t at = (size_t)s_ * lists + q;
           const TailOp &op = tail_ops[(size_t)en[2] + o];
           S.tw_l[at] = op.l;
           S.tw_u[at] = op.u;
