@@ -54,6 +54,8 @@ __device__ __forceinline__ unsigned cluster_rank() {
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+__device__ __forceinline__ void cluster_arrive_all() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait_all() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ double ld_peer(const double *local, unsigned peer) {
   const uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(local));
   uint32_t ra;
@@ -81,11 +83,18 @@ __device__ double lu_sparse_part(const DevSym &S, int nL, const double *__restri
     else __syncthreads();
   };
   double amax = 0.0;
-  for (int p = t0i; p < S.nnzLU; p += step) {
-    const int src = S.lu_init[p];
-    const double v = src >= 0 ? J[(size_t)src * S.N + sc] : 0.0;
-    A[p] = v;
-    amax = fmax(amax, fabs(v));
+  for (int p0 = t0i; p0 < S.nnzLU; p0 += 4 * step) {  // four entries' loads in flight
+    double v[4];
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const int p = p0 + b * step, src = p < S.nnzLU ? S.lu_init[p] : -1;
+      v[b] = src >= 0 ? J[(size_t)src * S.N + sc] : 0.0;
+    }
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      if (p0 + b * step < S.nnzLU) A[p0 + b * step] = v[b];
+      amax = fmax(amax, fabs(v[b]));
+    }
   }
   amax = block_max(amax, sh);
   if (CL) {
@@ -706,11 +715,14 @@ __global__ void __launch_bounds__(256) k_round_k(DevSym S, int nk, const double 
 // The same factorization by a cluster of two CTAs per scenario (two SMs'
 // FP64 units): the sparse part shared by index parity; the nd x nd
 // trailing block is then split by column panels of 16, panel q
-// held by CTA q mod 2 in its shared memory.  Per panel: its owner factors
-// it (pivots, L column scaling, the rest of the panel), both CTAs meet at a
-// cluster barrier, the other CTA copies the panel from the owner's shared
-// memory, and each CTA solves U12 = L11^{-1} A12 and updates A22 -= L21 U12
-// on its own columns (4 x 4 register tiles).
+// held by CTA q mod 2 in its shared memory.  Per panel, factored by its owner
+// and copied by the other CTA from the owner's shared memory, each CTA solves
+// U12 = L11^{-1} A12 and updates A22 -= L21 U12 on its own columns (4 x 4
+// register tiles), the next panel first.  Bound by the FP64 units in the
+// updates and by latency elsewhere: 890 us at 1,000 buses (179 init and
+// sparse levels, 87 trailing-block products, 46 the block's load, ~50 per
+// panel) -> NEW with the panels' factorization under the other SM's updates
+// and four loads in flight in the copies.
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(512, 1)
     k_lu_factor_pair(DevSym S, int nL, const double *__restrict__ J, double *LU, double *rd, int *flags,
                      double piv_tol) {
@@ -726,66 +738,77 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(512, 1)
   if (nd == 0) return;  // the same on both CTAs
   const int np = (ns + PB - 1) / PB, LDL = ((np + 1) / 2) * PB;
   double *Pb = Tl + (size_t)ns * LDL;  // the other CTA's panel [ns][PB]
-  const int *ts = S.tail_slot;
-  // own local column lc <-> block column (2 (lc / PB) + rank) PB + lc % PB
-  for (int e = tid; e < ns * LDL; e += bd) {
-    const int i = e / LDL, lc = e % LDL;
-    const int c = (2 * (lc / PB) + (int)rank) * PB + lc % PB;
-    Tl[e] = c < ns ? A[ts[i * nd + c]] : 0.0;
+  // own local column lc <-> block column (2 (lc / PB) + rank) PB + lc % PB;
+  // the block is column-major in LU storage (whole column segments per warp,
+  // four loads in flight per thread)
+  double *D = A + S.dense_base;
+  for (int e0 = tid; e0 < ns * LDL; e0 += 4 * bd) {
+    double v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int e = e0 + q * bd, lc = e / ns, i = e - lc * ns;
+      const int c = (2 * (lc / PB) + (int)rank) * PB + lc % PB;
+      v[q] = e < ns * LDL && c < ns ? D[(size_t)c * nd + i] : 0.0;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int e = e0 + q * bd, lc = e / ns, i = e - lc * ns;
+      if (e < ns * LDL) Tl[i * LDL + lc] = v[q];
+    }
   }
   __syncthreads();
-  for (int p = 0; p < np; ++p) {
-    const int kb = p * PB, ke = min(kb + PB, ns), pb = ke - kb;
-    const bool own = (p & 1) == (int)rank;
-    const int lc0 = (p >> 1) * PB;  // the panel's first local column in its owner
-    if (own) {
-      // One barrier per column: thread 0 holds row k + 1, so it forms the
-      // next pivot's reciprocal (a dependent FP64 division, ~565 cycles) as
-      // soon as its row has that entry, under the other rows' updates.
-      const auto pivot = [&](int k) {
-        const double d = Tl[k * LDL + lc0 + (k - kb)];
-        if (!(fabs(d) > piv_tol * amax)) flags[FLAG_SINGULAR] = 1;
-        const double rk = 1.0 / d;
-        r[t0 + k] = rk;
-        sh[17 + (k & 1)] = rk;
-      };
-      if (tid == 0) pivot(kb);
-      __syncthreads();
-      for (int k = kb; k < ke; ++k) {
-        const int lk = lc0 + (k - kb);
-        const double rk = sh[17 + (k & 1)];
-        for (int i = k + 1 + tid; i < ns; i += bd) {
-          const double l = Tl[i * LDL + lk] * rk;
-          Tl[i * LDL + lk] = l;
-          int j = k + 1;
-          if (j < ke) {
-            Tl[i * LDL + lk + 1] -= l * Tl[k * LDL + lk + 1];
-            if (i == k + 1) pivot(k + 1);
-            for (++j; j < ke; ++j) Tl[i * LDL + lc0 + (j - kb)] -= l * Tl[k * LDL + lc0 + (j - kb)];
-          }
+  // Panel p on its owner.  One barrier per column: thread 0 holds row k + 1,
+  // so it forms the next pivot's reciprocal (a dependent FP64 division, ~565
+  // cycles) as soon as its row has that entry, under the other rows' updates.
+  const auto factor = [&](int p) {
+    const int kb = p * PB, ke = min(kb + PB, ns), lc0 = (p >> 1) * PB;
+    const auto pivot = [&](int k) {
+      const double d = Tl[k * LDL + lc0 + (k - kb)];
+      if (!(fabs(d) > piv_tol * amax)) flags[FLAG_SINGULAR] = 1;
+      const double rk = 1.0 / d;
+      r[t0 + k] = rk;
+      sh[17 + (k & 1)] = rk;
+    };
+    if (tid == 0) pivot(kb);
+    __syncthreads();
+    for (int k = kb; k < ke; ++k) {
+      const int lk = lc0 + (k - kb);
+      const double rk = sh[17 + (k & 1)];
+      for (int i = k + 1 + tid; i < ns; i += bd) {
+        const double l = Tl[i * LDL + lk] * rk;
+        Tl[i * LDL + lk] = l;
+        int j = k + 1;
+        if (j < ke) {
+          Tl[i * LDL + lk + 1] -= l * Tl[k * LDL + lk + 1];
+          if (i == k + 1) pivot(k + 1);
+          for (++j; j < ke; ++j) Tl[i * LDL + lc0 + (j - kb)] -= l * Tl[k * LDL + lc0 + (j - kb)];
         }
-        __syncthreads();
       }
+      __syncthreads();
     }
-    cluster_sync_all();  // panel p factored
-    if (p == np - 1) break;
-    const double *Lp;
-    int ldp, cp0;
-    if (own) {
-      Lp = Tl;
-      ldp = LDL;
-      cp0 = lc0;
-    } else {
-      for (int e = tid; e < (ns - kb) * pb; e += bd) {
-        const int i = kb + e / pb, j = e % pb;
-        Pb[i * PB + j] = ld_peer(&Tl[i * LDL + lc0 + j], rank ^ 1u);
+  };
+  if (rank == 0) factor(0);
+  cluster_sync_all();
+  // Panel p is ready everywhere; the owner of panel p + 1 updates and factors
+  // that first and arrives at the barrier, and both update their other
+  // columns before waiting there: the factorization of a panel, a chain on
+  // one SM, runs under the other SM's updates.
+  for (int p = 0; p + 1 < np; ++p) {
+    const int kb = p * PB, ke = kb + PB;
+    const bool own = (p & 1) == (int)rank, next = !own;
+    const double *Lp = Tl;
+    int ldp = LDL, cp0 = (p >> 1) * PB;  // the panel's first local column in its owner
+    if (!own) {
+      for (int e = tid; e < (ns - kb) * PB; e += bd) {
+        const int i = kb + e / PB, j = e % PB;
+        Pb[i * PB + j] = ld_peer(&Tl[i * LDL + cp0 + j], rank ^ 1u);
       }
       __syncthreads();
       Lp = Pb;
       ldp = PB;
       cp0 = 0;
     }
-    // own columns right of the panel: local panels from lps on
+    // own columns right of the panel: local panels from lcs on
     const int lcs = ((p + 2 - (int)rank) / 2) * PB;
     for (int lj = lcs + tid; lj < LDL; lj += bd) {  // a full panel: only the last can be ragged
       double x[PB];
@@ -799,38 +822,49 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(512, 1)
       for (int k = 1; k < PB; ++k) Tl[(kb + k) * LDL + lj] = x[k];
     }
     __syncthreads();
-    const int m = ns - ke, nc = LDL - lcs, nt4r = (m + 3) / 4, nt4c = (nc + 3) / 4;
-    for (int e = tid; e < nt4r * nt4c; e += bd) {
-      const int i0 = ke + (e / nt4c) * 4, j0 = lcs + (e % nt4c) * 4;
-      double c[4][4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) c[a][b] = 0.0;
-      for (int k = kb; k < ke; ++k) {
-        double lv[4], uv[4];
-#pragma unroll
-        for (int a = 0; a < 4; ++a) lv[a] = i0 + a < ns ? Lp[(i0 + a) * ldp + cp0 + (k - kb)] : 0.0;
-#pragma unroll
-        for (int b = 0; b < 4; ++b) uv[b] = j0 + b < LDL ? Tl[k * LDL + j0 + b] : 0.0;
+    // A22 -= L21 U12 on the own columns [j0s, j1)
+    const auto update = [&](int j0s, int j1) {
+      const int m = ns - ke, nt4r = (m + 3) / 4, nt4c = (j1 - j0s) / 4;
+      for (int e = tid; e < nt4r * nt4c; e += bd) {
+        const int i0 = ke + (e / nt4c) * 4, j0 = j0s + (e % nt4c) * 4;
+        double c[4][4];
 #pragma unroll
         for (int a = 0; a < 4; ++a)
 #pragma unroll
-          for (int b = 0; b < 4; ++b) c[a][b] = fma(lv[a], uv[b], c[a][b]);
+          for (int b = 0; b < 4; ++b) c[a][b] = 0.0;
+        for (int k = kb; k < ke; ++k) {
+          double lv[4], uv[4];
+#pragma unroll
+          for (int a = 0; a < 4; ++a) lv[a] = i0 + a < ns ? Lp[(i0 + a) * ldp + cp0 + (k - kb)] : 0.0;
+#pragma unroll
+          for (int b = 0; b < 4; ++b) uv[b] = Tl[k * LDL + j0 + b];
+#pragma unroll
+          for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) c[a][b] = fma(lv[a], uv[b], c[a][b]);
+        }
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int b = 0; b < 4; ++b)
+            if (i0 + a < ns) Tl[(i0 + a) * LDL + j0 + b] -= c[a][b];
       }
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b)
-          if (i0 + a < ns && j0 + b < LDL) Tl[(i0 + a) * LDL + j0 + b] -= c[a][b];
+    };
+    if (next) {
+      update(lcs, lcs + PB);
+      __syncthreads();
+      factor(p + 1);
     }
+    cluster_arrive_all();
+    update(next ? lcs + PB : lcs, LDL);
     __syncthreads();
+    cluster_wait_all();
   }
   cluster_sync_all();  // no CTA leaves while the other may still read its panels
   for (int e = tid; e < ns * LDL; e += bd) {
-    const int i = e / LDL, lc = e % LDL;
+    const int lc = e / ns, i = e - lc * ns;
     const int c = (2 * (lc / PB) + (int)rank) * PB + lc % PB;
-    if (c < ns) A[ts[i * nd + c]] = Tl[e];
+    if (c < ns) D[(size_t)c * nd + i] = Tl[i * LDL + lc];
   }
 }
 }  // namespace
