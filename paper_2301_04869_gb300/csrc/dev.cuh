@@ -91,7 +91,17 @@ __device__ __forceinline__ double rsqrt_newton(double d) {
   r = fma(-h * y, y, 0.5);
   return fma(y, r, y);
 }
-
+// 1/d for d > 0, likewise: the single-precision estimate (relative error e
+// below 2^-22) and one third-order step y (1 + e + e^2), e = 1 - d y, whose
+// error is e^3: three dependent operations instead of a division's ~565
+// cycles.
+__device__ __forceinline__ double rcp_newton(double d) {
+  if (!(d > 1e-30 && d < 1e30)) return 1.0 / d;
+  float yf;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"((float)d));
+  const double y = (double)yf, e = fma(-d, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
 
 __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
