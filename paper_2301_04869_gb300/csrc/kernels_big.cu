@@ -110,9 +110,44 @@ __global__ void __launch_bounds__(128) k_blu_l21(int nd, int nx, int t0, long lo
     if (c < pb) A[(size_t)(kb + c) * nd + i] = a[c];
 }
 
-// U12 = L11^{-1} A12: columns [ke, nd) of rows [kb, ke); a warp per column,
+// U12 = L11^{-1} A12: columns [ke, nd) of rows [kb, ke), 64 columns per CTA
+// through shared memory (rows contiguous in global memory), a thread per
+// column with its 64 rows in registers.  FP64-bound: only the triangle's
+// multiply-adds are issued; a warp per column with a shuffle per row issued
+// four times as many (5.8 -> 3.85 ms at 1,776 states x 32 scenarios).
+__global__ void __launch_bounds__(64) k_blu_trsm(int nd, long long nnzlu, int dense_base, double *LU, int kb, int ke) {
+  extern __shared__ double smem_t[];
+  double(*L11)[PB] = reinterpret_cast<double(*)[PB]>(smem_t);            // L11[k][i]: broadcast reads
+  double(*X)[PB + 1] = reinterpret_cast<double(*)[PB + 1]>(smem_t + PB * PB);  // X[column][row]
+  const int sc = blockIdx.y, tid = threadIdx.x, pb = ke - kb;
+  double *A = LU + (size_t)sc * nnzlu + dense_base;
+  const int j0 = ke + blockIdx.x * 64;
+  for (int e = tid; e < PB * PB; e += 64) {
+    const int i = e % PB, k = e / PB;
+    L11[k][i] = i < pb && k < i ? A[(size_t)(kb + k) * nd + kb + i] : 0.0;
+    X[k][i] = i < pb && j0 + k < nd ? A[(size_t)(j0 + k) * nd + kb + i] : 0.0;
+  }
+  __syncthreads();
+  double x[PB];
+#pragma unroll
+  for (int i = 0; i < PB; ++i) x[i] = X[tid][i];
+#pragma unroll
+  for (int k = 0; k < PB; ++k)
+#pragma unroll
+    for (int i = k + 1; i < PB; ++i) x[i] -= L11[k][i] * x[k];
+#pragma unroll
+  for (int i = 0; i < PB; ++i) X[tid][i] = x[i];
+  __syncthreads();
+  for (int e = tid; e < PB * PB; e += 64) {
+    const int i = e % PB, k = e / PB;
+    if (i < pb && j0 + k < nd) A[(size_t)(j0 + k) * nd + kb + i] = X[k][i];
+  }
+}
+
+// The same with a warp per column, where columns are few: 16 times the warps,
+// each a chain a quarter as long, for four times the multiply-adds;
 // lane l holding rows kb + l and kb + 32 + l; L11 staged in shared memory.
-__global__ void __launch_bounds__(256) k_blu_trsm(int nd, long long nnzlu, int dense_base, double *LU, int kb,
+__global__ void __launch_bounds__(256) k_blu_trsm_warp(int nd, long long nnzlu, int dense_base, double *LU, int kb,
                                                   int ke) {
   __shared__ double L11[PB][PB + 1];
   const int sc = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -283,6 +318,7 @@ __global__ void __launch_bounds__(256) k_btrsm_update(int nd, int nx, int t0, in
 
 template <typename T>
 constexpr size_t update_smem() { return sizeof(T) * PB * (TT + 1) + sizeof(T) * PB * TT; }
+constexpr size_t trsm_smem() { return sizeof(double) * PB * PB + sizeof(double) * 64 * (PB + 1); }
 constexpr size_t gemm_smem() { return sizeof(double) * PB * TT + sizeof(double) * PB * (TT + 1); }
 
 template <typename T>
@@ -358,7 +394,10 @@ void launch_big_lu_dense(const DevSym &S, double *LU, double *rd, const double *
                          const EmuLuPlan *emu_lu) {
   static const bool cap = cudaFuncSetAttribute(k_blu_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)gemm_smem()) == cudaSuccess;
+  static const bool cap_t = cudaFuncSetAttribute(k_blu_trsm, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)trsm_smem()) == cudaSuccess;
   (void)cap;
+  (void)cap_t;
   const int nd = S.nd;
   for (int kb = 0; kb < nd; kb += PB) {
     const int ke = kb + PB < nd ? kb + PB : nd;
@@ -368,7 +407,13 @@ void launch_big_lu_dense(const DevSym &S, double *LU, double *rd, const double *
     k_blu_l21<<<dim3((nd - ke + 127) / 128, S.N), 128, 0, st>>>(nd, S.nx, S.t0, S.nnzLU, S.dense_base, LU, rd, kb,
                                                                  ke);
     ipm_count_launch();
-    k_blu_trsm<<<dim3((nd - ke + 7) / 8, S.N), 256, 0, st>>>(nd, S.nnzLU, S.dense_base, LU, kb, ke);
+    // a thread per column from two CTAs per SM on (541 states x 10 scenarios,
+    // 90 CTAs at most: 644 us against 229 by warps; 1,776 x 32: 3.85 ms
+    // against 5.8)
+    if ((long long)((nd - ke + 63) / 64) * S.N >= 2 * 152)
+      k_blu_trsm<<<dim3((nd - ke + 63) / 64, S.N), 64, trsm_smem(), st>>>(nd, S.nnzLU, S.dense_base, LU, kb, ke);
+    else
+      k_blu_trsm_warp<<<dim3((nd - ke + 7) / 8, S.N), 256, 0, st>>>(nd, S.nnzLU, S.dense_base, LU, kb, ke);
     ipm_count_launch();
     if (emu_lu) {
       // FP64-grade on the tensor cores (exact 7-bit slices of L21, U12)
