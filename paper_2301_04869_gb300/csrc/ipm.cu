@@ -562,10 +562,12 @@ void fp64_contraction(ipm_ctx *c, cudaStream_t st) {
                         c->partial, st);
 }
 
-// split the N*nx contraction rows into G chunks (a multiple of 16 rows each)
+// split the N*nx contraction rows into at most G chunks (a multiple of 16 rows each)
 void set_groups(ipm_ctx *c, long long G) {
   const long long krows = (long long)c->S.N * c->S.nx;
-  G = std::max(1LL, std::min(G, (krows + 15) / 16));
+  // at least 64 rows to a chunk: the small problems' tile sums (a thread per
+  // entry walks the chunks) cost more than their products otherwise
+  G = std::max(1LL, std::min(G, (krows + 63) / 64));
   long long kc = (krows + G - 1) / G;
   kc = (kc + 15) / 16 * 16;
   c->kchunk = kc;

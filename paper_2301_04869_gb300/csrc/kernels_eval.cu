@@ -14,6 +14,8 @@
 // 2 (dP dP^T + dQ dQ^T + P d2P + Q d2Q) come from the same closed forms.
 #include <atomic>
 
+#include <initializer_list>
+
 #include "dev.cuh"
 #include "kernels.h"
 
@@ -111,14 +113,29 @@ __device__ __forceinline__ double lam_Q(const DevSym &S, const double *y, const 
   return q >= 0 ? y[(size_t)sc * S.nx + q] : z[(size_t)sc * S.m + S.gen_of_bus[k]];
 }
 
-__global__ void k_functions(DevSym S, const double *__restrict__ x, const double *__restrict__ u,
-                            double *P, double *Q, double *g, double *h, double *fs) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= S.n * S.N) return;
-  const int i = t / S.N, sc = t - i * S.N;
+// Sum over LN neighbouring lanes (LN a power of two).
+template <int LN>
+__device__ __forceinline__ double lanes_sum(double v) {
+#pragma unroll
+  for (int o = LN / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// LN lanes per (bus, scenario), each with every LN-th incident line: one
+// where the pairs fill the GPU (coalesced over the scenarios), eight on the
+// smaller problems, where a bus's lines in turn (an FP64 sine and cosine and
+// ~100 dependent operations each) were the time of the kernel (functions +
+// derivatives, 30 buses x 1: 17 + 43 -> 6 + 12 us, 119 x 7: 19 + 78 -> 7 + 23).
+template <int LN>
+__global__ void __launch_bounds__(128) k_functions(DevSym S, const double *__restrict__ x, const double *__restrict__ u,
+                                                   double *P, double *Q, double *g, double *h, double *fs) {
+  const int tl = blockIdx.x * blockDim.x + threadIdx.x, sub = tl % LN;
+  const bool on_t = tl / LN < S.n * S.N;  // whole warps reach the sums below
+  const int t = on_t ? tl / LN : 0, i = t / S.N, sc = t - i * S.N;
   const double thi = bus_theta(S, x, sc, i), vi = bus_v(S, x, u, sc, i);
   double p = 0.0, q = 0.0;
-  for (int e = S.inc_ptr[i]; e < S.inc_ptr[i + 1]; ++e) {
+  const int e1 = on_t ? S.inc_ptr[i + 1] : 0;
+  for (int e = S.inc_ptr[i] + sub; e < e1; e += LN) {
     const int l = S.inc_line[e], k = S.inc_other[e];
     double sn, cs;
     sincos(thi - bus_theta(S, x, sc, k), &sn, &cs);
@@ -129,6 +146,9 @@ __global__ void k_functions(DevSym S, const double *__restrict__ x, const double
     q += le.Q;
     if (S.nflow) h[(size_t)sc * S.m + flow_row(S, l, i)] = le.P * le.P + le.Q * le.Q;
   }
+  p = lanes_sum<LN>(p);
+  q = lanes_sum<LN>(q);
+  if (!on_t || sub != 0) return;
   const size_t bi = (size_t)sc * S.n + i;
   P[bi] = p;
   Q[bi] = q;
@@ -144,18 +164,21 @@ __global__ void k_functions(DevSym S, const double *__restrict__ x, const double
   }
 }
 
-__global__ void k_derivatives(DevSym S, const double *__restrict__ x, const double *__restrict__ u,
-                              const double *__restrict__ y, const double *__restrict__ z,
-                              const double *__restrict__ h, double *J, double *W, double *JTl, double *HF) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= S.n * S.N) return;
-  const int i = t / S.N, sc = t - i * S.N, N = S.N;
+template <int LN>
+__global__ void __launch_bounds__(128) k_derivatives(DevSym S, const double *__restrict__ x,
+                                                     const double *__restrict__ u, const double *__restrict__ y,
+                                                     const double *__restrict__ z, const double *__restrict__ h,
+                                                     double *J, double *W, double *JTl, double *HF) {
+  const int tl = blockIdx.x * blockDim.x + threadIdx.x, sub = tl % LN;
+  const bool on_t = tl / LN < S.n * S.N;  // whole warps reach the sums below
+  const int t = on_t ? tl / LN : 0, i = t / S.N, sc = t - i * S.N, N = S.N;
   const double thi = bus_theta(S, x, sc, i), vi = bus_v(S, x, u, sc, i);
   const double lPi = lam_P(S, y, z, h, sc, i), lQi = lam_Q(S, y, z, sc, i);
   double jd0 = 0, jd1 = 0, jd2 = 0, jd3 = 0;   // dP/dth, dP/dv, dQ/dth, dQ/dv (own bus)
   double wtt = 0, wtv = 0, wvv = 0;            // diagonal Hessian block
   double gt = 0, gv = 0;                       // (J^T lambda) at (th_i, v_i)
-  for (int e = S.inc_ptr[i]; e < S.inc_ptr[i + 1]; ++e) {
+  const int e1 = on_t ? S.inc_ptr[i + 1] : 0;
+  for (int e = S.inc_ptr[i] + sub; e < e1; e += LN) {
     const int l = S.inc_line[e], k = S.inc_other[e], q = S.inc_aslot[e];
     const double vk = bus_v(S, x, u, sc, k);
     double sn, cs;
@@ -203,6 +226,8 @@ __global__ void k_derivatives(DevSym S, const double *__restrict__ x, const doub
       W[((size_t)q * 4 + 3) * N + sc] += zo * d2flow(own, 1, 3) + zk * d2flow(oth, 3, 1);
     }
   }
+  for (double *v : {&jd0, &jd1, &jd2, &jd3, &wtt, &wtv, &wvv, &gt, &gv}) *v = lanes_sum<LN>(*v);
+  if (!on_t || sub != 0) return;
   const int d = S.a_diag[i];
   J[((size_t)d * 4 + 0) * N + sc] = jd0;
   J[((size_t)d * 4 + 1) * N + sc] = jd1;
@@ -329,24 +354,31 @@ __global__ void k_rhs_x(DevSym S, DevWork D, const double *mu_d) {
 
 // u gradient of sum_i (f_i + y_i^T g_i + z_i^T h_i), summed over scenarios in
 // index order (first-stage coupling row of eq. (5)).
-__global__ void k_ugrad(DevSym S, DevWork D, double *gLu, double *HTt_u) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+// A warp per u row, lanes over the scenarios (fixed order: lane l takes
+// scenarios l, l + 32, ...): one thread walking them all waited for its loads
+// in turn (1,000 buses x 64: 52 us, less than 10 with this).
+__global__ void __launch_bounds__(256) k_ugrad(DevSym S, DevWork D, double *gLu, double *HTt_u) {
+  const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (j >= S.nu) return;
   double acc = 0.0, acc2 = 0.0;
   if (j < S.ng) {
     const int a = S.hrow_bus[j];
-    for (int sc = 0; sc < S.N; ++sc) {
+    for (int sc = lane; sc < S.N; sc += 32) {
       acc += D.JTl[(size_t)sc * 2 * S.n + S.n + a];
       if (HTt_u) acc2 += HT_at(S, D.J, D.HF, D.tv, sc, a, 1);
     }
   } else {
     const int k = j - S.ng + 1, a = S.hrow_bus[k];
     const double pg = D.u[j];
-    for (int sc = 0; sc < S.N; ++sc)
+    for (int sc = lane; sc < S.N; sc += 32)
       acc += (2.0 * S.c2[k] * pg + S.c1[k]) / S.N - D.y[(size_t)sc * S.nx + S.xth[a]];
   }
-  gLu[j] = acc;
-  if (HTt_u) HTt_u[j] = acc2;
+  acc = warp_sum(acc);
+  acc2 = warp_sum(acc2);
+  if (lane == 0) {
+    gLu[j] = acc;
+    if (HTt_u) HTt_u[j] = acc2;
+  }
 }
 
 __global__ void k_rhs_u(DevSym S, DevWork D, const double *gLu, const double *HTt_u, const double *mu_d) {
@@ -363,12 +395,23 @@ __global__ void k_rhs_u(DevSym S, DevWork D, const double *gLu, const double *HT
 // ---------------------------------------------------------------------------
 static inline int nblk(long long n, int b) { return (int)((n + b - 1) / b); }
 
+// eight lanes per (bus, scenario) until the pairs alone come to 256 threads
+// per SM
+static inline bool eval_lanes(const DevSym &S) { return (long long)S.n * S.N < 152 * 256; }
+
 void launch_functions(const DevSym &S, const double *x, const double *u, double *P, double *Q,
                       double *g, double *h, double *fs, cudaStream_t st) {
-  k_functions<<<nblk((long long)S.n * S.N, 128), 128, 0, st>>>(S, x, u, P, Q, g, h, fs); ipm_count_launch();
+  const long long t = (long long)S.n * S.N;
+  if (eval_lanes(S)) k_functions<8><<<nblk(8 * t, 128), 128, 0, st>>>(S, x, u, P, Q, g, h, fs);
+  else k_functions<1><<<nblk(t, 128), 128, 0, st>>>(S, x, u, P, Q, g, h, fs);
+  ipm_count_launch();
 }
 void launch_derivatives(const DevSym &S, DevWork &D, cudaStream_t st) {
-  k_derivatives<<<nblk((long long)S.n * S.N, 128), 128, 0, st>>>(S, D.x, D.u, D.y, D.z, D.h, D.J, D.W, D.JTl, D.HF); ipm_count_launch();
+  const long long t = (long long)S.n * S.N;
+  if (eval_lanes(S))
+    k_derivatives<8><<<nblk(8 * t, 128), 128, 0, st>>>(S, D.x, D.u, D.y, D.z, D.h, D.J, D.W, D.JTl, D.HF);
+  else k_derivatives<1><<<nblk(t, 128), 128, 0, st>>>(S, D.x, D.u, D.y, D.z, D.h, D.J, D.W, D.JTl, D.HF);
+  ipm_count_launch();
 }
 void launch_sigmas(const DevSym &S, DevWork &D, cudaStream_t st) {
   long long tot = (long long)S.N * S.nx + (long long)S.N * S.m + S.nu;
@@ -380,9 +423,9 @@ void launch_condense(const DevSym &S, DevWork &D, cudaStream_t st) {
 void launch_rhs(const DevSym &S, DevWork &D, const double *mu, double *gLu, double *HTt_u, cudaStream_t st) {
   k_rhs_s<<<nblk((long long)S.N * S.m, 256), 256, 0, st>>>(S, D, mu); ipm_count_launch();
   k_rhs_x<<<nblk((long long)S.N * S.nx, 256), 256, 0, st>>>(S, D, mu); ipm_count_launch();
-  k_ugrad<<<nblk(S.nu, 64), 64, 0, st>>>(S, D, gLu, HTt_u); ipm_count_launch();
+  k_ugrad<<<nblk(S.nu, 8), 256, 0, st>>>(S, D, gLu, HTt_u); ipm_count_launch();
   k_rhs_u<<<nblk(S.nu, 64), 64, 0, st>>>(S, D, gLu, HTt_u, mu); ipm_count_launch();
 }
 void launch_ugrad(const DevSym &S, DevWork &D, double *gLu, cudaStream_t st) {
-  k_ugrad<<<nblk(S.nu, 64), 64, 0, st>>>(S, D, gLu, nullptr); ipm_count_launch();
+  k_ugrad<<<nblk(S.nu, 8), 256, 0, st>>>(S, D, gLu, nullptr); ipm_count_launch();
 }

@@ -163,23 +163,28 @@ __global__ void k_res_x(DevSym S, DevWork D, double delta, const double *px, con
   warp_max2(res, scl, amax);
 }
 
-// u rows (scenarios summed in index order):
+// u rows (a warp per row, lanes over the scenarios):
 // rho_1u = -r1u - (sum_i kpu_i + diag1 p_u) - delta p_u - sum_i (G_u^T p_y,i + H_u^T tw_i)
-__global__ void k_res_u(DevSym S, DevWork D, double delta, const double *pu, const double *upart,
-                        const double *umag, const double *diag1, double *rho1u, unsigned long long *amax) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(256) k_res_u(DevSym S, DevWork D, double delta, const double *pu,
+                                               const double *upart, const double *umag, const double *diag1,
+                                               double *rho1u, unsigned long long *amax) {
+  const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   double res = 0.0, scl = 0.0;
   if (j < S.nu) {
     double acc = 0.0, mag = 0.0;
-    for (int sc = 0; sc < S.N; ++sc) {
+    for (int sc = lane; sc < S.N; sc += 32) {
       acc += upart[(size_t)sc * S.nu + j];
       mag = fmax(mag, umag[(size_t)sc * S.nu + j]);
     }
-    const double dp = (diag1[j] + delta) * pu[j];
-    const double r1 = -D.r1u[j] - acc - dp;
-    rho1u[j] = r1;
-    res = fabs(r1);
-    scl = fmax(fmax(fabs(D.r1u[j]), mag), fmax(fabs(acc), fabs(dp)));
+    acc = warp_sum(acc);
+    mag = warp_max(mag);
+    if (lane == 0) {
+      const double dp = (diag1[j] + delta) * pu[j];
+      const double r1 = -D.r1u[j] - acc - dp;
+      rho1u[j] = r1;
+      res = fabs(r1);
+      scl = fmax(fmax(fabs(D.r1u[j]), mag), fmax(fabs(acc), fabs(dp)));
+    }
   }
   warp_max2(res, scl, amax);
 }
@@ -266,7 +271,7 @@ void launch_aug_residual(const DevSym &S, const DevWork &D, double delta, const 
   k_res_x<<<nblk(NX + NU, 256), 256, 0, st>>>(S, D, delta, px, pu, py, tw, kpx_pos, kpu, rho1x, rho3, upart, umag,
                                                amax);
   ipm_count_launch();
-  k_res_u<<<nblk(S.nu, 128), 128, 0, st>>>(S, D, delta, pu, upart, umag, diag1, rho1u, amax); ipm_count_launch();
+  k_res_u<<<nblk(S.nu, 8), 256, 0, st>>>(S, D, delta, pu, upart, umag, diag1, rho1u, amax); ipm_count_launch();
 }
 
 void launch_htv(const DevSym &S, const DevWork &D, const double *ax, const double *au, const double *v, double *outx,

@@ -272,32 +272,33 @@ __global__ void k_gu_apply(DevSym S, const double *J, const double *pu, double *
   v[t] = acc;
 }
 
-// kpx = K_xx px (+ K_xu pu);  kpu = K_ux px + K_uu pu  (position rows, u rows)
-__global__ void k_kapply(DevSym S, const double *K, const double *px_pos, const double *pu,
-                         double *kpx, double *kpu) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+// kpx = K_xx px (+ K_xu pu);  kpu = K_ux px + K_uu pu  (position rows, u rows).
+// Eight lanes per row: the rows of buses next to a hub or a generator have
+// many entries, and one thread took their three dependent loads and the
+// multiply-add in turn (30 buses x 1: 13 -> 4 us,
+// 119 x 7: 15 -> 5, 1,000 x 64: 24 -> 17).
+__global__ void __launch_bounds__(256) k_kapply(DevSym S, const double *__restrict__ K, const double *px_pos,
+                                                const double *pu, double *kpx, double *kpu) {
+  const long long t = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+  const int sub = threadIdx.x & 7;
   const long long nX = (long long)S.N * S.nx;
-  if (t < nX) {
-    const int sc = (int)(t / S.nx), p = (int)(t - (long long)sc * S.nx);
-    double acc = 0.0;
-    for (int e = S.kx_ptr[p]; e < S.kx_ptr[p + 1]; ++e) {
-      const int col = S.kx_col[e];
-      const double v = K[(size_t)S.kx_src[e] * S.N + sc];
-      if (col < S.nx) acc += v * px_pos[(size_t)sc * S.nx + col];
-      else if (pu) acc += v * pu[col - S.nx];
+  const bool xrow = t < nX, urow = !xrow && kpu && t < nX + (long long)S.N * S.nu;
+  double acc = 0.0;
+  if (xrow || urow) {
+    const long long q = xrow ? t : t - nX;
+    const int len = xrow ? S.nx : S.nu, sc = (int)(q / len), p = (int)(q - (long long)sc * len);
+    const int *ptr = xrow ? S.kx_ptr : S.ku_ptr, *cols = xrow ? S.kx_col : S.ku_col, *src = xrow ? S.kx_src : S.ku_src;
+    for (int e = ptr[p] + sub; e < ptr[p + 1]; e += 8) {
+      const int col = cols[e];
+      if (col >= S.nx && !pu) continue;
+      acc += K[(size_t)src[e] * S.N + sc] * (col < S.nx ? px_pos[(size_t)sc * S.nx + col] : pu[col - S.nx]);
     }
-    kpx[t] = acc;
-  } else if (kpu && t < nX + (long long)S.N * S.nu) {
-    const long long q = t - nX;
-    const int sc = (int)(q / S.nu), j = (int)(q - (long long)sc * S.nu);
-    double acc = 0.0;
-    for (int e = S.ku_ptr[j]; e < S.ku_ptr[j + 1]; ++e) {
-      const int col = S.ku_col[e];
-      const double v = K[(size_t)S.ku_src[e] * S.N + sc];
-      acc += v * (col < S.nx ? px_pos[(size_t)sc * S.nx + col] : pu[col - S.nx]);
-    }
-    kpu[q] = acc;
   }
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (sub != 0) return;
+  if (xrow) kpx[t] = acc;
+  else if (urow) kpu[t - nX] = acc;
 }
 
 __global__ void k_lincomb(long long n, double *out, double a, const double *x, double b,
@@ -371,14 +372,15 @@ __global__ void __launch_bounds__(256) k_zt_part(DevSym S, const double *__restr
   }
 }
 
-// out[j] = beta*out[j] + sum_s part[s][j]  (scenarios in index order);
-// beta = 0 does not read out (it may hold anything, NaN included)
-__global__ void k_zt_sum(DevSym S, const double *part, double beta, double *out) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+// out[j] = beta*out[j] + sum_s part[s][j]  (a warp per u row, lanes over the
+// scenarios); beta = 0 does not read out (it may hold anything, NaN included)
+__global__ void __launch_bounds__(256) k_zt_sum(DevSym S, const double *part, double beta, double *out) {
+  const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (j >= S.nu) return;
   double acc = 0.0;
-  for (int sc = 0; sc < S.N; ++sc) acc += part[(size_t)sc * S.nu + j];
-  out[j] = beta == 0.0 ? acc : beta * out[j] + acc;
+  for (int sc = lane; sc < S.N; sc += 32) acc += part[(size_t)sc * S.nu + j];
+  acc = warp_sum(acc);
+  if (lane == 0) out[j] = beta == 0.0 ? acc : beta * out[j] + acc;
 }
 
 // v[s][p] = a * v[s][p] + (Z_s pu)[p]   (position rows)
@@ -411,14 +413,16 @@ __global__ void __launch_bounds__(256) k_gut_sum(DevSym S, const double *__restr
   if (lane == 0) out[j] = scale * acc;
 }
 
-// out[j] += sum_s kpu[s][j] + (diag[j] + delta) v[j]   (scenarios in index order)
-__global__ void k_apply_finish(DevSym S, const double *kpu, const double *diag, double delta, const double *v,
-                               double *out) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+// out[j] += sum_s kpu[s][j] + (diag[j] + delta) v[j]; a warp per u row, lanes
+// over the scenarios
+__global__ void __launch_bounds__(256) k_apply_finish(DevSym S, const double *kpu, const double *diag, double delta,
+                                                      const double *v, double *out) {
+  const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (j >= S.nu) return;
-  double acc = out[j];
-  for (int sc = 0; sc < S.N; ++sc) acc += kpu[(size_t)sc * S.nu + j];
-  out[j] = acc + (diag[j] + delta) * v[j];
+  double acc = 0.0;
+  for (int sc = lane; sc < S.N; sc += 32) acc += kpu[(size_t)sc * S.nu + j];
+  acc = warp_sum(acc);
+  if (lane == 0) out[j] = out[j] + acc + (diag[j] + delta) * v[j];
 }
 
 // out[0] = a.b, out[1] = c.d (one block, fixed partition and tree)
@@ -595,7 +599,7 @@ void launch_gu_apply(const DevSym &S, const double *J, const double *pu, double 
 void launch_kapply(const DevSym &S, const double *K, const double *px_pos, const double *pu, double *kpx,
                    double *kpu, cudaStream_t st) {
   long long n = (long long)S.N * S.nx + (kpu ? (long long)S.N * S.nu : 0);
-  k_kapply<<<nblk(n, 256), 256, 0, st>>>(S, K, px_pos, pu, kpx, kpu); ipm_count_launch();
+  k_kapply<<<nblk(n, 32), 256, 0, st>>>(S, K, px_pos, pu, kpx, kpu); ipm_count_launch();
 }
 void launch_lincomb(long long n, double *out, double a, const double *x, double b, const double *y,
                     double c, const double *z, cudaStream_t st) {
@@ -609,7 +613,7 @@ void launch_rhs_reduced(const DevSym &S, const double *J, const double *K, const
 void launch_zt_apply(const DevSym &S, const double *Z, const double *w, const double *K, const double *b,
                      double alpha, double beta, double *out, double *part, cudaStream_t st) {
   k_zt_part<<<dim3((S.nu + 31) / 32, S.N), 256, 0, st>>>(S, Z, w, K, b, alpha, part); ipm_count_launch();
-  k_zt_sum<<<nblk(S.nu, 64), 64, 0, st>>>(S, part, beta, out); ipm_count_launch();
+  k_zt_sum<<<nblk(S.nu, 8), 256, 0, st>>>(S, part, beta, out); ipm_count_launch();
 }
 void launch_z_apply(const DevSym &S, const double *Z, const double *pu, double a, double *v, cudaStream_t st) {
   k_z_apply<<<nblk((long long)S.N * S.nx * 32, 256), 256, 0, st>>>(S, Z, pu, a, v); ipm_count_launch();
@@ -620,7 +624,7 @@ void launch_gut_sum(const DevSym &S, const double *J, const double *a, double sc
 }
 void launch_apply_finish(const DevSym &S, const double *kpu, const double *diag, double delta, const double *v,
                          double *out, cudaStream_t st) {
-  k_apply_finish<<<nblk(S.nu, 128), 128, 0, st>>>(S, kpu, diag, delta, v, out); ipm_count_launch();
+  k_apply_finish<<<nblk(S.nu, 8), 256, 0, st>>>(S, kpu, diag, delta, v, out); ipm_count_launch();
 }
 void launch_dot2(int n, const double *a, const double *b, const double *c, const double *d, double *out,
                  cudaStream_t st) {
