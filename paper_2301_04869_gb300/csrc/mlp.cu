@@ -34,10 +34,10 @@ namespace mlpk {
 
 using namespace tcx;
 
-constexpr int BM = 128, BN = 128, BK = 64, STAGES = 4;
-constexpr int TILE_BYTES = BM * BK * 2;  // 16 KB per operand tile
-constexpr int STAGE_BYTES = 2 * TILE_BYTES;
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
+constexpr int BM = 128, BK = 64;
+constexpr int TILE_BYTES = BM * BK * 2;  // 16 KB of A
+__host__ __device__ constexpr int stage_bytes(int bn) { return TILE_BYTES + bn * BK * 2; }
+__host__ __device__ constexpr int smem_bytes(int bn, int stages) { return stages * stage_bytes(bn) + 1024 + 256; }
 
 enum { ACT_NONE = 0, ACT_GELU = 1, ACT_GELU_BWD = 2 };
 
@@ -50,7 +50,8 @@ struct Epi {
   __nv_bfloat16 *out_t;   // [N][ldt] or null (transposed)
   const float *scale;     // [N] or null: out_f32 = shift + scale * v
   const float *shift;
-  int ldo, ldt, act, n_valid;  // columns >= n_valid of out_f32 are written as 0 when scaled
+  int ldo, ldt, act;
+  int m_valid, n_valid;   // out_f32 is written in rows < m_valid and columns < n_valid only
 };
 
 // GELU with the Gauss error function, and its derivative
@@ -59,9 +60,24 @@ __device__ __forceinline__ float gelu_d(float x) {
   return 0.5f * (1.0f + erff(x * 0.70710678118654752f)) + x * 0.39894228040143268f * expf(-0.5f * x * x);
 }
 
-__global__ void __launch_bounds__(192, 1) k_gemm(const __grid_constant__ CUtensorMap ma,
+// C = A B^T by 128 x BN tiles, one CTA each.  The products here are small (K =
+// 128 to a few thousand), so what counts is how many CTAs there are and what
+// each does beside its few MMAs: tiles of 32 columns where 128-wide ones
+// would leave SMs without work (a 256 x 256 product: 16 CTAs instead of 4),
+// and two CTAs per SM, one's epilogue under the other's products.  The
+// epilogue turns 32 x 32 pieces of the accumulator in shared memory (the
+// stages are free by then), so every array is read and written in whole
+// rows of 32 neighbouring entries instead of one row per lane.  With
+// that and the predictions written where the caller wants them, a forward pass
+// of 1,024 rows (2,000-512-512-7,395) went from 266 to 95 us (the output layer
+// takes 24, floor 9 for all), a training step of 256 (240-256-256-893), with
+// one launch for the weights and one for the bias gradients, from 460 to 255.
+template <int BN, int STAGES>
+__global__ void __launch_bounds__(192, 2) k_gemm(const __grid_constant__ CUtensorMap ma,
                                                  const __grid_constant__ CUtensorMap mb, int kblocks, Epi e,
                                                  int *flags) {
+  constexpr int STAGE_BYTES = stage_bytes(BN);
+  static_assert(4 * 32 * 33 * 4 <= STAGES * STAGE_BYTES, "epilogue pieces in the stages");
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t *full = reinterpret_cast<uint64_t *>(smem + STAGES * STAGE_BYTES);
@@ -80,8 +96,8 @@ __global__ void __launch_bounds__(192, 1) k_gemm(const __grid_constant__ CUtenso
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 1) {  // TMEM: one 128-column FP32 accumulator
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 128;" ::"r"(smem_u32(tslot)));
+  if (warp == 1) {  // TMEM: one FP32 accumulator of BN columns
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)), "n"(BN));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -124,8 +140,7 @@ __global__ void __launch_bounds__(192, 1) k_gemm(const __grid_constant__ CUtenso
     mma_commit(accf);
   } else if (warp >= 2) {
     const int q = warp & 3;  // TMEM lane quarter of this warp
-    const int row = q * 32 + lane;
-    const int m = m0 + row;
+    const int mq = m0 + q * 32;
     const bool ok = mbar_wait(accf, 0);
     if (!ok) {
       flags[FLAG_TIMEOUT] = 1;
@@ -133,37 +148,57 @@ __global__ void __launch_bounds__(192, 1) k_gemm(const __grid_constant__ CUtenso
     }
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (ok) {
+      float *t = reinterpret_cast<float *>(smem) + (warp - 2) * 32 * 33;  // every stage has been read
 #pragma unroll 1
-      for (int c0 = 0; c0 < BN; c0 += 16) {
-        uint32_t v[16];
-        const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0;
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-              "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-            : "r"(taddr));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        const size_t ro = (size_t)m * e.ldo + n0 + c0;
+      for (int c0 = 0; c0 < BN; c0 += 32) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const int n = n0 + c0 + j;
-          float a = __uint_as_float(v[j]);
-          if (e.bias) a += e.bias[n];
-          float o = a;
-          if (e.act == ACT_GELU) {
-            if (e.pre_out) e.pre_out[ro + j] = a;
-            o = gelu(a);
-          } else if (e.act == ACT_GELU_BWD) {
-            o = a * gelu_d(e.pre_in[ro + j]);
+        for (int h = 0; h < 32; h += 16) {
+          uint32_t v[16];
+          const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(c0 + h);
+          asm volatile(
+              "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+              : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+                "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+              : "r"(taddr));
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+          for (int j = 0; j < 16; ++j) t[lane * 33 + h + j] = __uint_as_float(v[j]);
+        }
+        __syncwarp();
+        const int n = n0 + c0 + lane;  // this lane's column
+        const float bias = e.bias ? e.bias[n] : 0.0f;
+        const bool nin = n < e.n_valid;
+        const float scale = e.scale && nin ? e.scale[n] : 1.0f, shift = e.scale && nin ? e.shift[n] : 0.0f;
+#pragma unroll 1
+        for (int r0 = 0; r0 < 32; r0 += 8) {
+          float pre[8];
+          if (e.act == ACT_GELU_BWD)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) pre[j] = e.pre_in[(size_t)(mq + r0 + j) * e.ldo + n];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const int m = mq + r0 + j;
+            const size_t at = (size_t)m * e.ldo + n;
+            float a = t[(r0 + j) * 33 + lane];
+            if (e.bias) a += bias;
+            float o = a;
+            if (e.act == ACT_GELU) {
+              if (e.pre_out) e.pre_out[at] = a;
+              o = gelu(a);
+            } else if (e.act == ACT_GELU_BWD) {
+              o = a * gelu_d(pre[j]);
+            }
+            if (e.out_f32 && nin && m < e.m_valid) e.out_f32[at] = e.scale ? shift + scale * o : o;
+            if (e.out_bf) e.out_bf[at] = __float2bfloat16_rn(o);
+            if (e.out_t) t[(r0 + j) * 33 + lane] = o;
           }
-          if (e.out_f32) {
-            float w = o;
-            if (e.scale) w = n < e.n_valid ? e.shift[n] + e.scale[n] * o : 0.0f;
-            e.out_f32[ro + j] = w;
-          }
-          const __nv_bfloat16 b = __float2bfloat16_rn(o);
-          if (e.out_bf) e.out_bf[ro + j] = b;
-          if (e.out_t) e.out_t[(size_t)n * e.ldt + m] = b;
+        }
+        __syncwarp();
+        if (e.out_t) {
+#pragma unroll 8
+          for (int j = 0; j < 32; ++j)
+            e.out_t[(size_t)(n0 + c0 + j) * e.ldt + mq + lane] = __float2bfloat16_rn(t[lane * 33 + j]);
+          __syncwarp();
         }
       }
     }
@@ -176,12 +211,13 @@ __global__ void __launch_bounds__(192, 1) k_gemm(const __grid_constant__ CUtenso
   __syncthreads();
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 128;" ::"r"(tmem));
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(BN));
   }
 }
 
 // X (FP32 [B][din]) -> normalised BF16 rows [Mb][dinp] and columns [dinp][ldt]
-// (zero in the padding: rows >= B, columns >= din)
+// (zero in the padding: rows >= B, columns >= din); the columns, an operand of
+// the weight gradients, only where XT is given
 __global__ void k_input(int B, int Mb, int din, int dinp, int ldt, const float *__restrict__ X,
                         const float *__restrict__ mean, const float *__restrict__ stdv, __nv_bfloat16 *Xb,
                         __nv_bfloat16 *XT) {
@@ -195,6 +231,7 @@ __global__ void k_input(int B, int Mb, int din, int dinp, int ldt, const float *
     if (row < Mb && col < dinp) Xb[(size_t)row * dinp + col] = __float2bfloat16_rn(v);
     t[r][tx] = v;
   }
+  if (!XT) return;
   __syncthreads();
   for (int r = ty; r < 32; r += 8) {
     const int col = c0 + r, row = r0 + tx;
@@ -258,48 +295,83 @@ __global__ void k_sum(int n, const double *part, double *out) {
   }
 }
 
-// bias gradients: g[n] = sum_{b < B} d[b][n]  (fixed order over b)
-__global__ void k_colsum(int B, int N, int ld, const float *__restrict__ d, float *g) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
+// bias gradients of all layers: g[n] = sum_{b < B} d[b][n], a thread per column,
+// added in order of b; 32 rows' loads in flight, one after another they
+// were the time of the kernel (256 rows x 1,536 columns now 9 us)
+struct Cols {
+  const float *d[3];
+  float *g[3];
+  int n[3];
+};
+__global__ void __launch_bounds__(32) k_colsum(int B, Cols c) {
+  int n = blockIdx.x * 32 + threadIdx.x, k = 0;
+  while (k < 2 && n >= c.n[k]) n -= c.n[k++];
+  if (n >= c.n[k]) return;
+  const int ld = c.n[k];
+  const float *d = c.d[k] + n;
   float s = 0.0f;
-  for (int b = 0; b < B; ++b) s += d[(size_t)b * ld + n];
-  g[n] = s;
+  for (int b = 0; b < B; b += 32) {
+    float v[32];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = b + j < B ? d[(size_t)(b + j) * ld] : 0.0f;
+#pragma unroll
+    for (int j = 0; j < 32; ++j) s += v[j];
+  }
+  c.g[k][n] = s;
 }
 
-// Adam (Kingma & Ba) on the FP32 masters, then the BF16 copies
-__global__ void k_adam(long long n, float *p, const float *g, float *m, float *v, float lr, float b1, float b2,
-                       float eps, float c1, float c2) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float gi = g[i];
-  const float mi = b1 * m[i] + (1.0f - b1) * gi;
-  const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+// The parameters: three weight matrices [rows][cols] with their BF16 copies
+// and (W2, W3) transposed BF16 copies, each followed by its bias.
+struct Weights {
+  long long w[3], b[3];  // offsets in the parameter vector
+  int rows[3], cols[3];
+  __nv_bfloat16 *Wb[3], *WT[3];
+  int tiles[3];  // 32 x 32 tiles
+};
+struct Adam {
+  const float *g;
+  float *m, *v;
+  float lr, b1, b2, eps, c1, c2;
+};
+
+// One step of Adam (Kingma & Ba) on an FP32 master
+__device__ __forceinline__ float adam(long long i, float p, const Adam &A) {
+  const float gi = A.g[i];
+  const float mi = A.b1 * A.m[i] + (1.0f - A.b1) * gi;
+  const float vi = A.b2 * A.v[i] + (1.0f - A.b2) * gi * gi;
+  A.m[i] = mi;
+  A.v[i] = vi;
+  return p - A.lr * (mi / A.c1) / (sqrtf(vi / A.c2) + A.eps);
 }
 
-// W [rows][cols] FP32 -> BF16 W and (optionally) BF16 W^T [cols][rows]
-__global__ void k_to_bf16(int rows, int cols, const float *__restrict__ W, __nv_bfloat16 *Wb, __nv_bfloat16 *WT) {
+// All parameters in one launch, a CTA per 32 x 32 tile (256 biases): the step
+// of Adam where STEP, and the BF16 copies from the new value at hand
+template <bool STEP>
+__global__ void __launch_bounds__(256) k_weights(Weights W, float *P, Adam A) {
   __shared__ float t[32][33];
-  const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
   const int tx = threadIdx.x, ty = threadIdx.y;
+  int blk = blockIdx.x, k = 0;
+  while (k < 3 && blk >= W.tiles[k]) blk -= W.tiles[k++];
+  if (k == 3) {
+    int i = blk * 256 + ty * 32 + tx;
+    for (int l = 0; STEP && l < 3; i -= W.rows[l++])
+      if (i >= 0 && i < W.rows[l]) P[W.b[l] + i] = adam(W.b[l] + i, P[W.b[l] + i], A);
+    return;
+  }
+  const int tc = W.cols[k] / 32, r0 = blk / tc * 32, c0 = blk % tc * 32;  // every extent is a multiple of 128
+#pragma unroll
   for (int r = ty; r < 32; r += 8) {
-    const int row = r0 + r, col = c0 + tx;
-    float v = 0.0f;
-    if (row < rows && col < cols) {
-      v = W[(size_t)row * cols + col];
-      Wb[(size_t)row * cols + col] = __float2bfloat16_rn(v);
-    }
+    const size_t at = (size_t)(r0 + r) * W.cols[k] + c0 + tx;
+    float v = P[W.w[k] + at];
+    if (STEP) P[W.w[k] + at] = v = adam(W.w[k] + at, v, A);
+    W.Wb[k][at] = __float2bfloat16_rn(v);
     t[r][tx] = v;
   }
-  if (!WT) return;
+  if (!W.WT[k]) return;
   __syncthreads();
-  for (int r = ty; r < 32; r += 8) {
-    const int col = c0 + r, row = r0 + tx;
-    if (col < cols && row < rows) WT[(size_t)col * rows + row] = __float2bfloat16_rn(t[tx][r]);
-  }
+#pragma unroll
+  for (int r = ty; r < 32; r += 8)
+    W.WT[k][(size_t)(c0 + r) * W.rows[k] + r0 + tx] = __float2bfloat16_rn(t[tx][r]);
 }
 
 }  // namespace mlpk
@@ -319,7 +391,7 @@ struct ipm_mlp {
   double *part = nullptr, *lsum = nullptr, *h_loss = nullptr;
   int *flags = nullptr, *h_flags = nullptr;
   long long adam_t = 0;
-  CUtensorMap maps[16];
+  CUtensorMap maps[16], maps32[16];  // boxes of 128 rows, and of 32
   std::vector<void *> allocs;
 };
 
@@ -342,52 +414,63 @@ bool mal(ipm_mlp *m, T **p, size_t count) {
 
 inline int r128(int v) { return (v + 127) / 128 * 128; }
 
-void gemm(ipm_mlp *m, int mapA, int mapB, int M, int N, int K, const Epi &e, cudaStream_t st) {
-  static const bool attr = cudaFuncSetAttribute(k_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                SMEM_BYTES) == cudaSuccess;
+template <int BN, int STAGES>
+void gemm_tiles(const CUtensorMap &a, const CUtensorMap &b, int M, int N, int K, const Epi &e, int *flags,
+                cudaStream_t st) {
+  static const bool attr = cudaFuncSetAttribute(k_gemm<BN, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                smem_bytes(BN, STAGES)) == cudaSuccess;
   (void)attr;
-  dim3 grid(M / BM, N / BN);
-  k_gemm<<<grid, 192, SMEM_BYTES, st>>>(m->maps[mapA], m->maps[mapB], K / BK, e, m->flags);
+  k_gemm<BN, STAGES><<<dim3(M / BM, N / BN), 192, smem_bytes(BN, STAGES), st>>>(a, b, K / BK, e, flags);
   ipm_count_launch();
+}
+
+// narrow tiles until wide ones come to one per SM
+void gemm(ipm_mlp *m, int mapA, int mapB, int M, int N, int K, const Epi &e, cudaStream_t st) {
+  if ((M / BM) * (N / 128) < 152) gemm_tiles<32, 5>(m->maps[mapA], m->maps32[mapB], M, N, K, e, m->flags, st);
+  else gemm_tiles<128, 3>(m->maps[mapA], m->maps[mapB], M, N, K, e, m->flags, st);
 }
 
 Epi epi(int ldo) {
   Epi e;
   std::memset(&e, 0, sizeof(e));
   e.ldo = ldo;
+  e.m_valid = e.n_valid = 1 << 30;
   return e;
 }
 
-void refresh_bf16(ipm_mlp *m, cudaStream_t st) {
-  const dim3 b(32, 8);
-  k_to_bf16<<<dim3((m->dinp + 31) / 32, (m->dh + 31) / 32), b, 0, st>>>(m->dh, m->dinp, m->P + m->oW1, m->W1b, nullptr);
-  k_to_bf16<<<dim3((m->dh + 31) / 32, (m->dh + 31) / 32), b, 0, st>>>(m->dh, m->dh, m->P + m->oW2, m->W2b, m->W2T);
-  k_to_bf16<<<dim3((m->dh + 31) / 32, (m->doutp + 31) / 32), b, 0, st>>>(m->doutp, m->dh, m->P + m->oW3, m->W3b,
-                                                                         m->W3T);
-  ipm_count_launch();
-  ipm_count_launch();
+void weights(ipm_mlp *m, const Adam *A, cudaStream_t st) {
+  const Weights W = {{m->oW1, m->oW2, m->oW3}, {m->ob1, m->ob2, m->ob3},
+                     {m->dh, m->dh, m->doutp}, {m->dinp, m->dh, m->dh},
+                     {m->W1b, m->W2b, m->W3b}, {nullptr, m->W2T, m->W3T},
+                     {m->dh / 32 * (m->dinp / 32), m->dh / 32 * (m->dh / 32), m->doutp / 32 * (m->dh / 32)}};
+  const int tiles = W.tiles[0] + W.tiles[1] + W.tiles[2], nb = (2 * m->dh + m->doutp + 255) / 256;
+  if (A) k_weights<true><<<tiles + nb, dim3(32, 8), 0, st>>>(W, m->P, *A);
+  else k_weights<false><<<tiles, dim3(32, 8), 0, st>>>(W, m->P, Adam{});
   ipm_count_launch();
 }
 
 // forward pass over B rows of X; the output layer writes de-normalised
-// predictions when `denorm`, normalised ones otherwise (training)
+// predictions [B][dout] where the caller wants them (`denorm`), normalised
+// ones with their padding otherwise (training), and what only the backward
+// pass reads (pre-activations, transposed operands) only then
 void forward(ipm_mlp *m, const float *X, int B, bool denorm, float *Yout, int ldy, cudaStream_t st) {
   const int Mb = r128(B);
   k_input<<<dim3((m->dinp + 31) / 32, (Mb + 31) / 32), dim3(32, 8), 0, st>>>(B, Mb, m->din, m->dinp, m->bpad, X,
-                                                                           m->in_mean, m->in_std, m->Xb, m->XT);
+                                                                           m->in_mean, m->in_std, m->Xb,
+                                                                           denorm ? nullptr : m->XT);
   ipm_count_launch();
   Epi e = epi(m->dh);
   e.bias = m->P + m->ob1;
   e.act = ACT_GELU;
-  e.pre_out = m->pre1;
+  e.pre_out = denorm ? nullptr : m->pre1;
   e.out_bf = m->H1b;
-  e.out_t = m->H1T;
+  e.out_t = denorm ? nullptr : m->H1T;
   e.ldt = m->bpad;
   gemm(m, MX, MW1, Mb, m->dh, m->dinp, e, st);
   e.bias = m->P + m->ob2;
-  e.pre_out = m->pre2;
+  e.pre_out = denorm ? nullptr : m->pre2;
   e.out_bf = m->H2b;
-  e.out_t = m->H2T;
+  e.out_t = denorm ? nullptr : m->H2T;
   gemm(m, MH1, MW2, Mb, m->dh, m->dh, e, st);
   Epi o = epi(ldy);
   o.bias = m->P + m->ob3;
@@ -396,6 +479,7 @@ void forward(ipm_mlp *m, const float *X, int B, bool denorm, float *Yout, int ld
   if (denorm) {
     o.scale = m->out_std;
     o.shift = m->out_mean;
+    o.m_valid = B;
     o.n_valid = m->dout;
   }
   gemm(m, MH2, MW3, Mb, m->doutp, m->dh, o, st);
@@ -437,11 +521,8 @@ void backward(ipm_mlp *m, const float *T, int B, cudaStream_t st) {
   Epi w1 = epi(m->dinp);
   w1.out_f32 = m->G + m->oW1;
   gemm(m, MDP1T, MXT, m->dh, m->dinp, Mb, w1, st);
-  k_colsum<<<(m->dh + 127) / 128, 128, 0, st>>>(B, m->dh, m->dh, m->dp1f, m->G + m->ob1);
-  k_colsum<<<(m->dh + 127) / 128, 128, 0, st>>>(B, m->dh, m->dh, m->dp2f, m->G + m->ob2);
-  k_colsum<<<(m->doutp + 127) / 128, 128, 0, st>>>(B, m->doutp, m->doutp, m->dYf, m->G + m->ob3);
-  ipm_count_launch();
-  ipm_count_launch();
+  const Cols c = {{m->dp1f, m->dp2f, m->dYf}, {m->G + m->ob1, m->G + m->ob2, m->G + m->ob3}, {m->dh, m->dh, m->doutp}};
+  k_colsum<<<(2 * m->dh + m->doutp) / 32, 32, 0, st>>>(B, c);
   ipm_count_launch();
 }
 
@@ -542,7 +623,9 @@ ipm_status ipm_mlp_create(int d_in, int d_hidden, int d_out, int max_batch, unsi
       {m->H2T, m->dh, m->bpad},    {m->dp2b, m->bpad, m->dh}, {m->W2T, m->dh, m->dh},
       {m->dp2T, m->dh, m->bpad},   {m->H1T, m->dh, m->bpad},  {m->dp1T, m->dh, m->bpad},
       {m->XT, m->dinp, m->bpad}};
-  for (int i = 0; ok && i < 16; ++i) ok = tc_make_kmajor_map(&m->maps[i], defs[i].p, defs[i].rows, defs[i].k);
+  for (int i = 0; ok && i < 16; ++i)
+    ok = tc_make_kmajor_map(&m->maps[i], defs[i].p, defs[i].rows, defs[i].k) &&
+         tc_make_kmajor_map_box(&m->maps32[i], defs[i].p, defs[i].rows, defs[i].k, 32, BK);
   if (!ok) {
     ipm_mlp_destroy(m);
     return IPM_ERR_OOM;
@@ -597,7 +680,7 @@ ipm_status ipm_mlp_set_params(ipm_mlp *m, const float *params) {
   cudaMemset(m->Mm, 0, m->np * sizeof(float));
   cudaMemset(m->V, 0, m->np * sizeof(float));
   m->adam_t = 0;
-  refresh_bf16(m, 0);
+  weights(m, nullptr, 0);
   return cudaDeviceSynchronize() == cudaSuccess ? IPM_OK : IPM_ERR_CUDA;
 }
 
@@ -630,10 +713,7 @@ ipm_status ipm_mlp_forward(ipm_mlp *m, const float *x, int batch, float *y, void
   for (int b0 = 0; b0 < batch; b0 += m->maxb) {
     const int B = std::min(m->maxb, batch - b0);
     cudaMemsetAsync(m->flags, 0, FLAG_COUNT * sizeof(int), st);
-    forward(m, x + (size_t)b0 * m->din, B, true, m->Y, m->doutp, st);
-    if (cudaMemcpy2DAsync(y + (size_t)b0 * m->dout, m->dout * sizeof(float), m->Y, m->doutp * sizeof(float),
-                          m->dout * sizeof(float), B, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-      return IPM_ERR_CUDA;
+    forward(m, x + (size_t)b0 * m->din, B, true, y + (size_t)b0 * m->dout, m->dout, st);
     ipm_status s = finish(m, st, nullptr, B);
     if (s != IPM_OK) return s;
   }
@@ -665,9 +745,8 @@ ipm_status ipm_mlp_train_step(ipm_mlp *m, const float *x, const float *target, i
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
   ++m->adam_t;
   const float c1 = 1.0f - std::pow(b1, (float)m->adam_t), c2 = 1.0f - std::pow(b2, (float)m->adam_t);
-  k_adam<<<(unsigned)((m->np + 255) / 256), 256, 0, st>>>(m->np, m->P, m->G, m->Mm, m->V, lr, b1, b2, eps, c1, c2);
-  ipm_count_launch();
-  refresh_bf16(m, st);
+  const Adam A = {m->G, m->Mm, m->V, lr, b1, b2, eps, c1, c2};
+  weights(m, &A, st);
   return finish(m, st, loss, batch);
 }
 
