@@ -88,8 +88,8 @@ struct ipm_ctx {
   double *Hp = nullptr, *kpx = nullptr, *kpu = nullptr, *vpos = nullptr, *bpos = nullptr, *apos = nullptr;
   double *xt = nullptr, *ut = nullptr, *st = nullptr, *gt = nullptr, *ht = nullptr, *fst = nullptr,
          *Pt = nullptr, *Qt = nullptr;
-  double *red_partial = nullptr, *red_out = nullptr;
-  double *h_red = nullptr;  // pinned host mirror of reduction outputs
+  double *red_partial = nullptr, *red_out = nullptr;  // red_out: h_red as the kernels see it
+  double *h_red = nullptr;  // pinned host memory, written by the reductions (first 8)
   int *h_flags = nullptr;
   int nL = 0;
   long long n_bounds = 0;
