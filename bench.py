@@ -45,8 +45,7 @@ FP64_PEAK_TFLOPS = 1.25
 FP32_PEAK_TFLOPS = 80.5
 # DRAM bytes per launch from one ncu capture of the kernel as it stands (profiles/); None once the
 # kernel changes until it is captured again.
-TRAFFIC = {"k_gemm_tn64": 590.125568e6 + 25.997568e6,   # DRAM read + write, one launch, 1000 buses x 64
-           "k_zsolve64": 1.691865e9 + 865.253632e6,
+TRAFFIC = {"k_zsolve64": 2.7258e9,   # DRAM read + write, one launch, 1000 buses x 64
            "k_emu_schur": 1.137726e9 + 3.871488e6}
 UNIT = "scenario condensations/s"
 REF_BUDGET_S = 150.0  # timed host seconds of the reference arm on the 10,000-bus workload
@@ -168,8 +167,8 @@ def roofline(phases, dims, peaks, peak_kind, precision):
         # one vector per scenario through G_x or G_x^T: the factor read once, the vector in and out
         byt = 8.0 * (dims.nnz_lu + 2 * nx) * N
         ach = byt / per_call_s / 1e9
-        return {"kernel": "k_solve1 + k_trsv_first/k_trsv_step (single-vector FP64 solves: sparse levels in "
-                          "one CTA per scenario, the dense trailing block by multi-CTA sweeps)",
+        return {"kernel": "k_solve1 (single-vector FP64 solves: sparse levels and the dense trailing block by "
+                          "one CTA per scenario, or a cluster of them with a large block)",
                 "bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": ach / peaks["hbm_gbs"], "traffic": None,
                 "algorithmic": f"{byt:.4g} B/solve (the LU factors once, the vector in and out)",
@@ -178,7 +177,7 @@ def roofline(phases, dims, peaks, peak_kind, precision):
         # sparse eliminations (one FMA each) and, with a dense trailing block, its LU (2/3 nd^3)
         flops = (2.0 * dims.lu_sparse_ops + (2.0 / 3.0) * dims.nd ** 3) * N
         ach = flops / per_call_s / 1e12
-        return {"kernel": "k_lu_factor + trailing-block LU (k_blu_*; FP64-grade tensor-core updates on the "
+        return {"kernel": "k_lu_sparse + trailing-block LU (k_blu_*; FP64-grade tensor-core updates on the "
                           "mixed and FP64_TC paths)" if dims.big_block else "k_lu_factor_pair",
                 "bound": "alu", "achieved": ach, "peak": fp64_peak, "unit": "TFLOP/s", "frac": ach / fp64_peak,
                 "traffic": None, "algorithmic": f"{flops:.4g} FP64 flop/launch"}
