@@ -37,6 +37,7 @@ struct DevSym {
   const int2 *sw_item, *sw_extra;
   const int *sw_row, *swf_lev, *swb_lev;
   int swf_n, swb_n;
+  int ordered;  // small problems: every sum in one fixed order (ipm_internal.h)
   size_t sw_items;  // items of one direction (the transposed ones follow)
   double *dinv;
   const int *gu_ptr, *gu_col, *gu_src, *gut_ptr, *gut_col, *gut_src;
@@ -106,6 +107,24 @@ __device__ __forceinline__ double rcp_newton(double d) {
 __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   return v;
+}
+// term(0) + term(1) + ... over the N scenarios by a warp, the terms of 32
+// scenarios side by side; the sum is lane 0's.  In index order with S.ordered
+// (the rounding of a loop over them), else by lanes and a fixed tree.
+template <class Term>
+__device__ __forceinline__ double scenario_sum(const DevSym &S, Term term) {
+  const int lane = threadIdx.x & 31;
+  double acc = 0.0;
+  if (S.ordered) {
+    for (int s0 = 0; s0 < S.N; s0 += 32) {
+      const double v = s0 + lane < S.N ? term(s0 + lane) : 0.0;
+      const int n = min(32, S.N - s0);
+      for (int j = 0; j < n; ++j) acc += __shfl_sync(0xffffffffu, v, j);
+    }
+    return acc;
+  }
+  for (int sc = lane; sc < S.N; sc += 32) acc += term(sc);
+  return warp_sum(acc);
 }
 __device__ __forceinline__ double warp_max(double v) {
   for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));

@@ -128,6 +128,7 @@ ipm_status upload_symbolic(ipm_ctx *c, const HostNet &net, const double *pd, con
     TRY(upload(c, &q, S.sw_extra)); d.sw_extra = reinterpret_cast<const int2 *>(q);
   }
   d.sw_items = S.sw_item.size() / 4;
+  d.ordered = S.ordered ? 1 : 0;
   TRY(upload(c, &d.sw_row, S.sw_row)); TRY(upload(c, &d.swf_lev, S.swf_lev)); TRY(upload(c, &d.swb_lev, S.swb_lev));
   d.swf_n = (int)S.swf_lev.size() - 1;
   d.swb_n = (int)S.swb_lev.size() - 1;
@@ -309,9 +310,12 @@ ipm_status alloc_work(ipm_ctx *c) {
   // diagonal and the ragged edge do less work, and more waves level that out
   // (1,000 buses x 64, assembly included: one wave 12.1 ms, two 11.4, three
   // 10.9, four 10.6)
+  // Where chunks of 64 rows would not fill one wave, one wave of chunks of at
+  // least 16 rows (products and assembly, 30 buses x 1: 14 us, with one chunk
+  // 39; 120 x 17: 22 + 31, with chunks of 64 rows 38 + 15).
   {
     const long long G0 = std::max(1, (3 * 152) / c->ntiles);
-    set_groups(c, 4 * G0);
+    set_groups(c, (long long)S.N * S.nx <= 64 * G0 ? G0 : 4 * G0);
     c->max_groups = c->ngroups;
   }
   {
@@ -568,9 +572,7 @@ void fp64_contraction(ipm_ctx *c, cudaStream_t st) {
 // split the N*nx contraction rows into at most G chunks (a multiple of 16 rows each)
 void set_groups(ipm_ctx *c, long long G) {
   const long long krows = (long long)c->S.N * c->S.nx;
-  // at least 64 rows to a chunk: the small problems' tile sums (a thread per
-  // entry walks the chunks) cost more than their products otherwise
-  G = std::max(1LL, std::min(G, (krows + 63) / 64));
+  G = std::max(1LL, std::min(G, (krows + 15) / 16));
   long long kc = (krows + G - 1) / G;
   kc = (kc + 15) / 16 * 16;
   c->kchunk = kc;

@@ -8,6 +8,15 @@
 // lists of trailing-block products of the LU factorization: one per thread of
 // a cluster of two CTAs, or of eight with a large trailing block
 constexpr int LU_LISTS = 1024, LU_LISTS_BIG = 4096;
+// The largest problems whose sums keep one fixed order (Sym::ordered): whole
+// solves of small networks are compared to the ninth digit of the whole state,
+// and rho, raised by a quotient of differences at rounding level, does not keep
+// nine digits under another order.  Up to here it costs nothing (an iteration
+// of 30 buses x 1 781 us, with the shortest chain for each kernel 807; a solve
+// of 120 x 17 17.1 ms, 17.0).  At 433 x 19 a single-vector solve would take
+// 144 us instead of 55, and with 60 scenarios of 213 buses the sums and solves
+// 115 instead of 70.
+constexpr int ORDERED_NX = 400, ORDERED_N = 32;
 
 struct HostNet {
   int n = 0, L = 0, ng = 0;
@@ -81,11 +90,18 @@ struct Sym {
   // sw_item[2 ((4 u + h) 32 + l)], slot -1 for none; the same with the
   // transposed slots follows (second half).  sw_row[32 u + l]: the lane's row
   // and, from bit 26, the unit's code, -1 for no row; a row takes
-  // 2^(code & 7) neighbouring lanes.  Rows of more than 128 products (code &
+  // 2^(code & 7) neighbouring lanes.  Rows with products left over (code &
   // 8) go on in the units sw_extra[2 u] = {first, count}.  Units of level l:
   // swf_lev[l] .. swf_lev[l + 1] (forward: the sparse levels, then one more
   // for the sparse part of the trailing rows), swb_lev for the backward rows.
+  // With `ordered` a row takes 4 lanes (forward sparse rows) or 8 (trailing
+  // and backward rows) whatever its length, product f in lane f mod 4 or 8,
+  // several rows to a unit that goes on in sw_extra.
   std::vector<int> sw_item, sw_row, sw_extra, swf_lev, swb_lev;
+  // Small problems: every sum in one fixed order that no choice of lanes or
+  // launch shapes changes (the single-vector sweeps, the sums over the
+  // scenarios, the products with K).
+  bool ordered = false;
   // sparse operators by position (x rows) or u rows
   std::vector<int> gu_ptr, gu_col, gu_src;
   std::vector<int> gut_ptr, gut_col, gut_src;

@@ -121,9 +121,16 @@ __global__ void k_khat_assemble(int nu, int N, int ngroups, int ntiles, int nt1,
   if (i > j) return;
   const int ti = i / TB, tj = j / TB;
   const int tt = tile_of[ti * nt1 + tj];
+  const double *p = partial + (size_t)tt * TB * TB + (i - ti * TB) * TB + (j - tj * TB);
+  const size_t st = (size_t)ntiles * TB * TB;
   double v = 0.0;
-  for (int g = 0; g < ngroups; ++g)
-    v += partial[((size_t)g * ntiles + tt) * TB * TB + (i - ti * TB) * TB + (j - tj * TB)];
+  for (int g0 = 0; g0 < ngroups; g0 += 16) {  // added in order, the loads of 16 chunks in flight
+    double a[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) a[q] = g0 + q < ngroups ? p[(g0 + q) * st] : 0.0;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) v += a[q];
+  }
   if (Yu)
     for (int s = 0; s < N; ++s) v += Yu[(size_t)s * nu * nu + (size_t)i * nu + j];
   if (diag && i == j) v += diag[i];
@@ -158,19 +165,52 @@ __global__ void k_maxdiag(int n, const double *A, double *out) {
 }
 
 constexpr int CB = 32;  // Cholesky block
+constexpr int CHOL_SMALL = 64;  // rows of K_hat of the small problems (ipm_internal.h) with 15 % generators
 
 // factor the CB x CB diagonal block at (k0, k0) in place (lower), unblocked
 
 // Right-looking Cholesky of the nb x nb block a (lower part, in shared
-// memory) by the calling CTA, as L D L^T with the square roots taken for all
-// columns at the end: only a reciprocal is on the chain from pivot to pivot.
-// Warps 0-3 update the trailing columns (warp w: columns j = w mod 4; lane =
-// row; column entries by shuffles), the next column first, whose pivot's
-// reciprocal is formed under the others' updates; one barrier per column.  A
+// memory) by the calling CTA: thread 0 takes each pivot's reciprocal square
+// root, then warps 0-3 scale the column and update the trailing columns
+// (warp w: columns j = w mod 4; lane = row; column entries by shuffles).  A
 // non-positive or non-finite pivot raises FLAG_NOT_PD and is replaced by 1.
-// Latency-bound; the whole factorization at n_u = 299 412 -> 391 us, 899
-// 1,275 -> 1,215.
-__device__ void potrf_block(int nb, int *flags, double (*a)[CB + 1], double *rs_sh) {
+// For K_hat of at most CHOL_SMALL rows, the small problems, whose whole solves
+// keep these operations (ipm_internal.h).
+__device__ void potrf_plain(int nb, int *flags, double (*a)[CB + 1], double *rs_sh) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int k = 0; k < nb; ++k) {
+    if (tid == 0) {
+      double d = a[k][k];
+      if (!(d > 0.0) || !isfinite(d)) {
+        flags[FLAG_NOT_PD] = 1;
+        d = 1.0;
+      }
+      const double rs = rsqrt_newton(d);
+      *rs_sh = rs;
+      a[k][k] = d * rs;
+    }
+    __syncthreads();
+    double lik = 0.0;
+    if (warp < 4) {
+      lik = (lane > k && lane < nb) ? a[lane][k] * *rs_sh : 0.0;
+      for (int j = k + 1 + ((warp - (k + 1)) & 3); j < nb; j += 4) {
+        const double ljk = __shfl_sync(0xffffffffu, lik, j);
+        if (lane >= j && lane < nb) a[lane][j] -= lik * ljk;
+      }
+    }
+    __syncthreads();
+    // column k is read by no later step: written after the barrier
+    if (warp == 0 && lane > k && lane < nb) a[lane][k] = lik;
+  }
+  __syncthreads();
+}
+
+// The same as L D L^T with the square roots taken for all columns at the end:
+// only a reciprocal is on the chain from pivot to pivot, formed for the next
+// column, which is updated first, under the others' updates; one barrier per
+// column.  Latency-bound; the whole factorization at n_u = 299 412 -> 391 us,
+// 899 1,275 -> 1,215.
+__device__ void potrf_ldl(int nb, int *flags, double (*a)[CB + 1], double *rs_sh) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const auto pivot = [&](int k) {
     double d = a[k][k];
@@ -205,13 +245,21 @@ __device__ void potrf_block(int nb, int *flags, double (*a)[CB + 1], double *rs_
   __syncthreads();
 }
 
+// (rs_sh: 2 + CB doubles)
+template <bool LDL>
+__device__ __forceinline__ void potrf_block(int nb, int *flags, double (*a)[CB + 1], double *rs_sh) {
+  if (LDL) potrf_ldl(nb, flags, a, rs_sh);
+  else potrf_plain(nb, flags, a, rs_sh);
+}
+
 // Load, factor and store the diagonal block at (k0, k0) (upper part of the
 // block set to zero).
+template <bool LDL>
 __device__ void potrf_tile(int n, int k0, double *A, int *flags, double (*a)[CB + 1], double *rs_sh) {
   const int nb = min(CB, n - k0), tid = threadIdx.x;
   for (int e = tid; e < nb * nb; e += blockDim.x) a[e / nb][e % nb] = A[(size_t)(k0 + e / nb) * n + k0 + e % nb];
   __syncthreads();
-  potrf_block(nb, flags, a, rs_sh);
+  potrf_block<LDL>(nb, flags, a, rs_sh);
   for (int e = tid; e < nb * nb; e += blockDim.x) {
     const int i = e / nb, j = e % nb;
     A[(size_t)(k0 + i) * n + k0 + j] = (j <= i) ? a[i][j] : 0.0;
@@ -219,10 +267,11 @@ __device__ void potrf_tile(int n, int k0, double *A, int *flags, double (*a)[CB 
   __syncthreads();
 }
 
+template <bool LDL>
 __global__ void k_potrf_diag(int n, int k0, double *A, int *flags) {
   __shared__ double a[CB][CB + 1];
   __shared__ double rs_sh[2 + CB];
-  potrf_tile(n, k0, A, flags, a, rs_sh);
+  potrf_tile<LDL>(n, k0, A, flags, a, rs_sh);
 }
 
 // rows below the diagonal block: L_ik = A_ik L_kk^{-T}
@@ -302,12 +351,13 @@ __device__ void syrk_tile16(int n, int k0, int nb, int i0, int j0, double *A, do
   }
 }
 
+template <bool LDL>
 __global__ void __launch_bounds__(256) k_chol_coop(int n, double *A, int *flags) {
   cooperative_groups::grid_group grid = cooperative_groups::this_grid();
   __shared__ double a[CB][CB + 1], b2[CB][CB + 1];
   __shared__ double rinv[CB], rs_sh[2 + CB];
   const int G = gridDim.x, bk = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (bk == 0) potrf_tile(n, 0, A, flags, a, rs_sh);
+  if (bk == 0) potrf_tile<LDL>(n, 0, A, flags, a, rs_sh);
   grid.sync();
   for (int k0 = 0; k0 < n; k0 += CB) {
     const int nb = min(CB, n - k0), r0 = k0 + nb, rest = n - r0;
@@ -371,7 +421,7 @@ __global__ void __launch_bounds__(256) k_chol_coop(int n, double *A, int *flags)
         a[i][j] = A[(size_t)(r0 + i) * n + r0 + j] - ((s0 + s1) + (s2 + s3));
       }
       __syncthreads();
-      potrf_block(nb2, flags, a, rs_sh);
+      potrf_block<LDL>(nb2, flags, a, rs_sh);
       for (int e = tid; e < nb2 * nb2; e += blockDim.x) {
         const int i = e / nb2, j = e % nb2;
         A[(size_t)(r0 + i) * n + r0 + j] = (j <= i) ? a[i][j] : 0.0;
@@ -434,6 +484,59 @@ __global__ void __launch_bounds__(TH) k_chol_solve(int n, const double *__restri
   }
   trsv::sweep<TH, NB, MULTI>(L, (size_t)n, n, true, false, inv, NB * NB, C, rank, smc, ldx, stx);
   trsv::sweep<TH, NB, MULTI>(L, (size_t)n, n, false, true, inv, NB * NB, C, rank, smc, ldx, stx);
+}
+
+// The same for few rows, one CTA with the vector in shared memory: the
+// diagonal blocks step by step by one warp (lane = row, reciprocal pivots
+// formed by all lanes at once), the rows past a block by a thread each with
+// four partial sums: the order of operations of the small problems' whole
+// solves (ipm_internal.h).  n_u = 35 14 us and 63 22, against 7 and 7 by the
+// inverses, which take 12 to form once per factorization.
+__global__ void __launch_bounds__(128) k_chol_solve_small(int n, const double *__restrict__ L, double *b) {
+  __shared__ double x[CHOL_SMALL], blk[32][33];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid < n) x[tid] = b[tid];
+  __syncthreads();
+  const auto sweep = [&](bool up) {
+    for (int s = 0; s < n; s += 32) {
+      const int kb = up ? (n - 1) / 32 * 32 - s : s, w = min(32, n - kb);
+      for (int e = tid; e < 32 * w; e += 128) {
+        const int r = e >> 5, c = e & 31;
+        blk[r][c] = c <= r ? L[(size_t)(kb + r) * n + kb + c] : 0.0;
+      }
+      __syncthreads();
+      if (warp == 0) {
+        const double ri = lane < w ? 1.0 / blk[lane][lane] : 0.0;
+        double v = lane < w ? x[kb + lane] : 0.0;
+        for (int q = 0; q < w; ++q) {
+          const int k = up ? w - 1 - q : q;
+          if (lane == k) v *= ri;
+          const double xk = __shfl_sync(0xffffffffu, v, k);
+          if (up ? lane < k : lane > k && lane < w) v -= (up ? blk[k][lane] : blk[lane][k]) * xk;
+        }
+        if (lane < w) x[kb + lane] = v;
+      }
+      __syncthreads();
+      if (up ? tid < kb : tid >= kb + w && tid < n) {
+        const double *p = up ? L + (size_t)kb * n + tid : L + (size_t)tid * n + kb;
+        const size_t st = up ? n : 1;
+        double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+        int j = 0;
+        for (; j + 4 <= w; j += 4) {
+          s0 = fma(p[j * st], x[kb + j], s0);
+          s1 = fma(p[(j + 1) * st], x[kb + j + 1], s1);
+          s2 = fma(p[(j + 2) * st], x[kb + j + 2], s2);
+          s3 = fma(p[(j + 3) * st], x[kb + j + 3], s3);
+        }
+        for (; j < w; ++j) s0 = fma(p[j * st], x[kb + j], s0);
+        x[tid] -= (s0 + s1) + (s2 + s3);
+      }
+      __syncthreads();
+    }
+  };
+  sweep(false);
+  sweep(true);
+  if (tid < n) b[tid] = x[tid];
 }
 
 // diagonal blocks of 64 rows from here on
@@ -514,14 +617,15 @@ void launch_shift(int nu, const double *Khat, const double *M, double delta, dou
 void launch_maxdiag(int n, const double *A, double *out, cudaStream_t st) {
   k_maxdiag<<<1, 256, 0, st>>>(n, A, out); ipm_count_launch();
 }
-void launch_cholesky(int n, double *A, int *flags, cudaStream_t st) {
+template <bool LDL>
+static void cholesky(int n, double *A, int *flags, cudaStream_t st) {
   // one cooperative launch when the device allows it (all CTAs resident)
   static const int coop_ctas = [] {
     int dev = 0, ok = 0, sms = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&ok, cudaDevAttrCooperativeLaunch, dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (!ok || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_chol_coop, 256, 0) != cudaSuccess || per < 1)
+    if (!ok || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_chol_coop<LDL>, 256, 0) != cudaSuccess || per < 1)
       return 0;
     return sms;  // one CTA per SM
   }();
@@ -531,14 +635,14 @@ void launch_cholesky(int n, double *A, int *flags, cudaStream_t st) {
     G = G < coop_ctas ? G : coop_ctas;
     if (G < 1) G = 1;
     void *args[] = {(void *)&n, (void *)&A, (void *)&flags};
-    if (cudaLaunchCooperativeKernel((const void *)k_chol_coop, dim3(G), dim3(256), args, 0, st) == cudaSuccess) {
+    if (cudaLaunchCooperativeKernel((const void *)k_chol_coop<LDL>, dim3(G), dim3(256), args, 0, st) == cudaSuccess) {
       ipm_count_launch();
       return;
     }
     cudaGetLastError();
   }
   for (int k0 = 0; k0 < n; k0 += CB) {
-    k_potrf_diag<<<1, 256, 0, st>>>(n, k0, A, flags); ipm_count_launch();
+    k_potrf_diag<LDL><<<1, 256, 0, st>>>(n, k0, A, flags); ipm_count_launch();
     const int nb = n - k0 < CB ? n - k0 : CB;
     const int rest = n - k0 - nb;
     if (rest > 0) {
@@ -548,8 +652,13 @@ void launch_cholesky(int n, double *A, int *flags, cudaStream_t st) {
     }
   }
 }
+void launch_cholesky(int n, double *A, int *flags, cudaStream_t st) {
+  if (n <= CHOL_SMALL) cholesky<false>(n, A, flags, st);
+  else cholesky<true>(n, A, flags, st);
+}
 size_t chol_inverse_doubles(int n) { return (size_t)((n + 63) / 64) * 64 * 64; }
 void launch_chol_inverse(int n, const double *L, double *inv, cudaStream_t st) {
+  if (n <= CHOL_SMALL) return;
   if (n < CHOL_NB64) chol_inverse<32>(n, L, inv, st);
   else chol_inverse<64>(n, L, inv, st);
 }
@@ -557,7 +666,10 @@ void launch_chol_inverse(int n, const double *L, double *inv, cudaStream_t st) {
 // blocks on the tiles are dealt to a cluster, although its barrier costs ten
 // of a CTA's.
 void launch_chol_solve(int n, const double *L, const double *inv, double *b, cudaStream_t st) {
-  if (n <= 128) chol_solve_single<128>(n, L, inv, b, st);
+  if (n <= CHOL_SMALL) {
+    k_chol_solve_small<<<1, 128, 0, st>>>(n, L, b);
+    ipm_count_launch();
+  } else if (n <= 128) chol_solve_single<128>(n, L, inv, b, st);
   else if (n < CHOL_NB64) chol_solve_cluster<256, 32, 4>(n, L, inv, b, st);
   else if (n <= 16384) chol_solve_cluster<512, 64, 8>(n, L, inv, b, st);
   else chol_solve_cluster<256, 64, 8>(n, L, inv, b, st);  // 256 accumulators per block and CTA

@@ -14,8 +14,6 @@
 // 2 (dP dP^T + dQ dQ^T + P d2P + Q d2Q) come from the same closed forms.
 #include <atomic>
 
-#include <initializer_list>
-
 #include "dev.cuh"
 #include "kernels.h"
 
@@ -113,42 +111,71 @@ __device__ __forceinline__ double lam_Q(const DevSym &S, const double *y, const 
   return q >= 0 ? y[(size_t)sc * S.nx + q] : z[(size_t)sc * S.m + S.gen_of_bus[k]];
 }
 
-// Sum over LN neighbouring lanes (LN a power of two).
-template <int LN>
-__device__ __forceinline__ double lanes_sum(double v) {
+// The incident lines of a bus, LN lanes per (bus, scenario): line(e, q)
+// returns the NT terms of line e, which are added to acc in the order of the
+// lines.  One lane where the pairs fill the GPU (coalesced over the
+// scenarios), eight on the smaller problems, where a bus's lines in turn (an
+// FP64 sine and cosine and ~100 dependent operations each) were the time of
+// the kernel: the lanes form the terms of eight lines side by side and only
+// the additions follow one another (functions +
+// derivatives, 30 buses x 1: 17 + 43 -> 7 + 14 us, 119 x 7: 19 + 77 -> 8 + 25).
+// The last NF of the NT sums take a second term of a line each, after the
+// first, where `second` is set (the terms of the flow rows).
+template <int NT>
+struct Terms {
+  double v[NT];
+};
+template <int LN, int NT, int NF, class Line>
+__device__ __forceinline__ Terms<NT> sum_lines(const DevSym &S, int i, bool on_t, bool second, Line line) {
+  Terms<NT> acc = {};
+  const int e0 = S.inc_ptr[i], deg = on_t ? S.inc_ptr[i + 1] - e0 : 0;
+  if constexpr (LN == 1) {
+    for (int e = e0; e < e0 + deg; ++e) {
+      const Terms<NT + NF> q = line(e);
 #pragma unroll
-  for (int o = LN / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+      for (int k = 0; k < NT; ++k) acc.v[k] += q.v[k];
+      if (NF > 0 && second)
+#pragma unroll
+        for (int k = 0; k < NF; ++k) acc.v[NT - NF + k] += q.v[NT + k];
+    }
+    return acc;
+  }
+  const int sub = threadIdx.x % LN;
+  const int most = (int)__reduce_max_sync(0xffffffffu, (unsigned)deg);  // of the warp's pairs
+  for (int b = 0; b < most; b += LN) {
+    Terms<NT + NF> q = {};
+    if (b + sub < deg) q = line(e0 + b + sub);
+    const int n = min(LN, most - b);
+    for (int j = 0; j < n; ++j) {
+#pragma unroll
+      for (int k = 0; k < NT; ++k) acc.v[k] += __shfl_sync(0xffffffffu, q.v[k], j, LN);
+      if (NF > 0 && second)
+#pragma unroll
+        for (int k = 0; k < NF; ++k) acc.v[NT - NF + k] += __shfl_sync(0xffffffffu, q.v[NT + k], j, LN);
+    }
+  }
+  return acc;
 }
 
-// LN lanes per (bus, scenario), each with every LN-th incident line: one
-// where the pairs fill the GPU (coalesced over the scenarios), eight on the
-// smaller problems, where a bus's lines in turn (an FP64 sine and cosine and
-// ~100 dependent operations each) were the time of the kernel (functions +
-// derivatives, 30 buses x 1: 17 + 43 -> 6 + 12 us, 119 x 7: 19 + 78 -> 7 + 23).
 template <int LN>
 __global__ void __launch_bounds__(128) k_functions(DevSym S, const double *__restrict__ x, const double *__restrict__ u,
                                                    double *P, double *Q, double *g, double *h, double *fs) {
   const int tl = blockIdx.x * blockDim.x + threadIdx.x, sub = tl % LN;
-  const bool on_t = tl / LN < S.n * S.N;  // whole warps reach the sums below
+  const bool on_t = tl / LN < S.n * S.N;  // whole warps reach the sums
   const int t = on_t ? tl / LN : 0, i = t / S.N, sc = t - i * S.N;
   const double thi = bus_theta(S, x, sc, i), vi = bus_v(S, x, u, sc, i);
-  double p = 0.0, q = 0.0;
-  const int e1 = on_t ? S.inc_ptr[i + 1] : 0;
-  for (int e = S.inc_ptr[i] + sub; e < e1; e += LN) {
+  const Terms<2> sum = sum_lines<LN, 2, 0>(S, i, on_t, false, [&](int e) {
     const int l = S.inc_line[e], k = S.inc_other[e];
     double sn, cs;
     sincos(thi - bus_theta(S, x, sc, k), &sn, &cs);
     LineEnd le;
     const double on = S.lon ? S.lon[(size_t)l * S.N + sc] : 1.0;  // 0: line out of service
     line_end(vi, bus_v(S, x, u, sc, k), cs, sn, on * S.lg[l], on * S.lb[l], on * S.lbh[l], le);
-    p += le.P;
-    q += le.Q;
     if (S.nflow) h[(size_t)sc * S.m + flow_row(S, l, i)] = le.P * le.P + le.Q * le.Q;
-  }
-  p = lanes_sum<LN>(p);
-  q = lanes_sum<LN>(q);
+    return Terms<2>{le.P, le.Q};
+  });
   if (!on_t || sub != 0) return;
+  const double p = sum.v[0], q = sum.v[1];
   const size_t bi = (size_t)sc * S.n + i;
   P[bi] = p;
   Q[bi] = q;
@@ -170,15 +197,14 @@ __global__ void __launch_bounds__(128) k_derivatives(DevSym S, const double *__r
                                                      const double *__restrict__ z, const double *__restrict__ h,
                                                      double *J, double *W, double *JTl, double *HF) {
   const int tl = blockIdx.x * blockDim.x + threadIdx.x, sub = tl % LN;
-  const bool on_t = tl / LN < S.n * S.N;  // whole warps reach the sums below
+  const bool on_t = tl / LN < S.n * S.N;  // whole warps reach the sums
   const int t = on_t ? tl / LN : 0, i = t / S.N, sc = t - i * S.N, N = S.N;
   const double thi = bus_theta(S, x, sc, i), vi = bus_v(S, x, u, sc, i);
   const double lPi = lam_P(S, y, z, h, sc, i), lQi = lam_Q(S, y, z, sc, i);
-  double jd0 = 0, jd1 = 0, jd2 = 0, jd3 = 0;   // dP/dth, dP/dv, dQ/dth, dQ/dv (own bus)
-  double wtt = 0, wtv = 0, wvv = 0;            // diagonal Hessian block
-  double gt = 0, gv = 0;                       // (J^T lambda) at (th_i, v_i)
-  const int e1 = on_t ? S.inc_ptr[i + 1] : 0;
-  for (int e = S.inc_ptr[i] + sub; e < e1; e += LN) {
+  // dP/dth, dP/dv, dQ/dth, dQ/dv (own bus), the diagonal Hessian block (tt,
+  // tv, vv), (J^T lambda) at (th_i, v_i); the flow rows' terms of the last five
+  const Terms<9> sum = sum_lines<LN, 9, 5>(S, i, on_t, S.nflow != 0, [&](int e) {
+    Terms<14> c = {};
     const int l = S.inc_line[e], k = S.inc_other[e], q = S.inc_aslot[e];
     const double vk = bus_v(S, x, u, sc, k);
     double sn, cs;
@@ -191,20 +217,20 @@ __global__ void __launch_bounds__(128) k_derivatives(DevSym S, const double *__r
     line_end(vi, vk, cs, sn, lg, lb, lbh, own);
     line_end(vk, vi, cs, -sn, lg, lb, lbh, oth);
     const double lPk = lam_P(S, y, z, h, sc, k), lQk = lam_Q(S, y, z, sc, k);
-    jd0 += own.dPtm; jd1 += own.dPvm; jd2 += own.dQtm; jd3 += own.dQvm;
+    c.v[0] = own.dPtm; c.v[1] = own.dPvm; c.v[2] = own.dQtm; c.v[3] = own.dQvm;
     J[((size_t)q * 4 + 0) * N + sc] = own.dPto;
     J[((size_t)q * 4 + 1) * N + sc] = own.dPvo;
     J[((size_t)q * 4 + 2) * N + sc] = own.dQto;
     J[((size_t)q * 4 + 3) * N + sc] = own.dQvo;
-    wtt += lPi * Ptmtm(own) + lQi * Qtmtm(own) + lPk * Ptoto(oth) + lQk * Qtoto(oth);
-    wtv += lPi * Ptmvm(own) + lQi * Qtmvm(own) + lPk * Ptovo(oth) + lQk * Qtovo(oth);
-    wvv += lPi * Pvmvm(own) + lQi * Qvmvm(own);
+    c.v[4] = lPi * Ptmtm(own) + lQi * Qtmtm(own) + lPk * Ptoto(oth) + lQk * Qtoto(oth);
+    c.v[5] = lPi * Ptmvm(own) + lQi * Qtmvm(own) + lPk * Ptovo(oth) + lQk * Qtovo(oth);
+    c.v[6] = lPi * Pvmvm(own) + lQi * Qvmvm(own);
     W[((size_t)q * 4 + 0) * N + sc] = lPi * Ptmto(own) + lQi * Qtmto(own) + lPk * Ptmto(oth) + lQk * Qtmto(oth);
     W[((size_t)q * 4 + 1) * N + sc] = lPi * Ptmvo(own) + lQi * Qtmvo(own) + lPk * Ptovm(oth) + lQk * Qtovm(oth);
     W[((size_t)q * 4 + 2) * N + sc] = lPi * Ptovm(own) + lQi * Qtovm(own) + lPk * Ptmvo(oth) + lQk * Qtmvo(oth);
     W[((size_t)q * 4 + 3) * N + sc] = lPi * Pvmvo(own) + lQi * Qvmvo(own) + lPk * Pvmvo(oth) + lQk * Qvmvo(oth);
-    gt += lPi * own.dPtm + lQi * own.dQtm + lPk * oth.dPto + lQk * oth.dQto;
-    gv += lPi * own.dPvm + lQi * own.dQvm + lPk * oth.dPvo + lQk * oth.dQvo;
+    c.v[7] = lPi * own.dPtm + lQi * own.dQtm + lPk * oth.dPto + lQk * oth.dQto;
+    c.v[8] = lPi * own.dPvm + lQi * own.dQvm + lPk * oth.dPvo + lQk * oth.dQvo;
     if (S.nflow) {
       // flow rows of both ends of line l: h_own (this thread's row) and h_oth;
       // row i of W and of J^T lambda gets the terms in (theta_i, v_i)
@@ -215,30 +241,30 @@ __global__ void __launch_bounds__(128) k_derivatives(DevSym S, const double *__r
         HF[((size_t)(fo * 2 + (a >> 1)) * 2 + (a & 1)) * N + sc] =
             2.0 * (own.P * d1P(own, a) + own.Q * d1Q(own, a));
       // own end: i is m (0, 1), k is o (2, 3); other end: i is o, k is m
-      gt += zo * 2.0 * (own.P * own.dPtm + own.Q * own.dQtm) + zk * 2.0 * (oth.P * oth.dPto + oth.Q * oth.dQto);
-      gv += zo * 2.0 * (own.P * own.dPvm + own.Q * own.dQvm) + zk * 2.0 * (oth.P * oth.dPvo + oth.Q * oth.dQvo);
-      wtt += zo * d2flow(own, 0, 0) + zk * d2flow(oth, 2, 2);
-      wtv += zo * d2flow(own, 0, 1) + zk * d2flow(oth, 2, 3);
-      wvv += zo * d2flow(own, 1, 1) + zk * d2flow(oth, 3, 3);
+      c.v[12] = zo * 2.0 * (own.P * own.dPtm + own.Q * own.dQtm) + zk * 2.0 * (oth.P * oth.dPto + oth.Q * oth.dQto);
+      c.v[13] = zo * 2.0 * (own.P * own.dPvm + own.Q * own.dQvm) + zk * 2.0 * (oth.P * oth.dPvo + oth.Q * oth.dQvo);
+      c.v[9] = zo * d2flow(own, 0, 0) + zk * d2flow(oth, 2, 2);
+      c.v[10] = zo * d2flow(own, 0, 1) + zk * d2flow(oth, 2, 3);
+      c.v[11] = zo * d2flow(own, 1, 1) + zk * d2flow(oth, 3, 3);
       W[((size_t)q * 4 + 0) * N + sc] += zo * d2flow(own, 0, 2) + zk * d2flow(oth, 2, 0);
       W[((size_t)q * 4 + 1) * N + sc] += zo * d2flow(own, 0, 3) + zk * d2flow(oth, 2, 1);
       W[((size_t)q * 4 + 2) * N + sc] += zo * d2flow(own, 1, 2) + zk * d2flow(oth, 3, 0);
       W[((size_t)q * 4 + 3) * N + sc] += zo * d2flow(own, 1, 3) + zk * d2flow(oth, 3, 1);
     }
-  }
-  for (double *v : {&jd0, &jd1, &jd2, &jd3, &wtt, &wtv, &wvv, &gt, &gv}) *v = lanes_sum<LN>(*v);
+    return c;
+  });
   if (!on_t || sub != 0) return;
   const int d = S.a_diag[i];
-  J[((size_t)d * 4 + 0) * N + sc] = jd0;
-  J[((size_t)d * 4 + 1) * N + sc] = jd1;
-  J[((size_t)d * 4 + 2) * N + sc] = jd2;
-  J[((size_t)d * 4 + 3) * N + sc] = jd3;
-  W[((size_t)d * 4 + 0) * N + sc] = wtt;
-  W[((size_t)d * 4 + 1) * N + sc] = wtv;
-  W[((size_t)d * 4 + 2) * N + sc] = wtv;
-  W[((size_t)d * 4 + 3) * N + sc] = wvv;
-  JTl[(size_t)sc * 2 * S.n + i] = gt;
-  JTl[(size_t)sc * 2 * S.n + S.n + i] = gv;
+  J[((size_t)d * 4 + 0) * N + sc] = sum.v[0];
+  J[((size_t)d * 4 + 1) * N + sc] = sum.v[1];
+  J[((size_t)d * 4 + 2) * N + sc] = sum.v[2];
+  J[((size_t)d * 4 + 3) * N + sc] = sum.v[3];
+  W[((size_t)d * 4 + 0) * N + sc] = sum.v[4];
+  W[((size_t)d * 4 + 1) * N + sc] = sum.v[5];
+  W[((size_t)d * 4 + 2) * N + sc] = sum.v[5];
+  W[((size_t)d * 4 + 3) * N + sc] = sum.v[6];
+  JTl[(size_t)sc * 2 * S.n + i] = sum.v[7];
+  JTl[(size_t)sc * 2 * S.n + S.n + i] = sum.v[8];
 }
 
 __device__ __forceinline__ double sigma_of(double w, double l, double b, double zl, double zu) {
@@ -354,27 +380,22 @@ __global__ void k_rhs_x(DevSym S, DevWork D, const double *mu_d) {
 
 // u gradient of sum_i (f_i + y_i^T g_i + z_i^T h_i), summed over scenarios in
 // index order (first-stage coupling row of eq. (5)).
-// A warp per u row, lanes over the scenarios (fixed order: lane l takes
-// scenarios l, l + 32, ...): one thread walking them all waited for its loads
-// in turn (1,000 buses x 64: 52 us, less than 10 with this).
+// A warp per u row: one thread walking the scenarios waited for its loads in
+// turn (1,000 buses x 64: 53 us, with this 4; 120 x 17: 12 and 5).
 __global__ void __launch_bounds__(256) k_ugrad(DevSym S, DevWork D, double *gLu, double *HTt_u) {
   const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (j >= S.nu) return;
   double acc = 0.0, acc2 = 0.0;
   if (j < S.ng) {
     const int a = S.hrow_bus[j];
-    for (int sc = lane; sc < S.N; sc += 32) {
-      acc += D.JTl[(size_t)sc * 2 * S.n + S.n + a];
-      if (HTt_u) acc2 += HT_at(S, D.J, D.HF, D.tv, sc, a, 1);
-    }
+    acc = scenario_sum(S, [&](int sc) { return D.JTl[(size_t)sc * 2 * S.n + S.n + a]; });
+    if (HTt_u) acc2 = scenario_sum(S, [&](int sc) { return HT_at(S, D.J, D.HF, D.tv, sc, a, 1); });
   } else {
     const int k = j - S.ng + 1, a = S.hrow_bus[k];
     const double pg = D.u[j];
-    for (int sc = lane; sc < S.N; sc += 32)
-      acc += (2.0 * S.c2[k] * pg + S.c1[k]) / S.N - D.y[(size_t)sc * S.nx + S.xth[a]];
+    const double slope = (2.0 * S.c2[k] * pg + S.c1[k]) / S.N;
+    acc = scenario_sum(S, [&](int sc) { return slope - D.y[(size_t)sc * S.nx + S.xth[a]]; });
   }
-  acc = warp_sum(acc);
-  acc2 = warp_sum(acc2);
   if (lane == 0) {
     gLu[j] = acc;
     if (HTt_u) HTt_u[j] = acc2;

@@ -163,7 +163,7 @@ __global__ void k_res_x(DevSym S, DevWork D, double delta, const double *px, con
   warp_max2(res, scl, amax);
 }
 
-// u rows (a warp per row, lanes over the scenarios):
+// u rows (a warp per row):
 // rho_1u = -r1u - (sum_i kpu_i + diag1 p_u) - delta p_u - sum_i (G_u^T p_y,i + H_u^T tw_i)
 __global__ void __launch_bounds__(256) k_res_u(DevSym S, DevWork D, double delta, const double *pu,
                                                const double *upart, const double *umag, const double *diag1,
@@ -171,12 +171,11 @@ __global__ void __launch_bounds__(256) k_res_u(DevSym S, DevWork D, double delta
   const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   double res = 0.0, scl = 0.0;
   if (j < S.nu) {
-    double acc = 0.0, mag = 0.0;
-    for (int sc = lane; sc < S.N; sc += 32) {
-      acc += upart[(size_t)sc * S.nu + j];
+    double mag = 0.0;
+    const double acc = scenario_sum(S, [&](int sc) {
       mag = fmax(mag, umag[(size_t)sc * S.nu + j]);
-    }
-    acc = warp_sum(acc);
+      return upart[(size_t)sc * S.nu + j];
+    });
     mag = warp_max(mag);
     if (lane == 0) {
       const double dp = (diag1[j] + delta) * pu[j];

@@ -75,11 +75,62 @@ __global__ void __launch_bounds__(256) k_diag_inverse(DevSym S, const double *__
   }
 }
 
+// The trailing block of a small network (S.ordered), T = L or U^T going
+// down, U or L^T going up, on x (the block's entries): 32 x 32 diagonal
+// blocks step by step by one warp (lane = row; where T's diagonal is the
+// pivots, their reciprocals are in the block's columns), the rows past a
+// block by a thread each with four partial sums.  Bound by the chain; a solve
+// at 120 buses x 17 takes 31 us, by the diagonal blocks' inverses 24 and 7 to
+// form them once per factorization.
+template <int TH>
+__device__ void dense_small(const double *__restrict__ D, const double *__restrict__ r, int nd, bool trans, bool up,
+                            double *x, double (*blk)[33]) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const bool scale = trans != up;  // U^T going down, U going up
+  const size_t si = trans ? nd : 1, sk = trans ? 1 : nd;  // T(i, k) = D[i si + k sk]
+  for (int s = 0; s < nd; s += 32) {
+    const int kb = up ? (nd - 1) / 32 * 32 - s : s, w = min(32, nd - kb);
+    for (int e = tid; e < 32 * w; e += TH) {
+      const int i = e >> 5, k = e & 31;
+      double t = 0.0;
+      if (up ? k > i && k < w : k < i) t = D[(kb + i) * si + (kb + k) * sk] * (scale ? r[kb + k] : 1.0);
+      blk[i][k] = t;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      double v = lane < w ? x[kb + lane] : 0.0;
+      for (int q = 0; q < w; ++q) {
+        const int k = up ? w - 1 - q : q;
+        const double xk = __shfl_sync(0xffffffffu, v, k);
+        if (up ? lane < k : lane > k && lane < w) v = fma(-blk[lane][k], xk, v);
+      }
+      if (lane < w) x[kb + lane] = scale ? v * r[kb + lane] : v;
+    }
+    __syncthreads();
+    for (int i = up ? tid : kb + w + tid; i < (up ? kb : nd); i += TH) {
+      const double *p = D + i * si + kb * sk;
+      double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+      int j = 0;
+      for (; j + 4 <= w; j += 4) {
+        s0 = fma(p[j * sk], x[kb + j], s0);
+        s1 = fma(p[(j + 1) * sk], x[kb + j + 1], s1);
+        s2 = fma(p[(j + 2) * sk], x[kb + j + 2], s2);
+        s3 = fma(p[(j + 3) * sk], x[kb + j + 3], s3);
+      }
+      for (; j < w; ++j) s0 = fma(p[j * sk], x[kb + j], s0);
+      x[i] -= (s0 + s1) + (s2 + s3);
+    }
+    __syncthreads();
+  }
+}
+
 // Vector b of v ([N * vps][n_x]) belongs to scenario b / vps.  MULTI: a
 // cluster of C CTAs per vector, the vector in global memory (read and
 // written past L1); else one CTA per vector, the vector in shared memory
-// when it fits (in_smem).
-template <int TH, int NB, bool MULTI>
+// when it fits (in_smem).  ORDERED (small networks, the vector in shared
+// memory): the products of a lane one after the other, the lanes joined from
+// the widest distance down, the trailing block by dense_small.
+template <int TH, int NB, bool MULTI, bool ORDERED = false>
 __global__ void __launch_bounds__(TH, MULTI && TH == 512 ? 2 : 1) k_solve1(DevSym S, const double *__restrict__ LU, const double *__restrict__ rd,
                                                double *v, int trans, int vps, int C, int in_smem) {
   extern __shared__ double sm1[];
@@ -88,7 +139,8 @@ __global__ void __launch_bounds__(TH, MULTI && TH == 512 ? 2 : 1) k_solve1(DevSy
   const int vec = MULTI ? blockIdx.x / C : blockIdx.x, rank = MULTI ? blockIdx.x % C : 0;
   const int sc = vec / vps, nx = S.nx, t0 = S.t0, nd = S.nd, nblk = (nd + NB - 1) / NB;
   const double *A = LU + (size_t)sc * S.nnzLU, *r = rd + (size_t)sc * nx;
-  double *xsm = sm1 + trsv::smem_doubles<TH, NB>((nblk + C - 1) / C);
+  __shared__ double blk[ORDERED ? 32 : 1][33];
+  double *xsm = sm1 + (ORDERED ? 0 : trsv::smem_doubles<TH, NB>((nblk + C - 1) / C));
   double *vs = v + (size_t)vec * nx, *x = !MULTI && in_smem ? xsm : vs;
   const auto ldx = [&](int i) { return MULTI ? __ldcg(x + i) : x[i]; };
   const auto stx = [&](int i, double y) {
@@ -171,8 +223,14 @@ __global__ void __launch_bounds__(TH, MULTI && TH == 512 ? 2 : 1) k_solve1(DevSy
 #pragma unroll
       for (int h = 0; h < SWP; ++h) x0[h] = operand(p0[h]);
       const double xr = lead ? ldx(rc & 0x3ffffff) : 0.0;
-      double part = fma(a0[0], x0[0], a0[1] * x0[1]) + fma(a0[2], x0[2], a0[3] * x0[3]);
-      if (code & 8) {  // a row of more than 32 SWP products: the rest of it
+      double part = 0.0;
+      if (ORDERED) {
+#pragma unroll
+        for (int h = 0; h < SWP; ++h) part = fma(a0[h], x0[h], part);
+      } else {
+        part = fma(a0[0], x0[0], a0[1] * x0[1]) + fma(a0[2], x0[2], a0[3] * x0[3]);
+      }
+      if (code & 8) {  // the products left over
         const int2 ex = S.sw_extra[u0];
         for (int k = 0; k < ex.y; ++k) {
 #pragma unroll
@@ -182,7 +240,10 @@ __global__ void __launch_bounds__(TH, MULTI && TH == 512 ? 2 : 1) k_solve1(DevSy
           }
         }
       }
-      for (int o = 1; o < g; o <<= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+      if (ORDERED)
+        for (int o = g >> 1; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+      else
+        for (int o = 1; o < g; o <<= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
       if (lead) stx(rc & 0x3ffffff, (xr - part) * rr);
       for (; l0 < l1; ++l0) sync_all();
       u0 = u1;
@@ -202,6 +263,10 @@ __global__ void __launch_bounds__(TH, MULTI && TH == 512 ? 2 : 1) k_solve1(DevSy
   // the trailing block: T = L or U^T going down, U or L^T going up, at
   // LU[k nd + i], or LU[i nd + k] with trans
   const auto dense = [&](bool up) {
+    if (ORDERED) {
+      dense_small<TH>(A + S.dense_base, r + t0, nd, trans != 0, up, x + t0, blk);
+      return;
+    }
     const double *inv = S.dinv + (size_t)sc * nblk * 2 * NB * NB + ((trans != 0) != up ? NB * NB : 0);
     trsv::sweep<TH, NB, MULTI>(
         A + S.dense_base, (size_t)nd, nd, trans != 0, up, inv, 2 * NB * NB, C, rank, sm1,
@@ -238,6 +303,14 @@ void solve1_single(const DevSym &S, const double *LU, const double *rd, double *
   const int in = base + vec <= cap ? 1 : 0;
   k_solve1<TH, NB, false><<<(unsigned)(S.N * (long long)vps), TH, base + (in ? vec : 0), st>>>(S, LU, rd, v, trans, vps,
                                                                                          1, in);
+  ipm_count_launch();
+}
+
+// the small networks: one CTA per vector
+template <int TH>
+void solve1_ordered(const DevSym &S, const double *LU, const double *rd, double *v, int trans, int vps, cudaStream_t st) {
+  k_solve1<TH, NB_SMALL, false, true><<<(unsigned)(S.N * (long long)vps), TH, (size_t)S.nx * sizeof(double), st>>>(
+      S, LU, rd, v, trans, vps, 1, 1);
   ipm_count_launch();
 }
 
@@ -283,11 +356,12 @@ void diag_inverse(const DevSym &S, const double *LU, const double *rd, cudaStrea
 
 size_t diag_inverse_doubles(const DevSym &S) {
   const int NB = S.big ? NB_BIG : NB_SMALL;
+  if (S.ordered) return 0;  // k_solve1 does without
   return (size_t)S.N * ((S.nd + NB - 1) / NB) * 2 * NB * NB;
 }
 
 void launch_diag_inverse(const DevSym &S, const double *LU, const double *rd, cudaStream_t st) {
-  if (S.nd == 0) return;
+  if (S.nd == 0 || S.ordered) return;
   if (S.big) diag_inverse<NB_BIG>(S, LU, rd, st);
   else diag_inverse<NB_SMALL>(S, LU, rd, st);
 }
@@ -299,13 +373,15 @@ void launch_solve1(const DevSym &S, const double *LU, const double *rd, double *
   }
   // one warp per scheduled unit is enough on the small networks, and a
   // barrier over four warps is cheaper than over eight
-  if (S.nx <= 400) solve1_single<128, NB_SMALL>(S, LU, rd, v, trans, 1, st);
+  if (S.ordered) solve1_ordered<128>(S, LU, rd, v, trans, 1, st);
+  else if (S.nx <= 400) solve1_single<128, NB_SMALL>(S, LU, rd, v, trans, 1, st);
   else solve1_single<256, NB_SMALL>(S, LU, rd, v, trans, 1, st);
 }
 
 void launch_solve1_batched(const DevSym &S, const double *LU, const double *rd, double *v, int trans, int vps,
                            cudaStream_t st) {
-  if (!S.big) solve1_single<128, NB_SMALL>(S, LU, rd, v, trans, vps, st);
+  if (S.ordered) solve1_ordered<128>(S, LU, rd, v, trans, vps, st);
+  else if (!S.big) solve1_single<128, NB_SMALL>(S, LU, rd, v, trans, vps, st);
   else if (S.nd <= 4096) solve1_single<256, NB_BIG>(S, LU, rd, v, trans, vps, st);  // 128 KB of accumulators
   else solve1_cluster(S, LU, rd, v, trans, vps, st);
 }

@@ -27,11 +27,14 @@ __device__ __forceinline__ double warp_op(int op, double v) {
 }
 
 // One launch per reduction: every CTA leaves its partial values, and the one
-// that counts last joins them, a warp per value (lane l takes CTAs l, l + 32,
-// ..., then the lanes in a fixed tree), and sets the count back.  Joining the
-// 152 partial values one after the other in a launch of its own took 40 us
-// for the optimality error's seven (dependent FP64 additions), 11 for the
-// merit's three.
+// that counts last joins them and sets the count back.  Joining the 152
+// partial values in a launch of its own, one after the other, took 40 us for
+// the optimality error's seven, 11 for the merit's three.  Up to half of
+// RED_BLOCKS CTAs (19,456 elements) they are joined in the order of the CTAs
+// (a thread per value, from shared memory, so that only the additions are on
+// the chain), which the whole solves of the small problems keep
+// (ipm_internal.h); from there on by a warp per value (lane l takes CTAs l, l +
+// 32, ..., then the lanes in a fixed tree).
 template <class F>
 __global__ void __launch_bounds__(256) k_reduce(F f, long long n, double *partial, double *out, unsigned *count) {
   static_assert(F::NV <= 8, "a warp of the CTA per value");
@@ -40,7 +43,7 @@ __global__ void __launch_bounds__(256) k_reduce(F f, long long n, double *partia
   for (int i = 0; i < F::NV; ++i) acc[i] = op_init(F::op(i));
   for (long long t = (long long)blockIdx.x * 256 + threadIdx.x; t < n; t += (long long)gridDim.x * 256)
     f(t, acc);
-  __shared__ double sh[F::NV][8];
+  __shared__ double sh[F::NV][8], all[RED_BLOCKS / 2 * F::NV];
   __shared__ bool last;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
@@ -49,14 +52,12 @@ __global__ void __launch_bounds__(256) k_reduce(F f, long long n, double *partia
     if (lane == 0) sh[i][w] = v;
   }
   __syncthreads();
-  double v = op_init(OP_SUM);
-  if (w < F::NV) {
-    v = lane < 8 ? sh[w][lane] : op_init(F::op(w));
-    v = warp_op(F::op(w), v);
-    if (lane == 0) {
-      (gridDim.x == 1 ? out : partial + (size_t)blockIdx.x * F::NV)[w] = v;
-      __threadfence();
-    }
+  const int i = threadIdx.x;
+  if (i < F::NV) {
+    double v = sh[i][0];
+    for (int q = 1; q < 8; ++q) v = op_comb(F::op(i), v, sh[i][q]);
+    (gridDim.x == 1 ? out : partial + (size_t)blockIdx.x * F::NV)[i] = v;
+    __threadfence();
   }
   if (gridDim.x == 1) return;
   __syncthreads();
@@ -66,12 +67,24 @@ __global__ void __launch_bounds__(256) k_reduce(F f, long long n, double *partia
     if (last) *count = 0u;
   }
   __syncthreads();
-  if (!last || w >= F::NV) return;
+  if (!last) return;
   __threadfence();
-  v = op_init(F::op(w));
-  for (int b = lane; b < (int)gridDim.x; b += 32) v = op_comb(F::op(w), v, __ldcg(&partial[(size_t)b * F::NV + w]));
-  v = warp_op(F::op(w), v);
-  if (lane == 0) out[w] = v;
+  const int nb = gridDim.x;
+  if (nb > RED_BLOCKS / 2) {
+    if (w >= F::NV) return;
+    double v = op_init(F::op(w));
+    for (int b = lane; b < nb; b += 32) v = op_comb(F::op(w), v, __ldcg(&partial[(size_t)b * F::NV + w]));
+    v = warp_op(F::op(w), v);
+    if (lane == 0) out[w] = v;
+    return;
+  }
+  for (int e = threadIdx.x; e < nb * F::NV; e += 256) all[e] = __ldcg(&partial[e]);
+  __syncthreads();
+  if (i < F::NV) {
+    double v = all[i];
+    for (int b = 1; b < nb; ++b) v = op_comb(F::op(i), v, all[b * F::NV + i]);
+    out[i] = v;
+  }
 }
 
 template <class F>
@@ -273,29 +286,51 @@ __global__ void k_gu_apply(DevSym S, const double *J, const double *pu, double *
 }
 
 // kpx = K_xx px (+ K_xu pu);  kpu = K_ux px + K_uu pu  (position rows, u rows).
-// Eight lanes per row: the rows of buses next to a hub or a generator have
-// many entries, and one thread took their three dependent loads and the
-// multiply-add in turn (30 buses x 1: 13 -> 4 us,
-// 119 x 7: 15 -> 5, 1,000 x 64: 24 -> 17).
+// Eight lanes per row fetch its entries side by side (the rows of buses next
+// to a hub or a generator have many, and one thread took their three dependent
+// loads in turn: 30 buses x 1 14 us, with this 5; 1,000 x 64 24 and 16).  The
+// products are added in the order of the entries with S.ordered; past that by
+// lanes and a tree, which takes a fifth of the FP64 operations (1,000 x 64: 31
+// us in order).
 __global__ void __launch_bounds__(256) k_kapply(DevSym S, const double *__restrict__ K, const double *px_pos,
                                                 const double *pu, double *kpx, double *kpu) {
   const long long t = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
   const int sub = threadIdx.x & 7;
   const long long nX = (long long)S.N * S.nx;
   const bool xrow = t < nX, urow = !xrow && kpu && t < nX + (long long)S.N * S.nu;
-  double acc = 0.0;
+  const int *cols = xrow ? S.kx_col : S.ku_col, *src = xrow ? S.kx_src : S.ku_src;
+  int sc = 0, e0 = 0, len = 0;
   if (xrow || urow) {
     const long long q = xrow ? t : t - nX;
-    const int len = xrow ? S.nx : S.nu, sc = (int)(q / len), p = (int)(q - (long long)sc * len);
-    const int *ptr = xrow ? S.kx_ptr : S.ku_ptr, *cols = xrow ? S.kx_col : S.ku_col, *src = xrow ? S.kx_src : S.ku_src;
-    for (int e = ptr[p] + sub; e < ptr[p + 1]; e += 8) {
-      const int col = cols[e];
-      if (col >= S.nx && !pu) continue;
-      acc += K[(size_t)src[e] * S.N + sc] * (col < S.nx ? px_pos[(size_t)sc * S.nx + col] : pu[col - S.nx]);
-    }
+    const int rows = xrow ? S.nx : S.nu, p = (int)(q % rows), *ptr = xrow ? S.kx_ptr : S.ku_ptr;
+    sc = (int)(q / rows);
+    e0 = ptr[p];
+    len = ptr[p + 1] - e0;
   }
+  const auto entry = [&](int e, double &k, double &x) {
+    const int col = cols[e0 + e];
+    if (col >= S.nx && !pu) return;
+    k = K[(size_t)src[e0 + e] * S.N + sc];
+    x = col < S.nx ? px_pos[(size_t)sc * S.nx + col] : pu[col - S.nx];
+  };
+  double acc = 0.0;
+  if (S.ordered) {
+    const int most = (int)__reduce_max_sync(0xffffffffu, (unsigned)len);  // of the warp's four rows
+    for (int b = 0; b < most; b += 8) {
+      double k = 0.0, x = 0.0;
+      if (b + sub < len) entry(b + sub, k, x);
+      const int n = min(8, most - b);
+      for (int j = 0; j < n; ++j) acc = fma(__shfl_sync(0xffffffffu, k, j, 8), __shfl_sync(0xffffffffu, x, j, 8), acc);
+    }
+  } else {
+    for (int e = sub; e < len; e += 8) {
+      double k = 0.0, x = 0.0;
+      entry(e, k, x);
+      acc = fma(k, x, acc);
+    }
 #pragma unroll
-  for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  }
   if (sub != 0) return;
   if (xrow) kpx[t] = acc;
   else if (urow) kpu[t - nX] = acc;
@@ -356,6 +391,7 @@ __global__ void __launch_bounds__(256) k_zt_part(DevSym S, const double *__restr
   const double *ws = w + (size_t)sc * S.nx;
   double acc = 0.0;
   if (j < S.nu)
+#pragma unroll 4  // rows in flight; without it 139 us instead of 101 at 1,000 buses x 64
     for (int p = warp; p < S.nx; p += 8) acc += Zs[(size_t)p * S.nu + j] * ws[p];
   red[warp][lane] = acc;
   __syncthreads();
@@ -372,14 +408,12 @@ __global__ void __launch_bounds__(256) k_zt_part(DevSym S, const double *__restr
   }
 }
 
-// out[j] = beta*out[j] + sum_s part[s][j]  (a warp per u row, lanes over the
-// scenarios); beta = 0 does not read out (it may hold anything, NaN included)
+// out[j] = beta*out[j] + sum_s part[s][j]  (a warp per u row); beta = 0 does
+// not read out (it may hold anything, NaN included)
 __global__ void __launch_bounds__(256) k_zt_sum(DevSym S, const double *part, double beta, double *out) {
   const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (j >= S.nu) return;
-  double acc = 0.0;
-  for (int sc = lane; sc < S.N; sc += 32) acc += part[(size_t)sc * S.nu + j];
-  acc = warp_sum(acc);
+  const double acc = scenario_sum(S, [&](int sc) { return part[(size_t)sc * S.nu + j]; });
   if (lane == 0) out[j] = beta == 0.0 ? acc : beta * out[j] + acc;
 }
 

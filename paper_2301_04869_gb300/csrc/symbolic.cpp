@@ -82,15 +82,19 @@ void min_degree(int nv, std::vector<std::vector<int>> adj, std::vector<int> &ord
 // The units of the single-vector sweeps (layout in ipm_internal.h).  A level's
 // rows are taken longest first, so that rows packed into a unit are of about
 // one length and the long ones start early.
-static void build_sweeps(Sym &S) {
+static void build_sweeps(Sym &S, int N) {
   struct Prod {
     int col, slot, tslot;
   };
   struct Level {
     std::vector<std::pair<int, std::vector<Prod>>> rows;
   };
+  S.ordered = !S.big && S.nx <= ORDERED_NX && N <= ORDERED_N;
   // extra units follow all scheduled ones; they are kept aside until then
-  std::vector<std::array<int, 3>> long_rows;  // (unit, level list index, row index) of rows of more than one unit
+  struct Long {
+    int unit, level, first, rows, lg;
+  };
+  std::vector<Long> longs;  // units whose rows have products left over
   std::vector<Level> levels;
   const auto add = [&](const std::vector<int> &rows, size_t e0, size_t e1, bool fwd, int below) {
     Level L;
@@ -114,7 +118,7 @@ static void build_sweeps(Sym &S) {
   const size_t nf = levels.size();
   for (int l = 0; l < S.nlev_bs; ++l) add(S.bs_rows, S.bs_lev_ptr[l], S.bs_lev_ptr[l + 1], false, S.nx);
   // one unit: P products per lane, 2^lg lanes per row
-  constexpr int P = 4, FULL = 32 * P;
+  constexpr int P = 4;
   std::vector<int> titem;
   const auto put = [&](const std::vector<std::pair<int, const Prod *>> &rows, const std::vector<int> &n, int lg, int code) {
     const int g = 1 << lg;
@@ -133,7 +137,8 @@ static void build_sweeps(Sym &S) {
     }
   };
   int units = 0;
-  const auto lanes_lg = [](size_t n) {
+  const auto lanes_lg = [&](size_t l, size_t n) {
+    if (S.ordered) return l < (size_t)S.nlev_fs ? 2 : 3;
     int lg = 0;
     while (lg < 5 && (size_t)(P << lg) < n) ++lg;
     return lg;
@@ -143,15 +148,16 @@ static void build_sweeps(Sym &S) {
     if (lev.empty()) lev.push_back(units);
     const auto &rows = levels[l].rows;
     for (size_t e = 0; e < rows.size();) {
-      const int lg = lanes_lg(rows[e].second.size());
+      const int lg = lanes_lg(l, rows[e].second.size()), first = (int)e;
+      const size_t full = (size_t)P << lg;
       std::vector<std::pair<int, const Prod *>> rs;
       std::vector<int> n;
-      const bool over = rows[e].second.size() > FULL;
-      if (over) long_rows.push_back({units, (int)l, (int)e});
-      for (; e < rows.size() && rs.size() < (size_t)(32 >> lg) && lanes_lg(rows[e].second.size()) == lg; ++e) {
+      for (; e < rows.size() && rs.size() < (size_t)(32 >> lg) && lanes_lg(l, rows[e].second.size()) == lg; ++e) {
         rs.push_back({rows[e].first, rows[e].second.data()});
-        n.push_back((int)std::min<size_t>(rows[e].second.size(), FULL));
+        n.push_back((int)std::min(rows[e].second.size(), full));
       }
+      const bool over = rows[first].second.size() > full;  // the longest
+      if (over) longs.push_back({units, (int)l, first, (int)rs.size(), lg});
       put(rs, n, lg, lg | (over ? 8 : 0));
       ++units;
     }
@@ -161,12 +167,20 @@ static void build_sweeps(Sym &S) {
   if (S.swb_lev.empty()) S.swb_lev.assign(1, units);
   S.sw_extra.assign((size_t)std::max(units, 1) * 2, 0);
   int next = units;
-  for (const auto &lr : long_rows) {
-    const auto &row = levels[lr[1]].rows[lr[2]];
-    S.sw_extra[(size_t)lr[0] * 2] = next;
-    for (size_t f = FULL; f < row.second.size(); f += FULL, ++next) {
-      put({{row.first, row.second.data() + f}}, {(int)std::min<size_t>(row.second.size() - f, FULL)}, 5, 5 | 8);
-      ++S.sw_extra[(size_t)lr[0] * 2 + 1];
+  for (const Long &lu : longs) {
+    const auto *rows = &levels[lu.level].rows[lu.first];
+    const size_t full = (size_t)P << lu.lg;
+    S.sw_extra[(size_t)lu.unit * 2] = next;
+    for (size_t f = full; f < rows[0].second.size(); f += full, ++next) {
+      std::vector<std::pair<int, const Prod *>> rs;
+      std::vector<int> n;
+      for (int q = 0; q < lu.rows; ++q) {
+        const size_t len = rows[q].second.size();
+        rs.push_back({rows[q].first, rows[q].second.data() + std::min(f, len)});
+        n.push_back((int)std::min(len - std::min(f, len), full));
+      }
+      put(rs, n, lu.lg, lu.lg | 8);
+      ++S.sw_extra[(size_t)lu.unit * 2 + 1];
     }
   }
   S.sw_item.insert(S.sw_item.end(), titem.begin(), titem.end());
@@ -662,7 +676,7 @@ bool build_symbolic(const HostNet &net, int N, Sym &S, std::string &err, int big
     }
     S.nlev_bs = (int)S.bs_lev_ptr.size() - 1;
     for (int i : S.bs_rows) S.bs4.insert(S.bs4.end(), {i, S.br_ptr[i], S.br_ptr[i + 1], 0});
-    build_sweeps(S);
+    build_sweeps(S, N);
   }
   // ---- G_u (rows: positions) and its transpose (rows: u) ----
   const int nu = S.nu;
