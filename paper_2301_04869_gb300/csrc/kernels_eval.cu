@@ -416,9 +416,10 @@ __global__ void k_rhs_u(DevSym S, DevWork D, const double *gLu, const double *HT
 // ---------------------------------------------------------------------------
 static inline int nblk(long long n, int b) { return (int)((n + b - 1) / b); }
 
-// eight lanes per (bus, scenario) until the pairs alone come to 256 threads
-// per SM
-static inline bool eval_lanes(const DevSym &S) { return (long long)S.n * S.N < 152 * 256; }
+// eight lanes per (bus, scenario) until the pairs alone come to 160 threads
+// per SM: functions + derivatives of 1,000 buses with eight lanes and with one,
+// x 5 scenarios 34 and 68 us, x 20 67 and 79, x 38 112 and 81, x 64 177 and 106
+static inline bool eval_lanes(const DevSym &S) { return (long long)S.n * S.N < 152 * 160; }
 
 void launch_functions(const DevSym &S, const double *x, const double *u, double *P, double *Q,
                       double *g, double *h, double *fs, cudaStream_t st) {
