@@ -60,7 +60,7 @@ struct ipm_ctx {
   // mixed path
   bool mixed = false;
   float *Z32 = nullptr, *Y32 = nullptr;
-  void *zwork = nullptr;  // work buffer of the multi-RHS solves
+  ZsolveWork zwork, zwork64;  // work buffers of the multi-RHS solves in the path's own type and in FP64
   RoundedFactors rf;  // FP32 copies of the factors and K for the FP32 solve
   void *zpl = nullptr, *ypl = nullptr;  // BF16x3 planes, K-major [3][nu][kpad]
   double *tcpart = nullptr;

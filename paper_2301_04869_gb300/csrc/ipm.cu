@@ -268,6 +268,8 @@ ipm_status alloc_work(ipm_ctx *c) {
     c->ypl = (unsigned char *)c->zpl + pl * 2;
     c->Z = (double *)region;
     c->Y = (double *)(region + E * 8);
+    const size_t zy = (E * 16 + 255) / 256 * 256, all = (bytes + 255) / 256 * 256;
+    c->zwork64 = {region + zy, all > zy ? all - zy : 0};
     if ((size_t)((unsigned char *)c->ypl - region) + pl * 2 > (bytes + 255) / 256 * 256)
       return fail(c, IPM_ERR_ARG, "internal: mixed region layout");
     if (!tc_set_operands(c->planZY, c->zpl, c->ypl) || !tc_set_operands(c->planZZ, c->zpl, c->zpl))
@@ -318,13 +320,20 @@ ipm_status alloc_work(ipm_ctx *c) {
     set_groups(c, (long long)S.N * S.nx <= 64 * G0 ? G0 : 4 * G0);
     c->max_groups = c->ngroups;
   }
-  {
-    // the multi-RHS solve's panels in flight; a mixed context also runs the FP64 solve (fallback iterations)
-    unsigned char *zw = nullptr;
-    TRY(dalloc(c, &zw, zsolve_work_bytes(c->ds, sizeof(double))));
-    c->zwork = zw;
-  }
   c->zs_threads = (c->opt.solve_threads == 128 || c->opt.solve_threads == 256) ? c->opt.solve_threads : 256;
+  {
+    // the multi-RHS solve's panels in flight (a tuned thread count uses what
+    // the default one needs); the FP64 solve of a fallback iteration takes
+    // the region's end behind its Z and Y where it fits there
+    const size_t own = zsolve_work_bytes(c->ds, c->mixed ? sizeof(float) : sizeof(double), c->zs_threads);
+    const size_t need64 = zsolve_work_bytes(c->ds, sizeof(double), c->zs_threads);
+    const bool in_region = c->mixed && need64 <= c->zwork64.bytes;
+    c->zwork.bytes = c->mixed && !in_region ? std::max(own, need64) : own;
+    unsigned char *zw = nullptr;
+    TRY(dalloc(c, &zw, c->zwork.bytes));
+    c->zwork.p = zw;
+    if (!in_region) c->zwork64 = c->zwork;
+  }
   TRY(dalloc(c, &c->tiles, tl.size()));
   CK(cudaMemcpy(c->tiles, tl.data(), tl.size() * sizeof(int2), cudaMemcpyHostToDevice));
   TRY(dalloc(c, &c->tile_of, tof.size()));
@@ -646,8 +655,8 @@ ipm_status autotune(ipm_ctx *c, cudaStream_t st) {
   double best = 1e300;
   int best_thr = 256;
   for (int thr : {128, 256}) {
-    const double ms = fp64 ? time_ms([&] { launch_zsolve64(S, D.LU, D.rd, D.J, D.K, (double *)c->zwork, c->Z, c->Y, c->Yu, st, thr); }, st)
-                           : time_ms([&] { launch_zsolve32(S, D.LU, D.rd, D.J, D.K, c->rf, (float *)c->zwork, c->Z32, c->Y32, c->Yu, st, thr, tcs_of(c), D.flags); }, st);
+    const double ms = fp64 ? time_ms([&] { launch_zsolve64(S, D.LU, D.rd, D.J, D.K, c->zwork64, c->Z, c->Y, c->Yu, st, thr); }, st)
+                           : time_ms([&] { launch_zsolve32(S, D.LU, D.rd, D.J, D.K, c->rf, c->zwork, c->Z32, c->Y32, c->Yu, st, thr, tcs_of(c), D.flags); }, st);
     c->tune_ms[thr == 128 ? 0 : 1] = ms;
     if (ms < best) best = ms, best_thr = thr;
   }
@@ -655,9 +664,9 @@ ipm_status autotune(ipm_ctx *c, cudaStream_t st) {
   // the solve outputs are identical for every thread count; rerun the winner
   // so that the mixed planes are split from them below
   if (fp64) {
-    launch_zsolve64(S, D.LU, D.rd, D.J, D.K, (double *)c->zwork, c->Z, c->Y, c->Yu, st, best_thr);
+    launch_zsolve64(S, D.LU, D.rd, D.J, D.K, c->zwork64, c->Z, c->Y, c->Yu, st, best_thr);
   } else {
-    launch_zsolve32(S, D.LU, D.rd, D.J, D.K, c->rf, (float *)c->zwork, c->Z32, c->Y32, c->Yu, st, best_thr, tcs_of(c), D.flags);
+    launch_zsolve32(S, D.LU, D.rd, D.J, D.K, c->rf, c->zwork, c->Z32, c->Y32, c->Yu, st, best_thr, tcs_of(c), D.flags);
     launch_split_t((long long)S.N * S.nx, S.nu, c->planZY.kpad, c->Z32, c->zpl, st);
     launch_split_t((long long)S.N * S.nx, S.nu, c->planZY.kpad, c->Y32, c->ypl, st);
   }
@@ -810,9 +819,9 @@ ipm_status do_condense(ipm_ctx *c, cudaStream_t st) {
     if (fp64 && c->emu)
       cudaMemsetAsync(c->emu_rs, 0, 2 * (size_t)S.N * S.nx * sizeof(int), st);  // row exponent maxima
     if (fp64)
-      launch_zsolve64(S, D.LU, D.rd, D.J, D.K, (double *)c->zwork, c->Z, c->Y, c->Yu, st, c->zs_threads, D.g, c->bpos,
+      launch_zsolve64(S, D.LU, D.rd, D.J, D.K, c->zwork64, c->Z, c->Y, c->Yu, st, c->zs_threads, D.g, c->bpos,
                       c->emu ? c->emu_rs : nullptr);
-    else launch_zsolve32(S, D.LU, D.rd, D.J, D.K, c->rf, (float *)c->zwork, c->Z32, c->Y32, c->Yu, st, c->zs_threads, tcs_of(c), D.flags);
+    else launch_zsolve32(S, D.LU, D.rd, D.J, D.K, c->rf, c->zwork, c->Z32, c->Y32, c->Yu, st, c->zs_threads, tcs_of(c), D.flags);
     ph_end(c, PH_ZSOLVE, st);
     if (fp64) {
       // the reduced right-hand side needs Z and b only: on the side stream,

@@ -43,13 +43,19 @@ struct EmuLuPlan;
 // cores at FP64 grade; null: on the FP64 units)
 void launch_lu_factor(const DevSym &S, int nL, const double *J, double *LU, double *rd, int *flags,
                       cudaStream_t st, bool allow_pair = true, const EmuLuPlan *emu_lu = nullptr);
+// work buffer of the multi-RHS solves: the panels in flight
+struct ZsolveWork {
+  void *p = nullptr;
+  size_t bytes = 0;
+};
 // g, b (optional, [N][n_x]): also b = G_x^{-1} g in position order (g in
 // state order), in an extra right-hand-side lane, when zsolve64_folds_b
 void launch_zsolve64(const DevSym &S, const double *LU, const double *rd, const double *J, const double *K,
-                     double *work, double *Z, double *Y, double *Yu, cudaStream_t st, int threads = 256,
+                     ZsolveWork work, double *Z, double *Y, double *Yu, cudaStream_t st, int threads = 256,
                      const double *g = nullptr, double *b = nullptr, int *ezy = nullptr);
-// bytes of the multi-RHS solves' work buffer (elem: 8 FP64, 4 FP32)
-size_t zsolve_work_bytes(const DevSym &S, size_t elem);
+// bytes for all panels that a solve with CTAs of this many threads has in
+// flight (elem: 8 FP64, 4 FP32); with less, it has fewer in flight
+size_t zsolve_work_bytes(const DevSym &S, size_t elem, int threads);
 bool zsolve64_folds_b(const DevSym &S);
 // kernels_big.cu: the large trailing block (S.big) in global memory
 void launch_big_lu_dense(const DevSym &S, double *LU, double *rd, const double *amax, int *flags, cudaStream_t st,
@@ -68,7 +74,7 @@ struct RoundedFactors {
 };
 __host__ __device__ inline int round_lu_len(const DevSym &S) { return S.big ? S.dense_base : S.nnzLU; }
 void launch_zsolve32(const DevSym &S, const double *LU, const double *rd, const double *J, const double *K,
-                     const RoundedFactors &f, float *work, float *Z, float *Y, double *Yu, cudaStream_t st, int threads = 256,
+                     const RoundedFactors &f, ZsolveWork work, float *Z, float *Y, double *Yu, cudaStream_t st, int threads = 256,
                      const TcsPlan *tcs = nullptr, int *flags = nullptr);
 // kernels_solve1.cu: inverses of the trailing block's diagonal blocks (into
 // S.dinv, after every factorization), and solves of one vector per scenario

@@ -15,6 +15,7 @@
 // pattern with __syncthreads() between levels.  No grid-wide
 // synchronisation and no waits between CTAs other than the cluster
 // barriers.
+#include <algorithm>
 #include <atomic>
 
 #include "dev.cuh"
@@ -955,21 +956,21 @@ static int zsolve_grid(long long items, int threads) {
   return (int)(items < ZS_CTAS * (256 / threads) ? items : ZS_CTAS * (256 / threads));
 }
 
-size_t zsolve_work_bytes(const DevSym &S, size_t elem) {
-  size_t most = 0;
-  for (int threads : {128, 256})
-    for (int w : {8, 16, 32})
-      for (int extra : {0, 1}) {
-        const long long items = (long long)((S.nu + extra + w - 1) / w) * S.N;
-        const size_t b = (size_t)zsolve_grid(items, zsolve_cta(items, w, threads)) * S.nx * w * elem;
-        if (w == zsolve_width(S, S.nu + extra) && b > most) most = b;
-      }
-  return most;
+size_t zsolve_work_bytes(const DevSym &S, size_t elem, int threads) {
+  const int ncol = S.nu + (elem == sizeof(double) && zsolve64_folds_b(S) ? 1 : 0), w = zsolve_width(S, ncol);
+  const long long items = (long long)((ncol + w - 1) / w) * S.N;
+  return (size_t)zsolve_grid(items, zsolve_cta(items, w, threads)) * S.nx * w * elem;
+}
+// CTAs of a launch: what the GPU holds at once, no more than the work buffer
+// has panels for (at least one: a buffer of fewer than 32 columns belongs to a
+// problem of panels of 8)
+static int zsolve_ctas(long long items, int threads, size_t panel_bytes, size_t work_bytes) {
+  return (int)std::min((long long)zsolve_grid(items, threads), (long long)(work_bytes / panel_bytes));
 }
 
 template <int W, int C>
 static void zsolve64_launch(const DevSym &S, const double *LU, const double *rd, const double *J, const double *K,
-                            double *work, double *Z, double *Y, double *Yu, cudaStream_t st, int threads,
+                            ZsolveWork work, double *Z, double *Y, double *Yu, cudaStream_t st, int threads,
                             const double *g, double *b, int *ezy, int phase) {
   // dynamic plus static shared memory may pass the 48 KB default
   static const bool cap = raise_smem_cap(k_zsolve64<W, C>);
@@ -977,13 +978,13 @@ static void zsolve64_launch(const DevSym &S, const double *LU, const double *rd,
   const int npan = (S.nu + (b ? 1 : 0) + W * C - 1) / (W * C);
   const size_t bytes = phase == 0 ? (size_t)S.nd * W * C * sizeof(double) : 0;
   threads = zsolve_cta((long long)npan * S.N, W * C, threads);
-  k_zsolve64<W, C><<<zsolve_grid((long long)npan * S.N, threads), threads, bytes, st>>>(
-      S, npan, LU, rd, J, K, work, Z, Y, Yu, g, b, ezy, phase);
+  k_zsolve64<W, C><<<zsolve_ctas((long long)npan * S.N, threads, sizeof(double) * S.nx * W * C, work.bytes), threads,
+                     bytes, st>>>(S, npan, LU, rd, J, K, (double *)work.p, Z, Y, Yu, g, b, ezy, phase);
   ipm_count_launch();
 }
 
 void launch_zsolve64(const DevSym &S, const double *LU, const double *rd, const double *J,
-                     const double *K, double *work, double *Z, double *Y, double *Yu, cudaStream_t st, int threads,
+                     const double *K, ZsolveWork work, double *Z, double *Y, double *Yu, cudaStream_t st, int threads,
                      const double *g, double *b, int *ezy) {
   if (S.big) {
     // the block's right-hand sides, the block by the batched triangular
@@ -1001,20 +1002,20 @@ void launch_zsolve64(const DevSym &S, const double *LU, const double *rd, const 
 }
 
 template <int W, int C>
-static void zsolve32_launch(const DevSym &S, const RoundedFactors &f, const double *J, const double *K, float *work,
+static void zsolve32_launch(const DevSym &S, const RoundedFactors &f, const double *J, const double *K, ZsolveWork work,
                             float *Z, float *Y, double *Yu, cudaStream_t st, int threads, int phase) {
   static const bool cap = raise_smem_cap(k_zsolve32<W, C>);
   (void)cap;
   const int npan = (S.nu + W * C - 1) / (W * C);
   const size_t bytes = phase == 0 ? (size_t)S.nd * W * C * sizeof(float) : 0;
   threads = zsolve_cta((long long)npan * S.N, W * C, threads);
-  k_zsolve32<W, C><<<zsolve_grid((long long)npan * S.N, threads), threads, bytes, st>>>(
-      S, npan, f.LUf, f.rdf, f.Kf, J, K, work, Z, Y, Yu, phase);
+  k_zsolve32<W, C><<<zsolve_ctas((long long)npan * S.N, threads, sizeof(float) * S.nx * W * C, work.bytes), threads,
+                     bytes, st>>>(S, npan, f.LUf, f.rdf, f.Kf, J, K, (float *)work.p, Z, Y, Yu, phase);
   ipm_count_launch();
 }
 
 void launch_zsolve32(const DevSym &S, const double *LU, const double *rd, const double *J,
-                     const double *K, const RoundedFactors &f, float *work, float *Z, float *Y, double *Yu,
+                     const double *K, const RoundedFactors &f, ZsolveWork work, float *Z, float *Y, double *Yu,
                      cudaStream_t st, int threads, const TcsPlan *tcs, int *flags) {
   k_round_factors<<<dim3((round_lu_len(S) + S.nx + 255) / 256, S.N), 256, 0, st>>>(S, LU, rd, f.LUf, f.rdf);
   ipm_count_launch();
