@@ -320,14 +320,17 @@ ipm_status ipm_run_instances(const ipm_network *nets, int n, const int *n_scen, 
   if (!(bo.window_us >= 0)) return IPM_ERR_ARG;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return IPM_ERR_CUDA;
-  // footprint estimate: Z and Y (or the mixed operands, no larger), the
-  // per-scenario K_uu blocks, and a margin for vectors, LU values and tiles
+  // footprint estimate: Z and Y (or the mixed operands, no larger), the panels
+  // of their solve (as many as there are, at most those of 760 CTAs with 32
+  // columns each), the per-scenario K_uu blocks, and a margin for vectors, LU
+  // values and tiles
   std::vector<long long> est(n);
   for (int i = 0; i < n; ++i) {
     long long nx, nu;
     dims_of(nets[i], nx, nu);
     const long long N = n_scen[i];
-    est[i] = 16 * N * nx * nu + 8 * N * nu * nu + 8 * 96 * N * nx + (64LL << 20);
+    est[i] = 16 * N * nx * nu + 8 * nx * std::min(N * (nu + 32), 760LL * 32) + 8 * N * nu * nu + 8 * 96 * N * nx +
+             (64LL << 20);
   }
   Group G;
   if (!G.init(dev, bo.window_us)) {
