@@ -174,6 +174,7 @@ ipm_status upload_symbolic(ipm_ctx *c, const HostNet &net, const double *pd, con
 }
 
 void set_groups(ipm_ctx *c, long long G);
+long long default_groups(const ipm_ctx *c);
 
 ipm_status alloc_work(ipm_ctx *c) {
   const Sym &S = c->S;
@@ -315,11 +316,10 @@ ipm_status alloc_work(ipm_ctx *c) {
   // Where chunks of 64 rows would not fill one wave, one wave of chunks of at
   // least 16 rows (products and assembly, 30 buses x 1: 14 us, with one chunk
   // 39; 120 x 17: 22 + 31, with chunks of 64 rows 38 + 15).
-  {
-    const long long G0 = std::max(1, (3 * 152) / c->ntiles);
-    set_groups(c, (long long)S.N * S.nx <= 64 * G0 ? G0 : 4 * G0);
-    c->max_groups = c->ngroups;
-  }
+  // The buffer of partial tiles has room for the autotuner's candidates too.
+  set_groups(c, 4LL * std::max(1, (3 * 152) / c->ntiles));
+  c->max_groups = c->ngroups;
+  set_groups(c, default_groups(c));
   c->zs_threads = (c->opt.solve_threads == 128 || c->opt.solve_threads == 256) ? c->opt.solve_threads : 256;
   {
     // the multi-RHS solve's panels in flight (a tuned thread count uses what
@@ -578,6 +578,12 @@ void fp64_contraction(ipm_ctx *c, cudaStream_t st) {
                         c->partial, st);
 }
 
+// chunks of the contraction by default (reasons where the buffers are allocated)
+long long default_groups(const ipm_ctx *c) {
+  const long long krows = (long long)c->S.N * c->S.nx, G0 = std::max(1, (3 * 152) / c->ntiles);
+  return krows <= 64 * G0 ? G0 : std::min(4 * G0, (krows + 63) / 64);
+}
+
 // split the N*nx contraction rows into at most G chunks (a multiple of 16 rows each)
 void set_groups(ipm_ctx *c, long long G) {
   const long long krows = (long long)c->S.N * c->S.nx;
@@ -690,19 +696,24 @@ ipm_status autotune(ipm_ctx *c, cudaStream_t st) {
     emu_regroup(c->emuZZ, bestG);
     tc_groups = bestG;
   } else if (fp64) {
+    // products and assembly, the default among the candidates (left out of
+    // them, a tuned context was slower than an untuned one: condensation at
+    // 1,000 buses x 10 3.73 ms against 3.62)
     const long long G0 = std::max(1, (3 * 152) / c->ntiles);
-    long long bestG = G0;
+    long long bestG = default_groups(c);
     best = 1e300;
     int slot = 2;
-    for (long long G : {G0 / 2, G0, 2 * G0, 4 * G0}) {
-      if (G < 1 || G > c->max_groups) continue;
+    for (long long G : {bestG, G0 / 2, G0, 2 * G0, 4 * G0}) {
+      if (G < 1) continue;
       set_groups(c, G);
       if (c->ngroups > c->max_groups) continue;
       const double ms = time_ms([&] {
         launch_gemm_tn64((long long)S.N * S.nx, c->kchunk, S.nu, c->ngroups, c->Z, c->Y, c->tiles, c->ntiles,
                          c->partial, st);
+        launch_khat_assemble(S.nu, S.N, c->ngroups, c->ntiles, c->nt1, c->partial, c->tile_of, c->Yu, c->diag1,
+                             c->Khat, st);
       }, st);
-      if (slot < 8) c->tune_ms[slot++] = ms;
+      if (slot < 6) c->tune_ms[slot++] = ms;
       if (ms < best) best = ms, bestG = G;
     }
     set_groups(c, bestG);
