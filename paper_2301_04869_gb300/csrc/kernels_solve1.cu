@@ -339,9 +339,15 @@ void solve1_cluster_launch(const DevSym &S, const double *LU, const double *rd, 
 void solve1_cluster(const DevSym &S, const double *LU, const double *rd, double *v, int trans, int vps,
                     cudaStream_t st) {
   const int C = (long long)S.N * vps <= 38 || S.nd > 8192 ? 8 : 4;
-  // the accumulators take TH doubles per block and CTA
+  // the accumulators take TH doubles per block and CTA: fewer threads for the
+  // larger blocks, up to the largest that a scenario's factor can index
+  constexpr auto fits = [](size_t doubles) { return doubles * sizeof(double) <= 227 * 1024; };
+  static_assert(fits(trsv::smem_doubles<512, NB_BIG>(8192 / NB_BIG / 4)), "512 threads, clusters of 4");
+  static_assert(fits(trsv::smem_doubles<256, NB_BIG>(40448 / NB_BIG / 8)), "256 threads");
+  static_assert(fits(trsv::smem_doubles<128, NB_BIG>((46340 / NB_BIG + 8) / 8)), "nd^2 < 2^31");
   if (S.nd <= 8192) solve1_cluster_launch<512>(S, LU, rd, v, trans, vps, C, st);
-  else solve1_cluster_launch<256>(S, LU, rd, v, trans, vps, C, st);
+  else if (S.nd <= 40448) solve1_cluster_launch<256>(S, LU, rd, v, trans, vps, C, st);
+  else solve1_cluster_launch<128>(S, LU, rd, v, trans, vps, C, st);
 }
 
 template <int NB>
