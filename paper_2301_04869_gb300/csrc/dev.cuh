@@ -7,7 +7,7 @@
 constexpr int SWP = 4;  // products per lane of a single-vector sweep unit
 
 struct DevSym {
-  int n, L, ng, N, nx, nu, m, nnzA, nnzKB, nnzLU, nlev, nlev_b, nlev_f, t0, nd, nlev_fs, nlev_bs;
+  int n, L, ng, N, nx, nu, m, nnzKB, nnzLU, nlev_f, t0, nd, nlev_bs;
   int nflow;  // line-flow rows of h (2 L with ratings, else 0)
   // large trailing block (global-memory kernels): flag, offset of the block
   // in each scenario's LU values (column-major, leading dimension nd), and
@@ -19,7 +19,7 @@ struct DevSym {
   const double *lg, *lb, *lbh;
   const int *a_ptr, *a_col, *a_diag, *inc_ptr, *inc_line, *inc_other, *inc_aslot;
   const int *a_tslot;  // per A slot (i, k): the slot of (k, i)
-  const int *kb_ptr, *kb_col, *kb_row, *kb_aslot, *kbi_ptr, *kbi_r, *kbi_ja, *kbi_jb;
+  const int *kb_col, *kb_row, *kb_aslot, *kbi_ptr, *kbi_r, *kbi_ja, *kbi_jb;
   const int *hrow_bus, *hrow_comp, *ht_ptr, *ht_r, *ht_aslot;
   const int *perm, *iperm;
   const int *lu_diag, *lu_init, *tail_slot;
@@ -28,8 +28,6 @@ struct DevSym {
   int lu_lists;
   const int *lsc_slot, *lsc_k;
   const int *tw_len, *tw_l, *tw_u, *tw_e;  // trailing-block products per list
-  const int *fw_lev_ptr, *fw_rows, *fr_ptr, *fr_col, *fr_lslot, *fr_uslot;
-  const int *bw_lev_ptr, *bw_rows, *br_ptr, *br_col, *br_uslot, *br_lslot;
   const int *bs_lev_ptr;
   const int4 *bs4;  // backward sparse rows {row, first product, end, 0}
   // units of the single-vector sweeps (symbolic.cpp) and the inverses of the
@@ -42,7 +40,7 @@ struct DevSym {
   double *dinv;
   const int *gu_ptr, *gu_col, *gu_src, *gut_ptr, *gut_col, *gut_src;
   const int *kx_ptr, *kx_col, *kx_src, *ku_ptr, *ku_col, *ku_src;
-  // the same product lists as {column, slot} pairs (zp_col/zp_slot,
+  // product lists as {column, slot} pairs (Sym::zp_col/zp_slot,
   // zp_tcol/zp_tslot, br_col/br_uslot) and {column, K entry} (kx_col/kx_src)
   const int2 *zp2, *zpt2, *br2, *kx2;
   int zp_npan;  // forward schedules per 32-column panel of Z (symbolic.cpp)

@@ -98,8 +98,8 @@ ipm_status upload_symbolic(ipm_ctx *c, const HostNet &net, const double *pd, con
   Sym &S = c->S;
   DevSym &d = c->ds;
   d.n = S.n; d.L = S.L; d.ng = S.ng; d.N = S.N; d.nx = S.nx; d.nu = S.nu; d.m = S.m;
-  d.nnzA = S.nnzA; d.nnzKB = S.nnzKB; d.nnzLU = S.nnzLU; d.nlev = S.nlev; d.nlev_b = S.nlev_b;
-  d.nlev_f = S.nlev_f; d.t0 = S.t0; d.nd = S.nd; d.nlev_fs = S.nlev_fs; d.nlev_bs = S.nlev_bs;
+  d.nnzKB = S.nnzKB; d.nnzLU = S.nnzLU;
+  d.nlev_f = S.nlev_f; d.t0 = S.t0; d.nd = S.nd; d.nlev_bs = S.nlev_bs;
   d.nflow = S.nflow;
   d.big = S.big ? 1 : 0;
   d.dense_base = S.dense_base;
@@ -113,7 +113,7 @@ ipm_status upload_symbolic(ipm_ctx *c, const HostNet &net, const double *pd, con
   TRY(upload(c, &d.a_tslot, S.a_tslot));
   TRY(upload(c, &d.inc_ptr, S.inc_ptr)); TRY(upload(c, &d.inc_line, S.inc_line));
   TRY(upload(c, &d.inc_other, S.inc_other)); TRY(upload(c, &d.inc_aslot, S.inc_aslot));
-  TRY(upload(c, &d.kb_ptr, S.kb_ptr)); TRY(upload(c, &d.kb_col, S.kb_col)); TRY(upload(c, &d.kb_row, S.kb_row));
+  TRY(upload(c, &d.kb_col, S.kb_col)); TRY(upload(c, &d.kb_row, S.kb_row));
   TRY(upload(c, &d.kb_aslot, S.kb_aslot)); TRY(upload(c, &d.kbi_ptr, S.kbi_ptr)); TRY(upload(c, &d.kbi_r, S.kbi_r));
   TRY(upload(c, &d.kbi_ja, S.kbi_ja)); TRY(upload(c, &d.kbi_jb, S.kbi_jb));
   TRY(upload(c, &d.hrow_bus, S.hrow_bus)); TRY(upload(c, &d.hrow_comp, S.hrow_comp));
@@ -145,10 +145,6 @@ ipm_status upload_symbolic(ipm_ctx *c, const HostNet &net, const double *pd, con
   TRY(upload(c, &d.lsc_slot, S.lsc_slot)); TRY(upload(c, &d.lsc_k, S.lsc_k));
   TRY(upload(c, &d.tw_len, S.tw_len)); TRY(upload(c, &d.tw_l, S.tw_l)); TRY(upload(c, &d.tw_u, S.tw_u));
   TRY(upload(c, &d.tw_e, S.tw_e));
-  TRY(upload(c, &d.fw_lev_ptr, S.fw_lev_ptr)); TRY(upload(c, &d.fw_rows, S.fw_rows)); TRY(upload(c, &d.fr_ptr, S.fr_ptr));
-  TRY(upload(c, &d.fr_col, S.fr_col)); TRY(upload(c, &d.fr_lslot, S.fr_lslot)); TRY(upload(c, &d.fr_uslot, S.fr_uslot));
-  TRY(upload(c, &d.bw_lev_ptr, S.bw_lev_ptr)); TRY(upload(c, &d.bw_rows, S.bw_rows)); TRY(upload(c, &d.br_ptr, S.br_ptr));
-  TRY(upload(c, &d.br_col, S.br_col)); TRY(upload(c, &d.br_uslot, S.br_uslot)); TRY(upload(c, &d.br_lslot, S.br_lslot));
   TRY(upload(c, &d.gu_ptr, S.gu_ptr)); TRY(upload(c, &d.gu_col, S.gu_col)); TRY(upload(c, &d.gu_src, S.gu_src));
   TRY(upload(c, &d.gut_ptr, S.gut_ptr)); TRY(upload(c, &d.gut_col, S.gut_col)); TRY(upload(c, &d.gut_src, S.gut_src));
   d.zp_npan = S.zp_npan;

@@ -60,7 +60,7 @@ struct Sym {
   std::vector<int> perm, iperm;
   int nnzLU = 0;
   std::vector<int> lu_colptr, lu_row, lu_diag, lu_init;
-  int nlev = 0, nlev_b = 0;
+  int nlev = 0;
   int nlev_f = 0;          // levels of the sparse (non-tail) pivots
   int t0 = 0, nd = 0;      // dense trailing block: positions [t0, nx), nd = nx - t0
   std::vector<int> tail_slot;  // nd*nd LU slots of the trailing block, row-major
@@ -81,8 +81,8 @@ struct Sym {
   int lu_lists = LU_LISTS;
   std::vector<int> tw_len, tw_l, tw_u, tw_e;
   long long n_tail_ops = 0;
-  std::vector<int> fw_lev_ptr, fw_rows, fr_ptr, fr_col, fr_lslot, fr_uslot;
-  std::vector<int> bw_lev_ptr, bw_rows, br_ptr, br_col, br_uslot, br_lslot;
+  std::vector<int> fr_ptr, fr_col, fr_lslot, fr_uslot;
+  std::vector<int> br_ptr, br_col, br_uslot, br_lslot;
   // backward sparse rows by level, 4 ints each: {row, first product, end, 0}
   std::vector<int> bs4;
   // The single-vector sweeps in units of one warp and four products per lane:

@@ -407,14 +407,12 @@ bool build_symbolic(const HostNet &net, int N, Sym &S, std::string &err, int big
   // ---- levels: lev(p) = 1 + max over pivots k with p in pat(k) ----
   // (computed on the minimum-degree pattern; a widened trailing block below
   // only adds fill inside itself, which the dense kernels handle)
-  std::vector<int> lev(nx, 0), blev(nx, 0);
+  std::vector<int> lev(nx, 0);
   for (int k = 0; k < nx; ++k)
     for (int p : pat[k]) lev[p] = std::max(lev[p], lev[k] + 1);
-  for (int i = nx - 1; i >= 0; --i)
-    for (int k : pat[i]) blev[i] = std::max(blev[i], blev[k] + 1);
-  int nlev = 0, nlevb = 0;
-  for (int k = 0; k < nx; ++k) { nlev = std::max(nlev, lev[k] + 1); nlevb = std::max(nlevb, blev[k] + 1); }
-  S.nlev = nlev; S.nlev_b = nlevb;
+  int nlev = 0;
+  for (int k = 0; k < nx; ++k) nlev = std::max(nlev, lev[k] + 1);
+  S.nlev = nlev;
   // dense trailing block: the largest suffix [t0, nx) whose L columns are full
   int t0 = nx;
   while (t0 > 0 && (int)pat[t0 - 1].size() == nx - t0) --t0;
@@ -631,20 +629,10 @@ bool build_symbolic(const HostNet &net, int N, Sym &S, std::string &err, int big
       }
       S.br_ptr[i + 1] = (int)S.br_col.size();
     }
-    std::vector<std::vector<int>> fl(nlev), bl(nlevb);
-    for (int i = 0; i < nx; ++i) { fl[lev[i]].push_back(i); bl[blev[i]].push_back(i); }
-    S.fw_lev_ptr.assign(nlev + 1, 0);
-    for (int l = 0; l < nlev; ++l) {
-      for (int i : fl[l]) S.fw_rows.push_back(i);
-      S.fw_lev_ptr[l + 1] = (int)S.fw_rows.size();
-    }
-    S.bw_lev_ptr.assign(nlevb + 1, 0);
-    for (int l = 0; l < nlevb; ++l) {
-      for (int i : bl[l]) S.bw_rows.push_back(i);
-      S.bw_lev_ptr[l + 1] = (int)S.bw_rows.size();
-    }
-    // the same schedules over the sparse rows only (the dense trailing block
-    // [t0, nx) is solved separately); empty levels dropped
+    std::vector<std::vector<int>> fl(nlev);
+    for (int i = 0; i < nx; ++i) fl[lev[i]].push_back(i);
+    // schedules of the sparse rows (the dense trailing block [t0, nx) is
+    // solved separately); empty levels dropped
     S.fs_lev_ptr.assign(1, 0);
     for (int l = 0; l < nlev; ++l) {
       bool any = false;
