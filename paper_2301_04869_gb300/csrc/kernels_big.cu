@@ -9,7 +9,8 @@
 //  * LU (right-looking, panels of PB columns, static diagonal pivots as in
 //    the rest of the factorization): per panel, its diagonal block (one CTA
 //    per scenario, in shared memory), L21 = A21 U11^{-1} (a thread per row),
-//    U12 = L11^{-1} A12 (a warp per column), and the trailing update
+//    U12 = L11^{-1} A12 (a thread per column, or a warp where columns are
+//    few), and the trailing update
 //    A22 -= L21 U12 as 64 x 64 FP64 tiles over (tile, scenario) or on the
 //    tensor cores;
 //  * the multi-RHS solve of Z through the block: Z_d (the block's n_u

@@ -9,12 +9,13 @@
 //
 // Scheduling: the LU runs on a cluster of two CTAs per scenario (cluster
 // barriers between its steps; a one-CTA kernel when the trailing block does
-// not fit the pair's shared memory), the single-vector solves on one CTA per
-// scenario, the multi-RHS solves on one CTA per (scenario, RHS panel) pair
-// plus one per scenario for b; each walks a level schedule of the shared
-// pattern with __syncthreads() between levels.  No grid-wide
-// synchronisation and no waits between CTAs other than the cluster
-// barriers.
+// not fit the pair's shared memory; with a large trailing block up to eight
+// CTAs for the sparse part, the block by the kernels of kernels_big.cu), the
+// multi-RHS solves on CTAs that work through (scenario, RHS panel) items, b
+// in the last panel's free column; each walks a level schedule of the shared
+// pattern with a barrier between levels.  No grid-wide synchronisation and no
+// waits between CTAs other than the cluster barriers.  The single-vector
+// solves are in kernels_solve1.cu.
 #include <algorithm>
 #include <atomic>
 
@@ -392,10 +393,13 @@ __device__ __forceinline__ void sweep_rows(int nlev, Lev lev, Desc desc, Meta me
 // and by the latency of the operand loads on the mixed one.  Measured (the
 // whole solve, against a warp per row of 32 columns with one column and
 // every product's column, slot and value loaded by every lane): 1,000 buses
-// x 64 4.03 -> 3.63 ms FP64 and 3.08 -> 1.26 ms FP32, 433 buses x 19 685 ->
-// 413 us FP64, 10,000 buses x 32 67.3 -> 43.3 ms FP32 (17 ms of it the dense
-// block's own kernels).  CTAs of 512 or 1,024 threads for the large networks
-// were slower (50 and 60 ms), as were W x C = 16 x 2 (47 ms) and 32 x 1 (62).
+// x 64 4.03 -> 3.54 ms FP64 and 3.08 -> 1.13 ms FP32, 433 buses x 19 685 ->
+// 413 us FP64, 10,000 buses x 32 67.3 -> 39.1 ms FP32 (17 ms of it the dense
+// block's own kernels).  W x C = 8 x 4 on the mixed path: 22.1 ms at 10,000 x
+// 32 and 4.3 at 3,000 x 40, 16 x 2 24.4 and 4.6, 32 x 1 40.1 and 6.9.  CTAs of
+// 512 threads take 19.8 and 3.6 there, of 1,024 21.7 and 4.2, of 128 26.1
+// (10,000 x 32); 256 were taken when the backward sweep had many more levels
+// (817 instead of 25 at 10,000 buses), which the larger CTAs paid for.
 //
 // phase (large trailing block, S.big): 1 = the forward sparse rows and the
 // trailing rows' right-hand sides only (left in Z for the batched block
@@ -720,10 +724,10 @@ __global__ void __launch_bounds__(256) k_round_k(DevSym S, int nk, const double 
 // and copied by the other CTA from the owner's shared memory, each CTA solves
 // U12 = L11^{-1} A12 and updates A22 -= L21 U12 on its own columns (4 x 4
 // register tiles), the next panel first.  Bound by the FP64 units in the
-// updates and by latency elsewhere: 890 us at 1,000 buses (179 init and
-// sparse levels, 87 trailing-block products, 46 the block's load, ~50 per
-// panel) -> NEW with the panels' factorization under the other SM's updates
-// and four loads in flight in the copies.
+// updates and by latency elsewhere: 768 us at 1,000 buses x 64 (890 with the
+// panels' factorization in turn with the updates and one load in flight in
+// the copies: 179 init and sparse levels, 87 trailing-block products, 46 the
+// block's load, ~50 per panel).
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(512, 1)
     k_lu_factor_pair(DevSym S, int nL, const double *__restrict__ J, double *LU, double *rd, int *flags,
                      double piv_tol) {

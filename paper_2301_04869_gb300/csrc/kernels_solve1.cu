@@ -12,23 +12,26 @@
 //  * Sparse rows: the work of a level comes in units, one warp and four
 //    products per lane each, 1 to 32 lanes to a row by its length
 //    (symbolic.cpp; a warp-wide FP64 operation takes ~19 cycles of an SM
-//    whatever its lanes hold, so a row's products go to few lanes).  The schedule does not depend on the data, so a warp
-//    fetches its next unit's products two units ahead and their factor values
-//    one ahead, across the level barriers; a level then costs the operands'
-//    loads, a few FP64 operations and the barrier instead of four dependent
-//    loads.
-//  * Trailing block, by 64 x 64 blocks: the inverses of the diagonal blocks
-//    are formed once per factorization, so a block of the solution is two
-//    small products instead of 64 dependent steps, and the rest of the block
-//    column is applied behind the chain.
+//    whatever its lanes hold, so a row's products go to few lanes).  The
+//    schedule does not depend on the data, so a warp fetches its next unit's
+//    products two units ahead and their factor values one ahead, across the
+//    level barriers; a level then costs the operands' loads, a few FP64
+//    operations and the barrier instead of four dependent loads.
+//  * Trailing block, by 64 x 64 blocks (32 x 32 up to 400 states): the
+//    inverses of the diagonal blocks are formed once per factorization, so a
+//    block of the solution is two small products instead of as many dependent
+//    steps as it has rows, and the rest of the block column is applied behind
+//    the chain.
 //  * Large networks: a cluster of 4 or 8 CTAs per scenario shares both
 //    (hardware cluster barriers), the blocks dealt in turn to the CTAs; the
 //    CTA holding the next block updates and solves it first, and everybody
 //    updates the other blocks between arriving at the barrier and waiting.
+//  * Small problems (S.ordered): the same units with 4 or 8 lanes per row, the
+//    trailing block by substitution, so that their sums keep one order.
 //
 // Measured, one solve (before: one CTA per scenario, or 54 launches through
 // the large blocks, a row's loads issued in turn and 64 steps per diagonal
-// block): 1,000 buses x 64 scenarios 280-355 -> 91 us, 3,000 x 10 1,090 ->
+// block): 1,000 buses x 64 scenarios 280-355 -> 91-106 us, 3,000 x 10 1,090 ->
 // 235 us, 10,000 x 32 4,660 -> 700 us.
 #include "dev.cuh"
 #include "kernels.h"
